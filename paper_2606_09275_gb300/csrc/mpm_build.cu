@@ -1715,6 +1715,11 @@ void build_mesh(mpm_ctx* c, mpm_mesh* m, const mpm_domain& dom, const mpm_rigid&
     MPM_LAUNCH(k_slice_slots<<<grid_for(ns, 256), 256, 0, st>>>(ns, sw, slots));
     MPM_CUDA(cudaMemsetAsync(slots + ns, 0, sizeof(int), st));
     cub_exclusive_sum_int(c, slots, spos, ns + 1);
+    // the widths of a small mesh on the host, where the resident Krylov solves
+    // divide the rows among the SMs
+    m->slice_w_host.resize(ns <= RESIDENT_SLICES ? ns : 0);
+    if (!m->slice_w_host.empty())
+      MPM_CUDA(cudaMemcpyAsync(m->slice_w_host.data(), sw, sizeof(int) * ns, cudaMemcpyDeviceToHost, st));
     m->nslot = read_total(c, spos, slots, ns + 1);
     long long* sb = grow<long long>(c, m->slice_base, ns + 1);
     MPM_LAUNCH(k_slice_base64<<<grid_for(ns + 1, 256), 256, 0, st>>>(ns + 1, spos, sb));

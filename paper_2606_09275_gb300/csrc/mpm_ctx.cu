@@ -118,6 +118,9 @@ extern "C" int mpm_create(mpm_ctx** out, void* stream) {
   try {
     c->stream = (cudaStream_t)stream;
     MPM_CUDA(cudaGetDevice(&c->device));
+    int coop = 0;
+    MPM_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device));
+    if (coop) MPM_CUDA(cudaDeviceGetAttribute(&c->coop_sms, cudaDevAttrMultiProcessorCount, c->device));
     MPM_CUDA(cudaMallocAsync((void**)&c->d_err, sizeof(int), c->stream));
     MPM_CUDA(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
     MPM_CUDA(cudaMallocAsync((void**)&c->d_red, 64 * sizeof(double), c->stream));
@@ -177,6 +180,7 @@ extern "C" int mpm_destroy(mpm_ctx* c) {
   c->meshes.clear();
   free_buf(c, c->cub_tmp);
   free_buf(c, c->part);
+  free_buf(c, c->rk_slots);
   for (auto& b : c->tmp) free_buf(c, b);
   for (auto& b : c->v) free_buf(c, b);
   try {

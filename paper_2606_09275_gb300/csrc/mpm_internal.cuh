@@ -157,6 +157,7 @@ struct mpm_ctx {
   cudaStream_t stream = nullptr;
   cudaStream_t cap_stream = nullptr;  // private stream on which CUDA graphs are captured
   int device = 0;
+  int coop_sms = 0;            // SMs, where cooperative launches are supported (else 0)
   int* d_err = nullptr;        // device error word
   double* d_red = nullptr;     // device reduction slots (64 doubles)
   // fixed-order grid sums (mpm::GridRed): per-block partials and the ticket
@@ -167,6 +168,7 @@ struct mpm_ctx {
   int* h_int = nullptr;        // pinned host ints (counts)
   mpm::Buf cub_tmp;            // CUB temporary storage
   mpm::Buf tmp[8];             // general scratch
+  mpm::Buf rk_slots;           // sum slots of the resident Krylov solves
   std::string err;
   mpm_mesh* step_mesh = nullptr;
   std::vector<mpm_mesh*> meshes;  // meshes made by mpm_octree_build, freed with the context
@@ -213,6 +215,7 @@ struct mpm_mesh {
   long long nslot = 0;                  // padded block slots of the sliced storage
   mpm::Buf slice_w, slice_base, scol;   // width, first slot of each slice, slot columns
   mpm::Buf srow, spos;                  // storage row -> dof row, and back (npad each)
+  std::vector<int> slice_w_host;        // slice_w of a small mesh (resident solves; else empty)
   // sources of each row: (sorted point or ghost face) << 6 | local index
   long long nsrc = 0;
   long long npair = 0;  // sum of squared support sizes (host copy, read after the build)
@@ -266,6 +269,7 @@ struct Sliced {
   const int* row;        // dof row of each storage row
   const int* pos;        // storage row of each dof row
 };
+constexpr int RESIDENT_SLICES = 4096;  // most slices of a mesh whose solves may run resident (mpm_solve.cu)
 constexpr int SLICE_WINDOW = 256;  // storage rows over which the dof rows are sorted
 __host__ __device__ inline long long sliced_slot(long long base, int sr, int idx) {
   return base + ((long long)(idx >> 2) * 32 + (sr & 31)) * 4 + (idx & 3);

@@ -12,8 +12,10 @@
 #include <vector>
 #include <cmath>
 #include <string>
+#include <type_traits>
 
 #include "mpm_internal.cuh"
+#include "mpm_resident.cuh"
 #include "mpm_sliced.cuh"
 
 namespace mpm {
@@ -472,6 +474,75 @@ const float4* residual_split(mpm_ctx* c, const mpm_mesh* m, const T* K, const do
 
 Sliced sliced_of(const mpm_mesh* m) { return sliced_view(m); }
 
+// The plan of a resident solve (mpm_resident.cuh) of this mesh with nv vectors
+// per row, G = 0 for the launches per iteration.  Resident is the faster way
+// wherever the rows' state fits in shared memory, by 10x at 2 k rows down to
+// 1.08x at 131 k (FP32 PCG, the table there), where HBM bounds both: the limit
+// RESIDENT_SLICES.
+template <class T>
+RkPlan resident_plan(const mpm_ctx* c, const mpm_mesh* m, int nv) {
+  constexpr int SMEM = 200 * 1024;
+  RkPlan p{};
+  const std::vector<int>& w = m->slice_w_host;
+  int ns = m->nslice;
+  if (c->coop_sms < 2 || !ns || (int)w.size() != ns) return p;
+  int W = std::min(c->coop_sms - 1, 8 * ns);
+  // the workers' shares, as rk_range deals them out
+  long long total = 0, before = 0;
+  for (int s = 0; s < ns; ++s) total += 32LL * w[s] + 8 * RK_ROW;
+  int rows = 0, groups = 0, q = 0;
+  for (int b = 1, lo = 0; b <= W; ++b) {
+    long long want = total * b / W;
+    int g = 0, q1;
+    while (lo + 1 < ns && before + 32LL * w[lo] + 8 * RK_ROW <= want) before += 32LL * w[lo] + 8 * RK_ROW, ++lo;
+    q1 = b == W ? 8 * ns : rk_start(want, lo, before, w[lo]);
+    rows = std::max(rows, 4 * (q1 - q));
+    for (; q < q1; ++q) g += w[q >> 3] >> 2;
+    groups = std::max(groups, g);
+  }
+  p.rows = std::max(rows, 4);
+  long long state = (long long)p.rows * ((3 * nv + 9) * sizeof(T) + 2 * sizeof(int));
+  long long kept = (long long)groups * (rk_group<T>() * sizeof(T) + 16 * sizeof(int));
+  if (state > SMEM) return p;
+  if (state + kept <= SMEM) p.groups = groups;
+  p.smem = (int)(state + (p.groups ? kept : 0));
+  p.G = W + 1;
+  return p;
+}
+
+template <class A>
+struct Same {
+  typedef A T;
+};
+
+// a resident PCG or BiCGStab and its scalars on the host; *ran false: the
+// device cannot hold the grid at once, nothing was launched
+template <class... A>
+int run_resident(mpm_ctx* c, bool* ran, void (*kern)(A...), const RkPlan& pl, unsigned long long* slots, int maxit,
+                 Scal* sc_d, Scal* sc_h, double* relres, int* iters, bool pcg, typename Same<A>::T... a) {
+  cudaStream_t st = c->stream;
+  void* args[] = {(void*)&a...};
+  MPM_CUDA(cudaMemsetAsync(sc_d, 0, sizeof(Scal), st));
+  MPM_CUDA(cudaMemsetAsync(slots, 0xff, sizeof(*slots) * rk_slot_words(pl.G), st));
+  MPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.smem));
+  cudaError_t e = cudaLaunchCooperativeKernel((const void*)kern, dim3(pl.G), dim3(RK_T), args, pl.smem, st);
+  *ran = e != cudaErrorCooperativeLaunchTooLarge;
+  if (!*ran) {
+    cudaGetLastError();
+    return MPM_OK;
+  }
+  MPM_CUDA(e);
+  MPM_COUNT(c);
+  MPM_CUDA(cudaMemcpyAsync(sc_h, sc_d, sizeof(Scal), cudaMemcpyDeviceToHost, st));
+  MPM_CUDA(cudaStreamSynchronize(st));
+  *iters = 0;
+  *relres = 0.0;
+  if (sc_h->bb == 0.0 && !sc_h->breakdown) return MPM_OK;
+  *iters = sc_h->done ? sc_h->iters : maxit;
+  *relres = sqrt(sc_h->rr[pcg ? *iters % 3 : 0] / sc_h->bb);
+  return !sc_h->done || sc_h->breakdown ? MPM_ERR_KRYLOV : MPM_OK;
+}
+
 template <class T, class V>
 int run_pcg(mpm_ctx* c, const mpm_mesh* m, const T* K, const V* Dinv, const double* b, V* x,
             double tol, int maxit, Scal* sc_d, Scal* sc_h, double* relres, int* iters, V* r, V* z,
@@ -479,6 +550,16 @@ int run_pcg(mpm_ctx* c, const mpm_mesh* m, const T* K, const V* Dinv, const doub
   cudaStream_t st = c->stream;
   int nd = m->ndof, npad = 32 * m->nslice;
   Sliced S = sliced_of(m);
+  if constexpr (std::is_same<T, V>::value) {
+    RkPlan pl = resident_plan<T>(c, m, RK_PCG_VECS);
+    if (pl.G && maxit > 0) {
+      bool ran;
+      unsigned long long* slots = grow<unsigned long long>(c, c->rk_slots, rk_slot_words(pl.G));
+      int e = run_resident(c, &ran, k_pcg_resident<T>, pl, slots, maxit, sc_d, sc_h, relres, iters, true, nd,
+                           m->nslice, S, K, Dinv, ptr<int>(m->dof_mask), b, x, z, tol, maxit, sc_d, slots, pl);
+      if (ran) return e;
+    }
+  }
   MPM_CUDA(cudaMemsetAsync(sc_d, 0, sizeof(Scal), st));
   int vb = 4 * 152;
   GridRed gr = grid_red(c, 2, std::max(vb, grid_for(npad, 32 * SW)));
@@ -595,6 +676,16 @@ int run_bicgstab(mpm_ctx* c, const mpm_mesh* m, const T* K, const T* Dinv, const
   V* shv = grow<V>(c, c->v[11], n4);
   Sliced S = sliced_of(m);
   const int* mask = ptr<int>(m->dof_mask);
+  if constexpr (std::is_same<T, X>::value) {
+    RkPlan pl = Dinv ? resident_plan<T>(c, m, RK_BICG_VECS) : RkPlan{};
+    if (pl.G && maxit > 0) {
+      bool ran;
+      unsigned long long* slots = grow<unsigned long long>(c, c->rk_slots, rk_slot_words(pl.G));
+      int e = run_resident(c, &ran, k_bicg_resident<T>, pl, slots, maxit, sc_d, sc_h, relres, iters, false, nd,
+                           m->nslice, S, K, Dinv, mask, b, x, ph, shv, tol, maxit, sc_d, slots, pl);
+      if (ran) return e;
+    }
+  }
   MPM_CUDA(cudaMemsetAsync(sc_d, 0, sizeof(Scal), st));
   MPM_CUDA(cudaMemsetAsync(p, 0, sizeof(V) * n4, st));
   MPM_CUDA(cudaMemsetAsync(v, 0, sizeof(V) * n4, st));
@@ -1081,6 +1172,23 @@ extern "C" int mpm_solve_static(mpm_ctx* c, const mpm_mesh* m, const double* K, 
     Sliced S = sliced_of(m);
     // the array keeps the previous call's contents: every vector below is
     // written before it is read, and the scalars start from zero
+    RkPlan pl = resident_plan<double>(c, m, RK_PCG_VECS);
+    if (pl.G && need + sizeof(unsigned long long) * rk_slot_words(pl.G) <= kStaticBytes) {
+      MPM_LAUNCH(k_block_jacobi<double, double><<<grid_for(nd, 256), 256, 0, st>>>(nd, rp, col, S, K, Dinv, c->d_err));
+      unsigned long long* slots = (unsigned long long*)(base + need);  // behind the vectors
+      mpm_solve_stats s{};
+      bool ran;
+      s.status = run_resident(c, &ran, k_pcg_resident<double>, pl, slots, maxit, sc, (Scal*)(c->h_red + 32),
+                              &s.relres, &s.iterations, true, nd, m->nslice, S, K, Dinv, ptr<int>(m->dof_mask), rhs,
+                              x, z, tol, maxit, sc, slots, pl);
+      if (ran) {
+        int e = check_device_error(c, "mpm_solve_static");
+        if (stats) *stats = s;
+        if (e) return e;
+        if (s.status) set_error(c, "mpm_solve_static: PCG did not reach the tolerance");
+        return s.status;
+      }
+    }
     MPM_CUDA(cudaMemsetAsync(sc, 0, sizeof(Scal), st));
     MPM_CUDA(cudaMemsetAsync(ticket, 0, sizeof(unsigned), st));
     MPM_LAUNCH(k_block_jacobi<double, double><<<grid_for(nd, 256), 256, 0, st>>>(nd, rp, col, S, K, Dinv, c->d_err));
