@@ -7,6 +7,7 @@
 
 #include "mpm_internal.cuh"
 #include "mpm_law.cuh"
+#include "mpm_sliced.cuh"
 
 namespace mpm {
 namespace {
@@ -69,15 +70,17 @@ __global__ void k_kinematics(int P, const int* __restrict__ nsup, const int* __r
 // ------------------------------------------------------------------ constitutive
 
 // Full per-point update.  in: dF, b_e,n (6); out: tau (6: xx yy zz xy yz xz),
-// b_e (6), A' (81, layout [(i*9 + k*3 + m)*3 + j] = A_ijkm - tau_im delta_jk)
+// b_e (6), V0 A' (tangent_rotate)
 // The consistent spatial tangent from the spectral state: theta_ab =
 // (tau_a - tau_b)/(lam_a - lam_b) = g/2 * divided difference of ln (in FP64),
 // then the eigenbasis rotation of the 81 entries in the precision the tangent
 // is stored in (FP32 for the mixed path, where it runs on the FP32 pipe).
-// Layout [(i*9 + k*3 + m)*3 + j] = A_ijkm - tau_im delta_jk.
+// Layout [(i*9 + k*3 + m)*4 + j] = V0 (A_ijkm - tau_im delta_jk), the fourth
+// entry of each term unused: a lane of the row gather loads one term's three
+// factors in one 16-byte word (FP32).
 template <class TA>
 __device__ void tangent_rotate(const double* Q, const double* lam, const double* dd, double gr,
-                               const double* tau6, TA* Aout) {
+                               const double* tau6, double V0, TA* Aout) {
   // theta_ab = (tau_a - tau_b)/(lam_a - lam_b) = g/2 * divided difference of ln
   // (in FP64), then the eigenbasis rotation of the 81 entries in the
   // precision the tangent is stored in: FP32 for the mixed path, where it
@@ -95,6 +98,7 @@ __device__ void tangent_rotate(const double* Q, const double* lam, const double*
   }
 #pragma unroll
   for (int a = 0; a < 3; ++a) lr[a] = (R)lam[a];
+  const R v0 = (R)V0;
   R taum[9];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
@@ -104,9 +108,11 @@ __device__ void tangent_rotate(const double* Q, const double* lam, const double*
       taum[3 * i + j] = (R)tau6[s];
     }
   for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j)
-      for (int k = 0; k < 3; ++k)
-        for (int m = 0; m < 3; ++m) {
+    for (int k = 0; k < 3; ++k)
+      for (int m = 0; m < 3; ++m) {
+        R o[4];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
           R s = (R)0;
 #pragma unroll
           for (int a = 0; a < 3; ++a) {
@@ -120,13 +126,16 @@ __device__ void tangent_rotate(const double* Q, const double* lam, const double*
             }
           }
           if (j == k) s -= taum[3 * i + m];
-          Aout[(i * 9 + k * 3 + m) * 3 + j] = s;
+          o[j] = v0 * s;
         }
+        o[3] = (R)0;
+        st4(Aout + (i * 9 + k * 3 + m) * 4, o);
+      }
 }
 
 template <bool TANGENT, class TA>
 __device__ bool point_update_law(const Law& L, double E, double ys, const double* be, const double* dF,
-                                 double* tau6, double* be_new, TA* Aout, double* save = nullptr) {
+                                 double* tau6, double* be_new, double V0, TA* Aout, double* save = nullptr) {
   double b[9] = {be[0], be[3], be[5], be[3], be[1], be[4], be[5], be[4], be[2]};
   double t[9], bt[9];
 #pragma unroll
@@ -164,7 +173,7 @@ __device__ bool point_update_law(const Law& L, double E, double ys, const double
     tau6[s] = Q[3 * i] * ta[0] * Q[3 * j] + Q[3 * i + 1] * ta[1] * Q[3 * j + 1] + Q[3 * i + 2] * ta[2] * Q[3 * j + 2];
     be_new[s] = Q[3 * i] * bw[0] * Q[3 * j] + Q[3 * i + 1] * bw[1] * Q[3 * j + 1] + Q[3 * i + 2] * bw[2] * Q[3 * j + 2];
   }
-  if (TANGENT) tangent_rotate<TA>(Q, lam, dd, gr, tau6, Aout);
+  if (TANGENT) tangent_rotate<TA>(Q, lam, dd, gr, tau6, V0, Aout);
   if (save) {
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
@@ -198,8 +207,8 @@ __global__ void k_constitutive(int P, Law L, const double* __restrict__ E, const
   double det = det3(f);
   double t6[6], bn[6];
   bool ok = det > 0.0 && isfinite(det) &&
-            point_update_law<TANGENT, TA>(L, E[w], ys[w], be + 6 * (size_t)w, f, t6, bn,
-                                          Aalg + 81 * (size_t)w,
+            point_update_law<TANGENT, TA>(L, E[w], ys[w], be + 6 * (size_t)w, f, t6, bn, V0[w],
+                                          Aalg + 108 * (size_t)w,
                                           lawst ? lawst + 22 * (size_t)w : nullptr);
   if (!ok) {
     atomicOr(err, EB_NAN);
@@ -238,7 +247,7 @@ __global__ void k_constitutive(int P, Law L, const double* __restrict__ E, const
 // no second eigen-decomposition or return map
 template <class TA>
 __global__ void k_tangent_state(int P, const double* __restrict__ lawst, const double* __restrict__ tau,
-                                TA* Aalg) {
+                                const double* __restrict__ V0, TA* Aalg) {
   int w = blockIdx.x * blockDim.x + threadIdx.x;
   if (w >= P) return;
   const double* st = lawst + 22 * (size_t)w;
@@ -252,33 +261,33 @@ __global__ void k_tangent_state(int P, const double* __restrict__ lawst, const d
   for (int a = 0; a < 3; ++a) lam[a] = st[9 + a];
 #pragma unroll
   for (int i = 0; i < 6; ++i) t6[i] = tau[6 * (size_t)w + i];
-  tangent_rotate<TA>(Q, lam, dd, st[21], t6, Aalg + 81 * (size_t)w);
+  tangent_rotate<TA>(Q, lam, dd, st[21], t6, V0[w], Aalg + 108 * (size_t)w);
 }
 
-// grad_x S = grad S . dF^{-1} for the tangent gather (in its precision), without
-// the internal force; also V0 in that precision, so that the gather converts
-// nothing.  A conversion from FP64 occupies the FP64 pipe (2 lanes per clock
-// per SM on this part) as long as an FMA, for a whole warp instruction: dF^-1
-// is converted one entry per lane and shared by shuffles, and the FP32 path
-// reads grad S from its FP32 copy (TS = float), made once per mesh build.
+// grad_x S = grad S . dF^{-1} for the tangent gather (in its precision), one
+// 4-vector per support node at gx[4 (w pw + k)]: the gather loads a node's in
+// one 16-byte word (FP32).  Eight lanes per point.  A conversion from FP64
+// occupies the FP64 pipe as long as an FMA, for a whole warp instruction:
+// dF^-1 is converted one entry per lane and shared by shuffles, and the FP32
+// path reads grad S from its FP32 copy (TS = float), made once per mesh build.
 template <class TG, class TS>
-__global__ void k_gx(int P, const int* __restrict__ nsup, const TS* __restrict__ dS,
-                     const double* __restrict__ dFinv, const double* __restrict__ V0, TG* gx,
-                     TG* V0t) {
-  int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (w >= P) return;
-  TG mine = lane < 9 ? (TG)dFinv[9 * (size_t)w + lane] : lane == 9 ? (TG)V0[w] : (TG)0;
+__global__ void k_gx(int P, int pw, const int* __restrict__ nsup, const TS* __restrict__ dS,
+                     const double* __restrict__ dFinv, TG* gx) {
+  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  int w = (int)(t >> 3), sub = (int)(t & 7);
+  bool in = w < P;
+  TG mine = in ? (TG)dFinv[9 * (size_t)w + sub] : (TG)0, last = in ? (TG)dFinv[9 * (size_t)w + 8] : (TG)0;
   TG fi[9];
 #pragma unroll
-  for (int i = 0; i < 9; ++i) fi[i] = __shfl_sync(0xffffffffu, mine, i);
-  if (lane == 9) V0t[w] = mine;
-  int n = nsup[w];
-  for (int k = lane; k < n; k += 32) {
+  for (int i = 0; i < 8; ++i) fi[i] = __shfl_sync(0xffffffffu, mine, i, 8);
+  fi[8] = last;
+  int n = in ? nsup[w] : 0;
+  for (int k = sub; k < n; k += 8) {
     size_t o = (size_t)w * MAXS + k;
     TG a0 = (TG)dS[3 * o], a1 = (TG)dS[3 * o + 1], a2 = (TG)dS[3 * o + 2];
-    gx[3 * o] = a0 * fi[0] + a1 * fi[3] + a2 * fi[6];
-    gx[3 * o + 1] = a0 * fi[1] + a1 * fi[4] + a2 * fi[7];
-    gx[3 * o + 2] = a0 * fi[2] + a1 * fi[5] + a2 * fi[8];
+    TG g[4] = {a0 * fi[0] + a1 * fi[3] + a2 * fi[6], a0 * fi[1] + a1 * fi[4] + a2 * fi[7],
+               a0 * fi[2] + a1 * fi[5] + a2 * fi[8], (TG)0};
+    st4(gx + 4 * ((size_t)w * pw + k), g);
   }
 }
 
@@ -349,6 +358,7 @@ __global__ void k_residual_rows(int nd, int P, double load, const long long* __r
 // ------------------------------------------------------------------ tangent (row gather)
 
 constexpr int TW = 4;  // warps per block of the tangent gather (at most)
+constexpr int TANGENT_FEW_ROWS = 20000;  // below: a block per row (tangent_passes)
 
 // open-addressing table of a row's columns (dof -> position in the row), in
 // shared memory: a power of two at least twice the longest row
@@ -358,27 +368,76 @@ __host__ __device__ inline int tangent_hash_size(int mr) {
   return h;
 }
 
-// a block's 9 accumulators, padded to a 16-byte multiple so that one column
-// is read and written with vector accesses: 12 floats or 10 doubles
-template <class T>
-__host__ __device__ constexpr int tangent_acc_stride() {
-  return sizeof(T) == 4 ? 12 : 10;
-}
-
-// shared memory of one warp: the row's accumulators, the 32 terms of the
-// current source, then the row's column table
-template <class T>
-__host__ __device__ inline size_t tangent_warp_bytes(int mr) {
-  return (size_t)mr * tangent_acc_stride<T>() * sizeof(T) + 32 * sizeof(T) +
-         (size_t)tangent_hash_size(mr) * 2 * sizeof(int);
-}
-
 __device__ inline unsigned tangent_hash(int c, int hmask) {
   return ((unsigned)c * 2654435761u >> 7) & (unsigned)hmask;
 }
 
-// the 27 terms (grad_x S_k)^T A'_p of a source from shared memory (16-byte
-// aligned, 32 entries) in vector loads
+// row position of every (source, support node) pair, pw per source (0xffff
+// beyond the source's support, and for ghost faces): made once per mesh build,
+// so that the gather of every Newton iteration needs no lookup.  A hash table
+// of the row's columns in shared memory; a warp per row, or (SHARED, meshes of
+// few rows) a block per row, its warps taking the sources 32 at a time in turn.
+template <bool SHARED>
+__global__ void k_src_pos(int nd, int P, int pw, int hs, const int* __restrict__ rp, const int* __restrict__ col,
+                          const long long* __restrict__ sptr, const uint64_t* __restrict__ skeys,
+                          const int* __restrict__ nsup, const int* __restrict__ sidx, unsigned short* pos) {
+  extern __shared__ int smh[];
+  const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int t = SHARED ? threadIdx.x : lane, nt = SHARED ? blockDim.x : 32;
+  int *hkey = smh + (SHARED ? 0 : wi * 2 * hs), *hval = hkey + hs, hmask = hs - 1;
+  int r = SHARED ? blockIdx.x : blockIdx.x * nw + wi;
+  if (r >= nd) return;
+  auto sync = [] {
+    if (SHARED)
+      __syncthreads();
+    else
+      __syncwarp();
+  };
+  int s0 = rp[r], nb = rp[r + 1] - s0;
+  for (int i = t; i < hs; i += nt) hkey[i] = -1;
+  sync();
+  for (int i = t; i < nb; i += nt) {
+    int c = col[s0 + i];
+    unsigned h = tangent_hash(c, hmask);
+    while (atomicCAS(hkey + h, -1, c) != -1) h = (h + 1) & hmask;
+    hval[h] = i;
+  }
+  sync();
+  long long q1 = sptr[r + 1];
+  for (long long qb = sptr[r] + (SHARED ? 32 * wi : 0); qb < q1; qb += SHARED ? 32 * nw : 32) {
+    int cnt = (int)min(32LL, q1 - qb);
+    uint32_t kb = lane < cnt ? (uint32_t)skeys[qb + lane] : 0u;
+    for (int u = 0; u < cnt; ++u) {
+      int w = (int)(__shfl_sync(0xffffffffu, kb, u) >> 6);
+      int n = w < P ? nsup[w] : 0;
+      for (int l = lane; l < pw; l += 32) {
+        int v = 0xffff;
+        if (l < n) {
+          int c = sidx[(size_t)w * MAXS + l], key;
+          unsigned h = tangent_hash(c, hmask);
+          while ((key = hkey[h]) != c && key != -1) h = (h + 1) & hmask;
+          if (key == c) v = hval[h];
+        }
+        pos[(size_t)(qb + u) * pw + l] = (unsigned short)v;
+      }
+    }
+  }
+}
+
+template <class T>
+__device__ inline T dot3_add(const T* t, const T* g, T a) {
+  return fma(t[2], g[2], fma(t[1], g[1], fma(t[0], g[0], a)));
+}
+
+// ---- FP32: a column of the support per lane
+
+constexpr int TF_AS = 12;  // a block's 9 accumulators, padded for 16-byte accesses
+
+// shared memory of one row: the accumulators, then the 32 terms of two sources
+// (the rows of a warp 16 bytes apart in the banks)
+inline size_t tangent_row_bytes_f32(int mr) { return ((size_t)mr * TF_AS + 64) * sizeof(float) + 16; }
+
+// the 27 terms (grad_x S_k)^T A'_p of a source, 16-byte aligned, 32 entries
 __device__ inline void tangent_terms(const float* Tt, float* t) {
   const float4* v = reinterpret_cast<const float4*>(Tt);
 #pragma unroll
@@ -390,182 +449,368 @@ __device__ inline void tangent_terms(const float* Tt, float* t) {
     if (4 * i + 3 < 27) t[4 * i + 3] = a.w;
   }
 }
-__device__ inline void tangent_terms(const double* Tt, double* t) {
-  const double2* v = reinterpret_cast<const double2*>(Tt);
-#pragma unroll
-  for (int i = 0; i < 14; ++i) {
-    double2 a = v[i];
-    t[2 * i] = a.x;
-    if (2 * i + 1 < 27) t[2 * i + 1] = a.y;
-  }
-}
 
 // acc[0..8] += the block t (x) g of one (source, column) pair, with vector
 // shared-memory accesses
-__device__ inline void tangent_add(float* a, const float* t, float g0, float g1, float g2) {
+__device__ inline void tangent_add(float* a, const float* t, const float* g) {
   float4* v = reinterpret_cast<float4*>(a);
   float4 x = v[0], y = v[1];
   float z = a[8];
-  x.x += t[0] * g0 + t[1] * g1 + t[2] * g2;
-  x.y += t[3] * g0 + t[4] * g1 + t[5] * g2;
-  x.z += t[6] * g0 + t[7] * g1 + t[8] * g2;
-  x.w += t[9] * g0 + t[10] * g1 + t[11] * g2;
-  y.x += t[12] * g0 + t[13] * g1 + t[14] * g2;
-  y.y += t[15] * g0 + t[16] * g1 + t[17] * g2;
-  y.z += t[18] * g0 + t[19] * g1 + t[20] * g2;
-  y.w += t[21] * g0 + t[22] * g1 + t[23] * g2;
-  z += t[24] * g0 + t[25] * g1 + t[26] * g2;
+  x.x = dot3_add(t, g, x.x);
+  x.y = dot3_add(t + 3, g, x.y);
+  x.z = dot3_add(t + 6, g, x.z);
+  x.w = dot3_add(t + 9, g, x.w);
+  y.x = dot3_add(t + 12, g, y.x);
+  y.y = dot3_add(t + 15, g, y.y);
+  y.z = dot3_add(t + 18, g, y.z);
+  y.w = dot3_add(t + 21, g, y.w);
+  z = dot3_add(t + 24, g, z);
   v[0] = x;
   v[1] = y;
   a[8] = z;
 }
-__device__ inline void tangent_add(double* a, const double* t, double g0, double g1, double g2) {
-  double2* v = reinterpret_cast<double2*>(a);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    double2 x = v[i];
-    x.x += t[6 * i] * g0 + t[6 * i + 1] * g1 + t[6 * i + 2] * g2;
-    x.y += t[6 * i + 3] * g0 + t[6 * i + 4] * g1 + t[6 * i + 5] * g2;
-    v[i] = x;
-  }
-  a[8] += t[24] * g0 + t[25] * g1 + t[26] * g2;
-}
 
 // the loads of one source (point w, local index k) of a row, issued together:
-// lane l holds the l-th column of the point's support and its grad_x S, lanes
-// < 27 the three A'_p values of one of the 27 terms
-template <class T>
-struct TangentSrc {
-  int w, n, c;
-  T v0, gk0, gk1, gk2, a0, a1, a2, g0, g1, g2;
+// lane l of the row's HL lanes holds the grad_x S and row positions of support
+// nodes l, l + HL, ... < 32 and the three A'_p factors of terms l, l + HL, ...
+template <int HL>
+struct TangentSrcF {
+  static constexpr int NP = 32 / HL;
+  float gk[4], a[NP][4], g[NP][4];
+  unsigned pos[NP];
 };
 
-template <class T>
-__device__ inline void tangent_fetch(TangentSrc<T>& s, uint32_t sid, int P, int lane,
-                                     const int* __restrict__ nsup, const int* __restrict__ sidx,
-                                     const T* __restrict__ gx, const T* __restrict__ Aalg,
-                                     const T* __restrict__ V0) {
-  int w = (int)(sid >> 6), k = (int)(sid & 63);
-  s.w = w < P ? w : -1;  // w >= P: a ghost-face source, no point tangent
-  if (s.w < 0) return;
-  size_t ok = ((size_t)w * MAXS + k) * 3;
-  s.gk0 = gx[ok];
-  s.gk1 = gx[ok + 1];
-  s.gk2 = gx[ok + 2];
-  s.v0 = V0[w];
-  s.n = nsup[w];
-  if (lane < 27) {
-    const T* A = Aalg + 81 * (size_t)w + 3 * lane;
-    s.a0 = A[0];
-    s.a1 = A[1];
-    s.a2 = A[2];
-  }
-  // lane < 32 <= MAXS: inside the point's slot range whatever its support size
-  size_t o = (size_t)w * MAXS + lane;
-  s.c = sidx[o];
-  s.g0 = gx[3 * o];
-  s.g1 = gx[3 * o + 1];
-  s.g2 = gx[3 * o + 2];
-}
-
-// one (source, column) pair: its column's place in the row, then the block
-template <class T, bool UPPER>
-__device__ inline void tangent_pair(T* acc, const int* hkey, const int* hval, int hmask, int r, int c,
-                                    const T* t, T g0, T g1, T g2) {
-  constexpr int AS = tangent_acc_stride<T>();
-  if (UPPER && c < r) return;
-  unsigned h = tangent_hash(c, hmask);
-  int key;
-  while ((key = hkey[h]) != c && key != -1) h = (h + 1) & hmask;
-  if (key != c) return;
-  tangent_add(acc + AS * hval[h], t, g0, g1, g2);
-}
-
-// One warp owns block row r: for every point p with r in its support (local
-// index k), K_{r,w} += V0_p (grad_x S_k)^T A'_p (grad_x S_w) for all w in the
-// support of p.  The row accumulates in shared memory (mr = longest row, a
-// multiple of 4), in source order, free of atomics and deterministic; the
-// position of a column in the row comes from a per-row hash table.  Ghost coefficients and the
-// Dirichlet identity rows/columns are applied when the row is written out,
-// coalesced, in the sliced layout.
-// UPPER (a symmetric tangent: Hencky, von Mises, frictionless contact): only
-// the blocks of columns c >= r are formed and written, about half the work;
-// k_tangent_mirror then copies each into its transposed place.
-template <class T, bool UPPER>
-__global__ void __launch_bounds__(32 * TW)
-    k_tangent_rows(int nd, int P, int minlen, int mr, int last, const int* __restrict__ rp,
-                   const int* __restrict__ col,
-                   Sliced S, const long long* __restrict__ sptr, const uint64_t* __restrict__ skeys,
-                   const int* __restrict__ nsup, const int* __restrict__ sidx,
-                   const T* __restrict__ gx, const T* __restrict__ Aalg,
-                   const T* __restrict__ V0, const double* __restrict__ kg,
-                   const int* __restrict__ mask, T* K, int* err) {
-  constexpr int AS = tangent_acc_stride<T>();
-  extern __shared__ __align__(16) unsigned char smraw[];
-  int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  T* acc = (T*)(smraw + wi * tangent_warp_bytes<T>(mr));
-  T* Tt = acc + AS * (size_t)mr;
-  int* hkey = (int*)(Tt + 32);
-  int hs = tangent_hash_size(mr), hmask = hs - 1;
-  int* hval = hkey + hs;
-  int r = blockIdx.x * (blockDim.x >> 5) + wi;
-  if (r >= nd) return;
-  int s0 = rp[r], nb = rp[r + 1] - s0;
-  if (nb <= minlen) return;  // done by the pass for shorter rows
-  if (nb > mr) {
-    // left to the pass for longer rows; an error only in the last pass
-    if (lane == 0 && last) atomicOr(err, EB_ROW);
-    return;
-  }
-  for (int i = lane; i < hs; i += 32) hkey[i] = -1;
-  for (int i = lane; i < AS * nb; i += 32) acc[i] = (T)0;
-  __syncwarp();
-  for (int i = lane; i < nb; i += 32) {
-    int c = col[s0 + i];
-    unsigned h = tangent_hash(c, hmask);
-    while (atomicCAS(hkey + h, -1, c) != -1) h = (h + 1) & hmask;
-    hval[h] = i;
-  }
-  __syncwarp();
-  // the row's source keys 32 at a time (one coalesced load, then broadcast)
-  const unsigned FULL = 0xffffffffu;
-  long long q0 = sptr[r], q1 = sptr[r + 1];
-  for (long long qb = q0; qb < q1; qb += 32) {
-    int cnt = (int)min(32LL, q1 - qb);
-    uint32_t kb = lane < cnt ? (uint32_t)skeys[qb + lane] : 0u;
-    for (int u = 0; u < cnt; ++u) {
-      TangentSrc<T> s;
-      tangent_fetch(s, __shfl_sync(FULL, kb, u), P, lane, nsup, sidx, gx, Aalg, V0);
-      if (s.w < 0) continue;  // the same for every lane
-      if (lane < 27) Tt[lane] = s.v0 * (s.gk0 * s.a0 + s.gk1 * s.a1 + s.gk2 * s.a2);
-      __syncwarp();
-      T t[27];
-      tangent_terms(Tt, t);
-      if (lane < s.n) tangent_pair<T, UPPER>(acc, hkey, hval, hmask, r, s.c, t, s.g0, s.g1, s.g2);
-      // supports of more than 32 nodes (deep hanging chains)
-      for (int l = lane + 32; l < s.n; l += 32) {
-        size_t o = (size_t)s.w * MAXS + l;
-        tangent_pair<T, UPPER>(acc, hkey, hval, hmask, r, sidx[o], t, gx[3 * o], gx[3 * o + 1], gx[3 * o + 2]);
-      }
-      __syncwarp();
+template <int HL>
+__device__ inline void tangent_fetch_f(TangentSrcF<HL>& s, uint32_t sid, long long q, int pw, int l,
+                                       const float* gx, const float* Aalg, const unsigned short* pos) {
+  const float* gw = gx + 4 * (size_t)pw * (sid >> 6);
+  const float* aw = Aalg + 108 * (size_t)(sid >> 6);
+  const unsigned short* pq = pos + (size_t)q * pw;
+  ld4(gw + 4 * (sid & 63), s.gk);
+#pragma unroll
+  for (int j = 0; j < 32 / HL; ++j) {
+    int lj = l + HL * j;
+    if (lj < 27) ld4(aw + 4 * lj, s.a[j]);
+    s.pos[j] = 0xffffu;
+    if (lj < pw) {  // (beyond the support: a position of 0xffff, nothing is added)
+      ld4(gw + 4 * lj, s.g[j]);
+      s.pos[j] = pq[lj];
     }
+  }
+}
+
+// Block row r: for every point p with r in its support (local index k),
+// K_{r,w} += V0_p (grad_x S_k)^T A'_p (grad_x S_w) for all w in the support of
+// p, accumulated in shared memory in source order, free of atomics, and
+// written out, coalesced, in the sliced layout, with the ghost coefficients and
+// the Dirichlet identity (mr = longest row, a multiple of 4).
+// HL lanes work on a source.  HL = 16: a warp takes two rows (16 nodes is the
+// mean support), one per half, so that a warp instruction serves two sources.
+// Bound by shared-memory wavefronts: the accumulators' round trip at random
+// 48-byte slots, 37 of them per source, and 15 of the loads (ncu, LSU data
+// pipe 72 % busy).  Indentation, 1.9 M points, 29.7 M sources: 7.6 ms with a
+// hash lookup per pair and 13 loads per source, 6.4 with the precomputed
+// positions and 16-byte loads, 6.0 with two rows per warp (the long rows' pass
+// 1.2 -> 0.36 of it); an entry of the block per lane, as in FP64, 7.0.  HL = 32, WPR > 1: the warps of a block share a
+// row, each taking a contiguous part of its sources with a copy of the
+// accumulators, added up in warp order: for rows whose serial chain of sources
+// would be the time (few rows, and the long rows near hanging nodes).
+template <int HL, int WPR>
+__global__ void __launch_bounds__(32 * TW)
+    k_tangent_rows_f32(int nd, int P, int pw, int minlen, int mr, int last, const int* __restrict__ rp,
+                   const int* __restrict__ col, Sliced S, const long long* __restrict__ sptr,
+                   const uint64_t* __restrict__ skeys, const unsigned short* __restrict__ spos,
+                   const float* __restrict__ gx, const float* __restrict__ Aalg, const double* __restrict__ kg,
+                   const int* __restrict__ mask, float* K, int* err) {
+  static_assert(HL == 32 || WPR == 1, "shared rows take whole warps");
+  constexpr int AS = TF_AS, RPW = 32 / HL, NP = 32 / HL;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const unsigned FULL = 0xffffffffu;
+  int wi = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane % HL, part = wi % WPR;
+  const size_t rsz = (size_t)mr * AS + 68;
+  float* acc = (float*)smraw + (wi * RPW + lane / HL) * rsz;
+  float* Tt = acc + AS * (size_t)mr;
+  // rows in storage order: the two rows of a warp have about the same length
+  int sr = (blockIdx.x * ((blockDim.x >> 5) / WPR) + wi / WPR) * RPW + lane / HL;
+  int r = sr < nd ? S.row[sr] : nd, s0 = 0, nb = 0;
+  bool live = r < nd;
+  if (live) {
+    s0 = rp[r];
+    nb = rp[r + 1] - s0;
+    if (nb > mr && last && l == 0) atomicOr(err, EB_ROW);
+    live = nb > minlen && nb <= mr;  // else done by the other pass
+  }
+  if (WPR == 1 && !__any_sync(FULL, live)) return;
+  int n = 0;  // this row's (part's) sources
+  long long q0 = 0;
+  if (live) {
+    for (int i = l; i < AS * nb; i += HL) acc[i] = 0.f;
+    // the point sources come first in the row's key order, the ghost faces last
+    long long lo = sptr[r], hi = sptr[r + 1];
+    q0 = lo;
+    while (lo < hi) {
+      long long mid = (lo + hi) >> 1;
+      if ((int)((uint32_t)skeys[mid] >> 6) < P)
+        lo = mid + 1;
+      else
+        hi = mid;
+    }
+    n = (int)(lo - q0);
+    if (WPR > 1) {
+      int e = (int)((long long)n * (part + 1) / WPR);
+      n = (int)((long long)n * part / WPR);
+      q0 += n;
+      n = e - n;
+    }
+  }
+  int nmax = HL == 32 ? n : (int)__reduce_max_sync(FULL, n);
+  __syncwarp();
+  // the source keys HL at a time (one coalesced load, then broadcast); a row
+  // with no source left repeats a source of its own without adding it
+  if (nmax > 0) {
+    auto keys = [&](int u0) { return u0 + l < n ? (uint32_t)skeys[q0 + u0 + l] : 0u; };
+    uint32_t kb = keys(0), sid = __shfl_sync(FULL, kb, 0, HL);
+    TangentSrcF<HL> s;
+    tangent_fetch_f<HL>(s, sid, q0, pw, l, gx, Aalg, spos);
+    for (int u = 0; u < nmax; ++u) {
+      TangentSrcF<HL> nx;
+      uint32_t nsid = 0;
+      if (u + 1 < nmax) {
+        if ((u + 1) % HL == 0) kb = keys(u + 1);
+        nsid = __shfl_sync(FULL, kb, (u + 1) % HL, HL);
+        tangent_fetch_f<HL>(nx, nsid, u + 1 < n ? q0 + u + 1 : 0, pw, l, gx, Aalg, spos);
+      }
+      // two sets of terms in turn: one __syncwarp per source separates both
+      // the terms' writes from their reads and the row's updates
+      float* tt = Tt + 32 * (u & 1);
+#pragma unroll
+      for (int j = 0; j < NP; ++j)
+        if (l + HL * j < 27) tt[l + HL * j] = dot3_add(s.a[j], s.gk, 0.f);
+      __syncwarp();
+      float t[27];
+      tangent_terms(tt, t);
+      const bool on = u < n;
+#pragma unroll
+      for (int j = 0; j < NP; ++j)
+        if (on && s.pos[j] != 0xffffu) tangent_add(acc + AS * s.pos[j], t, s.g[j]);
+      // supports of more than 32 nodes (deep hanging chains)
+      if (pw > 32)
+        for (int i = l + 32; on && i < pw; i += HL) {
+          unsigned pl = spos[(size_t)(q0 + u) * pw + i];
+          if (pl == 0xffffu) continue;
+          float g[4];
+          ld4(gx + 4 * ((size_t)(sid >> 6) * pw + i), g);
+          tangent_add(acc + AS * pl, t, g);
+        }
+      s = nx;
+      sid = nsid;
+    }
+  }
+  if (WPR > 1) {
+    __syncthreads();
+    acc = (float*)smraw + (wi - part) * rsz;
+  } else {
+    __syncwarp();
+  }
+  if (!live) return;
+  // ghost, then the Dirichlet identity, then the row (and its padding slots,
+  // zero) into the sliced storage
+  int mr_ = mask[r];
+  int sl = sr >> 5, W = S.w[sl];
+  long long b0 = S.base[sl];
+  for (int i = l + HL * part; i < W; i += HL * WPR) {
+    long long slot = sliced_slot(b0, sr, i);
+    if (i >= nb) {
+#pragma unroll
+      for (int e = 0; e < 9; ++e) K[sliced_entry(b0, W, slot, e)] = 0.f;
+      continue;
+    }
+    // the ghost coefficient is zero away from the cut cells: convert only
+    // where some lane of the warp has one
+    double kd = kg[s0 + i];
+    float kv = __any_sync(__activemask(), kd != 0.0) ? (float)kd : 0.f;
+    int c = col[s0 + i];
+    int mc = mask[c];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        int e = 3 * a + b;
+        float v = acc[AS * i + e];
+#pragma unroll
+        for (int w = 1; w < WPR; ++w) v += acc[w * rsz + AS * i + e];
+        if (a == b) v += kv;
+        if (((mr_ >> a) & 1) || ((mc >> b) & 1)) v = (c == r && a == b) ? 1.f : 0.f;
+        K[sliced_entry(b0, W, slot, e)] = v;
+      }
+  }
+}
+
+// ---- FP64: an entry of the block per lane
+
+// shared memory of one warp: the gradients (and, in their fourth component,
+// row positions) of the support nodes of two sources, then the row's 9
+// accumulators per block
+inline size_t tangent_warp_bytes_f64(int mr) { return (9 * (size_t)mr + 256) * sizeof(double); }
+
+// the loads of one source (point w, local index k) of a row, issued together:
+// lane l holds the l-th support node's grad_x S and row position, lanes < 27
+// the three A'_p factors of one of the 27 terms
+struct TangentSrcD {
+  double gk[4], a[4], g[4];
+  unsigned pos;
+};
+
+__device__ inline void tangent_fetch_d(TangentSrcD& s, uint32_t sid, long long q, int pw, int lane, const double* gx,
+                                       const double* Aalg, const unsigned short* pos) {
+  const double* gw = gx + 4 * (size_t)pw * (sid >> 6);
+  ld4(gw + 4 * (sid & 63), s.gk);
+  if (lane < 27) ld4(Aalg + 108 * (size_t)(sid >> 6) + 4 * lane, s.a);
+  s.pos = 0xffffu;
+  if (lane < pw) {  // (beyond the support: a position of 0xffff)
+    ld4(gw + 4 * lane, s.g);
+    s.pos = pos[(size_t)q * pw + lane];
+  }
+}
+
+// Block row r: for every point p with r in its support (local index k),
+// K_{r,w} += V0_p (grad_x S_k)^T A'_p (grad_x S_w) for all w in the support of
+// p, accumulated in shared memory in source order, free of atomics, and
+// written out, coalesced, in the sliced layout, with the ghost coefficients and
+// the Dirichlet identity (mr = longest row, a multiple of 4).
+// The 27 working lanes of a warp are the 9 entries of a block times three
+// columns: a lane keeps the three terms (grad_x S_k)^T A'_p of its entry in
+// registers and walks the support three columns at a time.  Bound by the FP64
+// rate (an FP64 instruction takes 16 SM cycles however many lanes are active),
+// which this spends on ceil(n / 3) times 3 FMAs for n columns, or half of them
+// in the upper triangle; a column per lane takes 27 (36 before the sums were
+// nested FMAs) whatever n.  Punch, 17.8 k points: 2.47 ms with a column per
+// lane and a warp per row, 0.75 with four warps per row, 0.52 so.
+// WPR > 1: the warps of a block share a row, each taking a contiguous part of
+// its sources with a copy of the accumulators, added up in warp order.
+// UPPER (a symmetric tangent: Hencky, von Mises, frictionless contact): only
+// the blocks of columns c >= r are formed and written; k_tangent_mirror then
+// copies each into its transposed place.
+template <bool UPPER, int WPR>
+__global__ void __launch_bounds__(32 * TW)
+    k_tangent_rows_f64(int nd, int P, int pw, int minlen, int mr, int last, const int* __restrict__ rp,
+                   const int* __restrict__ col, Sliced S, const long long* __restrict__ sptr,
+                   const uint64_t* __restrict__ skeys, const unsigned short* __restrict__ spos,
+                   const double* __restrict__ gx, const double* __restrict__ Aalg, const double* __restrict__ kg,
+                   const int* __restrict__ mask, double* K, int* err) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const unsigned FULL = 0xffffffffu;
+  int wi = threadIdx.x >> 5, lane = threadIdx.x & 31, part = wi % WPR;
+  const int e = lane % 9, cg = lane < 27 ? lane / 9 : 1 << 20;  // (idle lanes: no column)
+  const size_t wsz = 9 * (size_t)mr + 256;
+  double* sg = (double*)smraw + wi * wsz;  // [2][32][4]
+  double* acc = sg + 256;
+  int r = blockIdx.x * ((blockDim.x >> 5) / WPR) + wi / WPR;
+  int s0 = 0, nb = 0;
+  bool live = r < nd;
+  if (live) {
+    s0 = rp[r];
+    nb = rp[r + 1] - s0;
+    if (nb > mr && last && lane == 0) atomicOr(err, EB_ROW);
+    live = nb > minlen && nb <= mr;  // else done by the other pass
+  }
+  if (WPR == 1 && !live) return;
+  if (live) {
+    for (int i = lane; i < 9 * nb; i += 32) acc[i] = 0.0;
+    // the point sources come first in the row's key order, the ghost faces last
+    long long q0 = sptr[r], q1 = sptr[r + 1];
+    {
+      long long lo = q0;
+      while (lo < q1) {
+        long long mid = (lo + q1) >> 1;
+        if ((int)((uint32_t)skeys[mid] >> 6) < P)
+          lo = mid + 1;
+        else
+          q1 = mid;
+      }
+    }
+    if (WPR > 1) {
+      long long n = q1 - q0;
+      q1 = q0 + n * (part + 1) / WPR;
+      q0 += n * part / WPR;
+    }
+    int n = (int)(q1 - q0);
+    if (n > 0) {
+      // the row's source keys 32 at a time (one coalesced load, then broadcast)
+      uint32_t kb = lane < n ? (uint32_t)skeys[q0 + lane] : 0u, sid = __shfl_sync(FULL, kb, 0);
+      TangentSrcD s;
+      tangent_fetch_d(s, sid, q0, pw, lane, gx, Aalg, spos);
+      for (int u = 0; u < n; ++u) {
+        double tv = dot3_add(s.a, s.gk, 0.0), t[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) t[j] = __shfl_sync(FULL, tv, 3 * e + j);
+        s.g[3] = __longlong_as_double((long long)s.pos);
+        double* sb = sg + 128 * (u & 1);  // two sets in turn: one __syncwarp per source
+        st4(sb + 4 * lane, s.g);
+        int ns = __popc(__ballot_sync(FULL, s.pos != 0xffffu));
+        // (UPPER: the supports are sorted, so the columns c >= r are the nodes
+        // from the source's own on)
+        const int k0 = UPPER ? (int)(sid & 63) : 0;
+        const uint32_t w = sid >> 6;
+        if (u + 1 < n) {
+          if (((u + 1) & 31) == 0) kb = u + 1 + lane < n ? (uint32_t)skeys[q0 + u + 1 + lane] : 0u;
+          sid = __shfl_sync(FULL, kb, (u + 1) & 31);
+          tangent_fetch_d(s, sid, q0 + u + 1, pw, lane, gx, Aalg, spos);
+        }
+        __syncwarp();
+        // three trips at a time: their columns are distinct
+        for (int c = k0 + cg; c < ns; c += 9) {
+          double v[3][4], x[3];
+          double* a[3];
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            int cj = min(c + 3 * j, 31);
+            ld4(sb + 4 * cj, v[j]);
+            a[j] = acc + 9 * (unsigned)__double_as_longlong(v[j][3]) + e;
+          }
+#pragma unroll
+          for (int j = 0; j < 3; ++j)
+            if (c + 3 * j < ns) x[j] = *a[j];
+#pragma unroll
+          for (int j = 0; j < 3; ++j)
+            if (c + 3 * j < ns) *a[j] = dot3_add(t, v[j], x[j]);
+        }
+        // supports of more than 32 nodes (deep hanging chains)
+        if (pw > 32) {
+          const unsigned short* pq = spos + (size_t)(q0 + u) * pw;
+          for (int i = max(32, k0) + cg; i < pw && pq[i] != 0xffffu; i += 3) {
+            double g[4];
+            ld4(gx + 4 * ((size_t)w * pw + i), g);
+            double* a = acc + 9 * (unsigned)pq[i] + e;
+            *a = dot3_add(t, g, *a);
+          }
+        }
+      }
+    }
+  }
+  if (WPR > 1) {
+    __syncthreads();
+    if (!live) return;
+    acc -= part * (ptrdiff_t)wsz;
+  } else {
+    __syncwarp();
   }
   // ghost, then the Dirichlet identity, then the row (and its padding slots,
   // zero) into the sliced storage
   int mr_ = mask[r];
   int sr = S.pos[r], sl = sr >> 5, W = S.w[sl];
   long long b0 = S.base[sl];
-  for (int i = lane; i < W; i += 32) {
+  for (int i = lane + 32 * part; i < W; i += 32 * WPR) {
     long long slot = sliced_slot(b0, sr, i);
     if (i >= nb) {
 #pragma unroll
-      for (int e = 0; e < 9; ++e) K[sliced_entry(b0, W, slot, e)] = (T)0;
+      for (int k = 0; k < 9; ++k) K[sliced_entry(b0, W, slot, k)] = 0.0;
       continue;
     }
     // the ghost coefficient is zero away from the cut cells: convert only
     // where some lane of the warp has one
     double kd = kg[s0 + i];
-    T kv = __any_sync(__activemask(), kd != 0.0) ? (T)kd : (T)0;
+    double kv = __any_sync(__activemask(), kd != 0.0) ? kd : 0.0;
     int c = col[s0 + i];
     if (UPPER && c < r) continue;  // written by k_tangent_mirror
     int mc = mask[c];
@@ -573,20 +818,21 @@ __global__ void __launch_bounds__(32 * TW)
     for (int a = 0; a < 3; ++a)
 #pragma unroll
       for (int b = 0; b < 3; ++b) {
-        int e = 3 * a + b;
-        T v = acc[AS * i + e];
+        int k = 3 * a + b;
+        double v = acc[9 * i + k];
+#pragma unroll
+        for (int u = 1; u < WPR; ++u) v += acc[u * wsz + 9 * i + k];
         if (a == b) v += kv;
-        if (((mr_ >> a) & 1) || ((mc >> b) & 1)) v = (c == r && a == b) ? (T)1 : (T)0;
-        K[sliced_entry(b0, W, slot, e)] = v;
+        if (((mr_ >> a) & 1) || ((mc >> b) & 1)) v = (c == r && a == b) ? 1.0 : 0.0;
+        K[sliced_entry(b0, W, slot, k)] = v;
       }
   }
 }
 
 // the lower blocks of a symmetric tangent: block (r, c), c < r, is the
 // transpose of block (c, r), found by binary search in row c (one warp per row)
-template <class T>
 __global__ void k_tangent_mirror(int nd, const int* __restrict__ rp, const int* __restrict__ col,
-                                 Sliced S, T* K) {
+                                 Sliced S, double* K) {
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   int r = (int)(t >> 5), lane = (int)(t & 31);
   if (r >= nd) return;
@@ -611,7 +857,7 @@ __global__ void k_tangent_mirror(int nd, const int* __restrict__ rp, const int* 
     if (j < 0) continue;  // (the pattern is symmetric: never)
     int src = S.pos[c], slc = src >> 5, Wc = S.w[slc];
     long long bc = S.base[slc], sc = sliced_slot(bc, src, j - rp[c]);
-    T v[9];
+    double v[9];
 #pragma unroll
     for (int e = 0; e < 9; ++e) v[e] = K[sliced_entry(bc, Wc, sc, e)];
     long long slot = sliced_slot(b0, sr, i);
@@ -1112,23 +1358,53 @@ void contact_terms(mpm_ctx* c, mpm_mesh* m, const mpm_material& mat, const mpm_r
 
 namespace {
 
-// one pass of the tangent gather (rows of lo < length <= hi blocks)
-template <class T>
-void tangent_launch(mpm_ctx* c, mpm_mesh* m, bool upper, int lo, int hi, int last, const void* gx,
-                    const void* Aalg, const void* V0t, void* K) {
-  cudaStream_t st = c->stream;
-  int nd = m->ndof, P = m->np;
-  size_t wb = tangent_warp_bytes<T>(hi);
-  int tw = (int)std::min<size_t>(TW, (size_t)(220 * 1024) / wb);
+// one pass of the tangent gather (rows of lo < length <= hi blocks): rpw rows
+// per warp, or wpr warps per row
+template <class T, class F>
+void tangent_launch(mpm_ctx* c, mpm_mesh* m, F kern, size_t row_bytes, int rpw, int wpr, int pw, int lo, int hi,
+                    int last, const void* gx, const void* Aalg, void* K) {
+  size_t wb = rpw * row_bytes;
+  int tw = (int)std::min<size_t>(TW, (size_t)(220 * 1024) / wb) / wpr * wpr;
   if (tw < 1) throw CudaError(MPM_ERR_SUPPORT, "stiffness row too long for the tangent gather");
   size_t smem = wb * tw;
   Sliced S = sliced_view(m);
-  auto kern = upper ? k_tangent_rows<T, true> : k_tangent_rows<T, false>;
   MPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  MPM_LAUNCH_P(MPM_PROF_TANGENT, kern<<<grid_for(nd, tw), 32 * tw, smem, st>>>(
-      nd, P, lo, hi, last, ptr<int>(m->row_ptr), ptr<int>(m->col), S, ptr<long long>(m->src_ptr),
-      ptr<uint64_t>(m->src_key), ptr<int>(m->nsup), ptr<int>(m->sidx), (const T*)gx, (const T*)Aalg,
-      (const T*)V0t, ptr<double>(m->kg), ptr<int>(m->dof_mask), (T*)K, c->d_err));
+  MPM_LAUNCH_P(MPM_PROF_TANGENT, kern<<<grid_for(m->ndof, tw / wpr * rpw), 32 * tw, smem, c->stream>>>(
+      m->ndof, m->np, pw, lo, hi, last, ptr<int>(m->row_ptr), ptr<int>(m->col), S, ptr<long long>(m->src_ptr),
+      ptr<uint64_t>(m->src_key), ptr<unsigned short>(m->src_pos), (const T*)gx, (const T*)Aalg, ptr<double>(m->kg),
+      ptr<int>(m->dof_mask), (T*)K, c->d_err));
+}
+
+// two passes: rows up to 128 blocks (the 5^3 interior stencil and below) with
+// a small shared-memory footprint per row, for occupancy, then the longer rows
+// near hanging nodes, which are few and have many sources.  The block's four
+// warps share a row there, and everywhere on meshes of few rows, where a
+// row's serial chain of sources is the time: below 20,000 rows a warp per row
+// leaves most of the 152 x 24 resident warps idle (the cone at 2.4 k rows:
+// 0.68 -> 0.16 ms).
+void tangent_passes(mpm_ctx* c, mpm_mesh* m, bool mixed, bool upper, int pw, const void* gx, const void* Aalg,
+                    void* K) {
+  const int SHORT = 128;
+  int mr = (m->maxrow + 3) & ~3;
+  int passes[2][2] = {{-1, std::min(mr, SHORT)}, {SHORT, mr}};
+  int np_ = mr > SHORT ? 2 : 1;
+  for (int ps = 0; ps < np_; ++ps) {
+    int lo = passes[ps][0], hi = passes[ps][1], last = ps == np_ - 1;
+    size_t rb = mixed ? tangent_row_bytes_f32(hi) : tangent_warp_bytes_f64(hi);
+    bool share = (ps > 0 || m->ndof < TANGENT_FEW_ROWS) && 4 * rb <= 220 * 1024;
+    if (mixed) {
+      if (share)
+        tangent_launch<float>(c, m, k_tangent_rows_f32<32, 4>, rb, 1, 4, pw, lo, hi, last, gx, Aalg, K);
+      else if (ps == 0)
+        tangent_launch<float>(c, m, k_tangent_rows_f32<16, 1>, rb, 2, 1, pw, lo, hi, last, gx, Aalg, K);
+      else
+        tangent_launch<float>(c, m, k_tangent_rows_f32<32, 1>, rb, 1, 1, pw, lo, hi, last, gx, Aalg, K);
+    } else {
+      auto kern = upper ? (share ? k_tangent_rows_f64<true, 4> : k_tangent_rows_f64<true, 1>)
+                        : (share ? k_tangent_rows_f64<false, 4> : k_tangent_rows_f64<false, 1>);
+      tangent_launch<double>(c, m, kern, rb, 1, share ? 4 : 1, pw, lo, hi, last, gx, Aalg, K);
+    }
+  }
 }
 
 }  // namespace
@@ -1185,9 +1461,20 @@ void assemble(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const mpm
   Sliced S = sliced_view(m);
   bool mixed = precision == MPM_MIXED;
   size_t asz = mixed ? sizeof(float) : sizeof(double);
-  void* Aalg = K ? grow_bytes(c, m->Aalg, 81 * (size_t)P * asz) : nullptr;
-  void* gx = K ? grow_bytes(c, m->gx, 3 * (size_t)P * MAXS * asz) : nullptr;
-  void* V0t = K ? grow_bytes(c, m->V0t, (size_t)P * asz) : nullptr;
+  int pw = (std::max(m->maxs, 1) + 3) & ~3;  // support nodes stored per point by the gather's arrays
+  void* Aalg = K ? grow_bytes(c, m->Aalg, 108 * (size_t)P * asz) : nullptr;
+  void* gx = K ? grow_bytes(c, m->gx, 4 * (size_t)P * pw * asz) : nullptr;
+  if (K && m->src_pos_gen != m->gen) {
+    int hs = tangent_hash_size(m->maxrow);
+    unsigned short* sp = grow<unsigned short>(c, m->src_pos, (size_t)m->nsrc * pw);
+    bool few = nd < TANGENT_FEW_ROWS;
+    size_t smem = (few ? 1 : 4) * 2 * sizeof(int) * (size_t)hs;
+    auto kern = few ? k_src_pos<true> : k_src_pos<false>;
+    MPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MPM_LAUNCH_P(MPM_PROF_PATTERN, kern<<<grid_for(nd, few ? 1 : 4), 128, smem, st>>>(
+        nd, P, pw, hs, rp, col, ptr<long long>(m->src_ptr), ptr<uint64_t>(m->src_key), nsup, sidx, sp));
+    m->src_pos_gen = m->gen;
+  }
   const float* dS32 = nullptr;
   if (K && mixed) {
     float* d32 = grow<float>(c, m->dS32, 3 * (size_t)P * MAXS);
@@ -1217,11 +1504,11 @@ void assemble(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const mpm
     // Newton's tangent at the increment of the last residual evaluation: its
     // dF, dF^-1, tau and spectral state are still in place, R is complete
     if (mixed) {
-      MPM_LAUNCH_P(MPM_PROF_CONSTITUTIVE, k_tangent_state<float><<<grid_for(P, 128), 128, 0, st>>>(P, lawst, tau, (float*)Aalg));
-      MPM_LAUNCH_P(MPM_PROF_FORCE, k_gx<float, float><<<grid_for(P, 8), 256, 0, st>>>(P, nsup, dS32, dFinv, V0, (float*)gx, (float*)V0t));
+      MPM_LAUNCH_P(MPM_PROF_CONSTITUTIVE, k_tangent_state<float><<<grid_for(P, 128), 128, 0, st>>>(P, lawst, tau, V0, (float*)Aalg));
+      MPM_LAUNCH_P(MPM_PROF_FORCE, k_gx<float, float><<<grid_for(8LL * P, 256), 256, 0, st>>>(P, pw, nsup, dS32, dFinv, (float*)gx));
     } else {
-      MPM_LAUNCH_P(MPM_PROF_CONSTITUTIVE, k_tangent_state<double><<<grid_for(P, 128), 128, 0, st>>>(P, lawst, tau, (double*)Aalg));
-      MPM_LAUNCH_P(MPM_PROF_FORCE, k_gx<double, double><<<grid_for(P, 8), 256, 0, st>>>(P, nsup, dS, dFinv, V0, (double*)gx, (double*)V0t));
+      MPM_LAUNCH_P(MPM_PROF_CONSTITUTIVE, k_tangent_state<double><<<grid_for(P, 128), 128, 0, st>>>(P, lawst, tau, V0, (double*)Aalg));
+      MPM_LAUNCH_P(MPM_PROF_FORCE, k_gx<double, double><<<grid_for(8LL * P, 256), 256, 0, st>>>(P, pw, nsup, dS, dFinv, (double*)gx));
     }
   } else {
     MPM_LAUNCH_P(MPM_PROF_KINEMATICS, k_kinematics<<<grid_for(8LL * P, 256), 256, 0, st>>>(P, nsup, sidx, dS, du, dF));
@@ -1250,39 +1537,20 @@ void assemble(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const mpm
     }
     if (K) {
       if (mixed)
-        MPM_LAUNCH_P(MPM_PROF_FORCE, k_gx<float, float><<<grid_for(P, 8), 256, 0, st>>>(P, nsup, dS32, dFinv, V0, (float*)gx, (float*)V0t));
+        MPM_LAUNCH_P(MPM_PROF_FORCE, k_gx<float, float><<<grid_for(8LL * P, 256), 256, 0, st>>>(P, pw, nsup, dS32, dFinv, (float*)gx));
       else
-        MPM_LAUNCH_P(MPM_PROF_FORCE, k_gx<double, double><<<grid_for(P, 8), 256, 0, st>>>(P, nsup, dS, dFinv, V0, (double*)gx, (double*)V0t));
+        MPM_LAUNCH_P(MPM_PROF_FORCE, k_gx<double, double><<<grid_for(8LL * P, 256), 256, 0, st>>>(P, pw, nsup, dS, dFinv, (double*)gx));
     }
   }
   if (K) {
-    // two passes: rows up to 128 blocks (the 5^3 interior stencil and below)
-    // with a small shared-memory footprint per warp, for occupancy, then the
-    // longer rows near hanging nodes; a symmetric tangent forms only its upper
-    // blocks and mirrors them
     // a symmetric FP64 tangent forms only its upper blocks and mirrors them:
-    // its pairs are bound by the FP64 FMA rate, which the halving pays for
-    // (about 5 ms of 108 per load step at the indentation workload); the FP32
-    // gather is bound by its per-source loads and table lookups instead, and
-    // the mirror pass would cost more than the halved pairs save
+    // its pairs are bound by the FP64 FMA rate, which the halving pays for; the
+    // FP32 gather is bound by its shared-memory traffic, and the mirror pass
+    // would cost more than the halved pairs save
     bool upper = !mixed && (mat.model == 0 || mat.model == 1) && !(mat.mu > 0.0 && contact);
-    int mr = (m->maxrow + 3) & ~3;
-    const int SHORT = 128;
-    int passes[2][2] = {{-1, std::min(mr, SHORT)}, {SHORT, mr}};
-    int np_ = mr > SHORT ? 2 : 1;
-    for (int ps = 0; ps < np_; ++ps) {
-      int lo = passes[ps][0], hi = passes[ps][1], last = ps == np_ - 1;
-      if (mixed)
-        tangent_launch<float>(c, m, upper, lo, hi, last, gx, Aalg, V0t, K);
-      else
-        tangent_launch<double>(c, m, upper, lo, hi, last, gx, Aalg, V0t, K);
-    }
-    if (upper) {
-      if (mixed)
-        MPM_LAUNCH_P(MPM_PROF_TANGENT, k_tangent_mirror<float><<<grid_for(32LL * nd, 256), 256, 0, st>>>(nd, rp, col, S, (float*)K));
-      else
-        MPM_LAUNCH_P(MPM_PROF_TANGENT, k_tangent_mirror<double><<<grid_for(32LL * nd, 256), 256, 0, st>>>(nd, rp, col, S, (double*)K));
-    }
+    tangent_passes(c, m, mixed, upper, pw, gx, Aalg, K);
+    if (upper)
+      MPM_LAUNCH_P(MPM_PROF_TANGENT, k_tangent_mirror<<<grid_for(32LL * nd, 256), 256, 0, st>>>(nd, rp, col, S, (double*)K));
     if (inertia) {
       double c2 = 2.0 / (dyn->dt * dyn->dt);
       if (mixed)
@@ -1375,7 +1643,7 @@ __global__ void k_point_update(int P, Law L, const int* __restrict__ perm,
     }
   }
   double t6[6], bn[6];
-  if (!point_update_law<false, double>(L, pE[w], pys[w], pbe + 6 * (size_t)w, dF, t6, bn, nullptr)) {
+  if (!point_update_law<false, double>(L, pE[w], pys[w], pbe + 6 * (size_t)w, dF, t6, bn, 0.0, nullptr)) {
     atomicOr(err, EB_NAN);
     return;
   }

@@ -235,7 +235,9 @@ struct mpm_mesh {
   mpm::Buf tri_fn, tri_en, tri_vn;
   double tri_lo[3] = {0, 0, 0}, tri_hi[3] = {0, 0, 0};
   // per-iteration point data (Mf: V0 tau dF^-T, 12 per point)
-  mpm::Buf dF, dFinv, tau, Aalg, gx, Mf, V0t;
+  mpm::Buf dF, dFinv, tau, Aalg, gx, Mf;
+  mpm::Buf src_pos;                     // row position of each (source, support node) pair (k_src_pos)
+  long long src_pos_gen = -1;           // build it belongs to
   mpm::Buf dS32;                        // FP32 copy of dS for the mixed tangent's grad_x S
   mpm::Buf pv;                          // sorted point velocities (time steps)
   bool has_v = false;                   // the points of this mesh build carried velocities
