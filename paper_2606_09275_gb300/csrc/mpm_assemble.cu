@@ -1037,92 +1037,150 @@ __global__ void k_contact_corner(int nc8, const int* __restrict__ cand, const in
   }
 }
 
+// the set entries of a chunk of NPER blockDim.x, in order, in list (shared
+// memory): on(i) tells whether entry i of the chunk is set, its value goes in;
+// returns their number.  Every thread of the block calls; ends with a
+// __syncthreads.
+template <int NPER, class F, class G>
+__device__ inline int block_compact(F on, G value, int* list, int* wsum) {
+  int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned m[NPER];
+  int mine = 0;
+#pragma unroll
+  for (int u = 0; u < NPER; ++u) {
+    m[u] = __ballot_sync(0xffffffffu, on((w * NPER + u) * 32 + lane));
+    mine += __popc(m[u]);
+  }
+  if (lane == 0) wsum[w] = mine;
+  __syncthreads();
+  int base = 0, n = 0;
+  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) {
+    if (i < w) base += wsum[i];
+    n += wsum[i];
+  }
+#pragma unroll
+  for (int u = 0; u < NPER; ++u) {
+    if ((m[u] >> lane) & 1) list[base + __popc(m[u] & ((1u << lane) - 1u))] = value((w * NPER + u) * 32 + lane);
+    base += __popc(m[u]);
+  }
+  __syncthreads();
+  return n;
+}
+
 // The rigid body's sums over the contact corners, in a fixed order (one
-// block; each thread takes the corners i = t, t + blockDim, ..., then the
-// block's fixed tree): out[0..5] the residual terms f and d x f, out[6..41]
-// their derivative in the body's increment q (row-major 6 x 6):
+// block): the corners in contact, a few of the candidates, are listed in order
+// and dealt to the threads in turn; the threads' 42 sums are added up through
+// shared memory, a warp per value.  out[0..5] the residual terms f and d x f,
+// out[6..41] their derivative in the body's increment q (row-major 6 x 6):
 // [d f / d qt, d f / d qr; [f]x + [d]x d f / d qt, [d]x d f / d qr] with
-// d f / d qt = -d f / d y
-__global__ void k_body_sums(int nc8, const double* __restrict__ cf, const double* __restrict__ ck,
-                            const double* __restrict__ ct, const double* __restrict__ cdv,
-                            const int* __restrict__ con, double* out) {
-  __shared__ double sh[32];
+// d f / d qt = -d f / d y.  (A tree of shuffles per value and warp, 5 FP64
+// additions at 16 SM cycles each, made this 51 us on the rolling sphere's 2.4 k candidates; 47 so, most of it the scan.)
+constexpr int BSUM_T = 256, BSUM_N = 8;
+__global__ void __launch_bounds__(BSUM_T)
+    k_body_sums(int nc8, const double* __restrict__ cf, const double* __restrict__ ck, const double* __restrict__ ct,
+                const double* __restrict__ cdv, const int* __restrict__ con, double* out) {
+  __shared__ int list[BSUM_N * BSUM_T], wsum[BSUM_T / 32];
+  __shared__ double sh[14][BSUM_T];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   double acc[42];
   for (int e = 0; e < 42; ++e) acc[e] = 0.0;
-  for (int i = threadIdx.x; i < nc8; i += blockDim.x) {
-    if (!con[i]) continue;
-    const double* f = cf + 3 * (size_t)i;
-    const double* d = cdv + 3 * (size_t)i;
-    const double* Ft = ct + 9 * (size_t)i;
-    double FX[9], Dx[9], Fx[9], DF[9], DT[9];
-    for (int e = 0; e < 9; ++e) FX[e] = ck[9 * (size_t)i + e];  // -d f / d y
-    cross_mat(d, Dx);
-    cross_mat(f, Fx);
-    mul33(Dx, FX, DF);
-    mul33(Dx, Ft, DT);
-    for (int a = 0; a < 3; ++a) {
-      acc[a] += f[a];
-      acc[3 + a] += d[(a + 1) % 3] * f[(a + 2) % 3] - d[(a + 2) % 3] * f[(a + 1) % 3];
-      for (int b = 0; b < 3; ++b) {
-        acc[6 + 6 * a + b] += FX[3 * a + b];
-        acc[6 + 6 * a + 3 + b] += Ft[3 * a + b];
-        acc[6 + 6 * (3 + a) + b] += Fx[3 * a + b] + DF[3 * a + b];
-        acc[6 + 6 * (3 + a) + 3 + b] += DT[3 * a + b];
+  int busy = 0, next = 0;  // threads with a sum; thread of the next corner
+  for (int base = 0; base < nc8; base += BSUM_N * BSUM_T) {
+    int n = block_compact<BSUM_N>([&](int i) { return base + i < nc8 && con[base + i] != 0; },
+                                  [&](int i) { return base + i; }, list, wsum);
+    // corner j of the list goes to thread (next + j) % BSUM_T
+    for (int j = (t - next + BSUM_T) % BSUM_T; j < n; j += BSUM_T) {
+      int i = list[j];
+      const double* f = cf + 3 * (size_t)i;
+      const double* d = cdv + 3 * (size_t)i;
+      const double* Ft = ct + 9 * (size_t)i;
+      double FX[9], Dx[9], Fx[9], DF[9], DT[9];
+      for (int e = 0; e < 9; ++e) FX[e] = ck[9 * (size_t)i + e];  // -d f / d y
+      cross_mat(d, Dx);
+      cross_mat(f, Fx);
+      mul33(Dx, FX, DF);
+      mul33(Dx, Ft, DT);
+      for (int a = 0; a < 3; ++a) {
+        acc[a] += f[a];
+        acc[3 + a] += d[(a + 1) % 3] * f[(a + 2) % 3] - d[(a + 2) % 3] * f[(a + 1) % 3];
+        for (int b = 0; b < 3; ++b) {
+          acc[6 + 6 * a + b] += FX[3 * a + b];
+          acc[6 + 6 * a + 3 + b] += Ft[3 * a + b];
+          acc[6 + 6 * (3 + a) + b] += Fx[3 * a + b] + DF[3 * a + b];
+          acc[6 + 6 * (3 + a) + 3 + b] += DT[3 * a + b];
+        }
       }
     }
+    busy = min(BSUM_T, busy + n);
+    next = (next + n) % BSUM_T;
+    __syncthreads();
   }
-  for (int e = 0; e < 42; ++e) {
-    double v = block_sum(acc[e], sh);
-    if (threadIdx.x == 0) out[e] = v;
+#pragma unroll
+  for (int h = 0; h < 3; ++h) {
+    if (t < busy)
+      for (int e = 0; e < 14; ++e) sh[e][t] = acc[14 * h + e];
+    __syncthreads();
+    for (int e = w; e < 14; e += BSUM_T / 32) {
+      double v = lane < busy ? sh[e][lane] : 0.0;
+      for (int u = lane + 32; u < busy; u += 32) v += sh[e][u];
+      v = warp_sum(v);
+      if (lane == 0) out[14 * h + e] = v;
+    }
+    __syncthreads();
   }
 }
 
 // the body's coupling columns and rows at the rows of the contact list (one
-// warp per row, a lane per output value, the row's corner entries in list
-// order): Kgb[j][3r + a] = d R_{r,a} / d q_j = sum phi (d f / d y)[a][j] for
-// the translation (j < 3) and -sum phi (d f / d qr)[a][j - 3] for the
-// rotation; Kbg[j][3r + b] = d Rb_j / d du_{r,b} = sum phi (d f / d y)[j][b]
-// (j < 3) and sum phi ([d]x d f / d y - [f]x)[j - 3][b]
-__global__ void k_body_rows(int nrow, const int* __restrict__ crow, const int* __restrict__ cptr,
-                            const int* __restrict__ cent, const double* __restrict__ cb_phi,
-                            const double* __restrict__ cf, const double* __restrict__ ck,
-                            const double* __restrict__ ct, const double* __restrict__ cdv,
-                            const int* __restrict__ con, long long n3, double* Kgb, double* Kbg) {
-  int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (t >= nrow) return;
+// block of 64 per row, a thread per output value, the row's corner entries in
+// contact in list order): Kgb[j][3r + a] = d R_{r,a} / d q_j = sum phi (d f /
+// d y)[a][j] for the translation (j < 3) and -sum phi (d f / d qr)[a][j - 3]
+// for the rotation; Kbg[j][3r + b] = d Rb_j / d du_{r,b} = sum phi (d f / d
+// y)[j][b] (j < 3) and sum phi ([d]x d f / d y - [f]x)[j - 3][b]
+__global__ void __launch_bounds__(64)
+    k_body_rows(const int* __restrict__ crow, const int* __restrict__ cptr, const int* __restrict__ cent,
+                const double* __restrict__ cb_phi, const double* __restrict__ cf, const double* __restrict__ ck,
+                const double* __restrict__ ct, const double* __restrict__ cdv, const int* __restrict__ con,
+                long long n3, double* Kgb, double* Kbg) {
+  __shared__ int list[64], wsum[2];
+  const int t = blockIdx.x, o = threadIdx.x;
   int r = crow[t], e0 = cptr[t], e1 = cptr[t + 1];
-  for (int o = lane; o < 36; o += 32) {
-    // o < 18: Kgb, component a = o / 6 of row r, body column j = o % 6;
-    // o >= 18: Kbg, body row j = (o - 18) / 3, component b = (o - 18) % 3
-    bool gb = o < 18;
-    int a = gb ? o / 6 : (o - 18) % 3, j = gb ? o % 6 : (o - 18) / 3;
-    double s = 0.0;
-    for (int e = e0; e < e1; ++e) {
-      int pk = cent[e], i = pk >> 5;
-      if (!con[i]) continue;
-      double ph = cb_phi[(size_t)i * MAXCB + (pk & 31)];
-      const double* Fm = ck + 9 * (size_t)i;  // -d f / d y
-      double v;
-      if (gb) {
-        v = j < 3 ? -Fm[3 * a + j] : -ct[9 * (size_t)i + 3 * a + (j - 3)];
-      } else if (j < 3) {
-        v = -Fm[3 * j + a];
-      } else {
-        const double* d = cdv + 3 * (size_t)i;
-        const double* f = cf + 3 * (size_t)i;
-        int jr = j - 3, j1 = (jr + 1) % 3, j2 = (jr + 2) % 3;
-        // ([d]x (d f / d y))[jr][a] - ([f]x)[jr][a]
-        double dF = -(d[j1] * Fm[3 * j2 + a] - d[j2] * Fm[3 * j1 + a]);
-        double fx = (a == j2 ? f[j1] : 0.0) - (a == j1 ? f[j2] : 0.0);
-        v = dF - fx;
+  // o < 18: Kgb, component a = o / 6 of row r, body column j = o % 6;
+  // o >= 18: Kbg, body row j = (o - 18) / 3, component b = (o - 18) % 3
+  bool gb = o < 18;
+  int a = gb ? o / 6 : (o - 18) % 3, j = gb ? o % 6 : (o - 18) / 3;
+  double s = 0.0;
+  for (int base = e0; base < e1; base += 64) {
+    int pk0 = base + o < e1 ? cent[base + o] : 0;
+    int n = block_compact<1>([&](int) { return base + o < e1 && con[pk0 >> 5] != 0; }, [&](int) { return pk0; }, list,
+                             wsum);
+    if (o < 36)
+      for (int u = 0; u < n; ++u) {
+        int pk = list[u], i = pk >> 5;
+        double ph = cb_phi[(size_t)i * MAXCB + (pk & 31)];
+        const double* Fm = ck + 9 * (size_t)i;  // -d f / d y
+        double v;
+        if (gb) {
+          v = j < 3 ? -Fm[3 * a + j] : -ct[9 * (size_t)i + 3 * a + (j - 3)];
+        } else if (j < 3) {
+          v = -Fm[3 * j + a];
+        } else {
+          const double* d = cdv + 3 * (size_t)i;
+          const double* f = cf + 3 * (size_t)i;
+          int jr = j - 3, j1 = (jr + 1) % 3, j2 = (jr + 2) % 3;
+          // ([d]x (d f / d y))[jr][a] - ([f]x)[jr][a]
+          double dF = -(d[j1] * Fm[3 * j2 + a] - d[j2] * Fm[3 * j1 + a]);
+          double fx = (a == j2 ? f[j1] : 0.0) - (a == j1 ? f[j2] : 0.0);
+          v = dF - fx;
+        }
+        s += ph * v;
       }
-      s += ph * v;
-    }
-    if (gb)
-      Kgb[(size_t)j * n3 + 3 * (size_t)r + a] = s;
-    else
-      Kbg[(size_t)j * n3 + 3 * (size_t)r + a] = s;
+    __syncthreads();
   }
+  if (o >= 36) return;
+  if (gb)
+    Kgb[(size_t)j * n3 + 3 * (size_t)r + a] = s;
+  else
+    Kbg[(size_t)j * n3 + 3 * (size_t)r + a] = s;
 }
 
 // Newmark inertia of each point (time steps): m_p a_p with
@@ -1172,105 +1230,151 @@ __global__ void k_inertia_rows(int nd, int P, const long long* __restrict__ sptr
 }
 
 // the consistent mass of a time step, (2 / dt^2) m_p S_vp S_wp I, added to the
-// tangent's diagonal entries: one warp per row r, the row's point sources in
-// key order, the lanes over the source point's support (distinct columns),
+// tangent's diagonal entries: one block per row r, its warps taking a
+// contiguous part of the row's point sources each (the lanes over the source
+// point's support) into their own copy of the row's sums in shared memory, by
+// the row positions of the tangent gather; the copies added in warp order,
 // the Dirichlet components skipped
 template <class T>
-__global__ void k_mass_rows(int nd, int P, const long long* __restrict__ sptr,
-                            const uint64_t* __restrict__ skeys, const int* __restrict__ nsup,
-                            const int* __restrict__ sidx, const double* __restrict__ S,
-                            const double* __restrict__ mass, double c2, const int* __restrict__ rp,
-                            const int* __restrict__ col, Sliced SL, const int* __restrict__ mask, T* K) {
-  int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (r >= nd) return;
-  int s0r = rp[r], ma = mask[r];
-  int srr = SL.pos[r], slc = srr >> 5, W = SL.w[slc];
-  long long b0 = SL.base[slc];
-  for (long long q = sptr[r]; q < sptr[r + 1]; ++q) {
+__global__ void k_mass_rows(int P, int pw, int mr, const long long* __restrict__ sptr,
+                            const uint64_t* __restrict__ skeys, const unsigned short* __restrict__ spos,
+                            const double* __restrict__ S, const double* __restrict__ mass, double c2,
+                            const int* __restrict__ rp, const int* __restrict__ col, Sliced SL,
+                            const int* __restrict__ mask, T* K) {
+  extern __shared__ double smm[];
+  const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, nw = blockDim.x >> 5, r = blockIdx.x;
+  double* acc = smm + (size_t)wi * mr;
+  int s0 = rp[r], nb = rp[r + 1] - s0;
+  for (int i = lane; i < nb; i += 32) acc[i] = 0.0;
+  __syncwarp();
+  long long q0 = sptr[r], n = sptr[r + 1] - q0;
+  for (long long q = q0 + n * wi / nw; q < q0 + n * (wi + 1) / nw; ++q) {
     uint32_t sid = (uint32_t)skeys[q];
     int w = (int)(sid >> 6), k = (int)(sid & 63);
     if (w >= P) continue;
     double sk = c2 * mass[w] * S[(size_t)w * MAXS + k];
-    int n = nsup[w];
-    for (int l = lane; l < n; l += 32) {
-      size_t o = (size_t)w * MAXS + l;
-      int cb = sidx[o];
-      int sl = find_slot(rp, col, r, cb);
-      if (sl < 0) continue;
-      long long slot = sliced_slot(b0, srr, sl - s0r);
-      int mb = mask[cb];
-      double v = sk * S[o];
-      for (int a = 0; a < 3; ++a) {
-        if (((ma >> a) & 1) || ((mb >> a) & 1)) continue;
-        T* kv = K + sliced_entry(b0, W, slot, 4 * a);
-        *kv += (T)v;
-      }
+    for (int l = lane; l < pw; l += 32) {
+      unsigned p = spos[(size_t)q * pw + l];
+      if (p != 0xffffu) acc[p] += sk * S[(size_t)w * MAXS + l];
     }
     __syncwarp();
   }
+  __syncthreads();
+  int ma = mask[r], srr = SL.pos[r], slc = srr >> 5, W = SL.w[slc];
+  long long b0 = SL.base[slc];
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+    double v = smm[i];
+    for (int u = 1; u < nw; ++u) v += smm[(size_t)u * mr + i];
+    int m = ma | mask[col[s0 + i]];
+    long long slot = sliced_slot(b0, srr, i);
+    for (int a = 0; a < 3; ++a)
+      if (!((m >> a) & 1)) {
+        T* kv = K + sliced_entry(b0, W, slot, 4 * a);
+        *kv += (T)v;
+      }
+  }
 }
 
-// One warp per row r of the contact list (the rows that the background basis
+// One block per row r of the contact list (the rows that the background basis
 // of some candidate corner touches; entries (corner, basis entry) in sorted
-// order).  RES: R_r -= sum of phi_e f and f_c,r += the same sum, lanes strided
-// over the entries and combined by the fixed shuffle tree.  TANGENT: K_{r,b}
-// += phi_e phi_b k_c over the basis entries b of each corner, one corner entry
-// at a time in list order (the lanes of one entry write distinct columns), the
-// Dirichlet components skipped.  No atomics: the same sums on every run.
+// order).  RES: R_r -= sum of phi_e f and f_c,r += the same sum, threads strided
+// over the entries, each warp's by the fixed shuffle tree, the warps in order.
+// TANGENT: K_{r,b} += phi_e phi_b k_c over the basis entries b of each corner
+// in contact, the Dirichlet components skipped.  Each warp takes the entries
+// 32 at a time in turn, looks which of their corners are in contact (most are
+// not) in one step, and adds into its own copy of the row in shared memory, 9
+// lanes per column as in the FP64 tangent gather; the copies are added in warp
+// order.  No atomics: the same sums on every run.  (A warp per row that walked
+// the list entry by entry, a flag and a binary search in memory per corner,
+// took 346 us on the punch's 81 k corners; 240 on the cone's.)
 template <class T, bool RES, bool TANGENT>
-__global__ void k_contact_rows(int nrow, const int* __restrict__ crow, const int* __restrict__ cptr,
-                               const int* __restrict__ cent, const int* __restrict__ cb_n,
-                               const int* __restrict__ cb_idx, const double* __restrict__ cb_phi,
-                               const double* __restrict__ cf, const double* __restrict__ ck,
-                               const int* __restrict__ con, double* R, double* fc,
-                               const int* __restrict__ rp, const int* __restrict__ col, Sliced S,
-                               const int* __restrict__ mask, T* K) {
-  int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (t >= nrow) return;
-  int r = crow[t], e0 = cptr[t], e1 = cptr[t + 1];
+__global__ void __launch_bounds__(128)
+    k_contact_rows(int mr, const int* __restrict__ crow, const int* __restrict__ cptr, const int* __restrict__ cent,
+                   const int* __restrict__ cb_n, const int* __restrict__ cb_idx, const double* __restrict__ cb_phi,
+                   const double* __restrict__ cf, const double* __restrict__ ck, const int* __restrict__ con,
+                   double* R, double* fc, const int* __restrict__ rp, const int* __restrict__ col, Sliced S,
+                   const int* __restrict__ mask, T* K) {
+  extern __shared__ double smc[];
+  __shared__ double fs[3][4];
+  __shared__ int touched;
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int t = blockIdx.x, r = crow[t], e0 = cptr[t], e1 = cptr[t + 1];
   if (RES) {
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    for (int e = e0 + lane; e < e1; e += 32) {
+    for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
       int pk = cent[e], i = pk >> 5;
+      if (!con[i]) continue;  // (no force)
       double ph = cb_phi[(size_t)i * MAXCB + (pk & 31)];
       s0 += ph * cf[3 * (size_t)i];
       s1 += ph * cf[3 * (size_t)i + 1];
       s2 += ph * cf[3 * (size_t)i + 2];
     }
-    s0 = warp_sum(s0);
-    s1 = warp_sum(s1);
-    s2 = warp_sum(s2);
-    if (lane < 3) {
-      double v = lane == 0 ? s0 : (lane == 1 ? s1 : s2);
-      R[3 * (size_t)r + lane] -= v;
-      fc[3 * (size_t)r + lane] += v;
+    if (__any_sync(FULL, s0 != 0.0 || s1 != 0.0 || s2 != 0.0)) {
+      s0 = warp_sum(s0);
+      s1 = warp_sum(s1);
+      s2 = warp_sum(s2);
+    }
+    if (lane < 3) fs[lane][wi] = lane == 0 ? s0 : (lane == 1 ? s1 : s2);
+    __syncthreads();
+    if (threadIdx.x < 3) {
+      double v = 0.0;
+      for (int w = 0; w < nw; ++w) v += fs[threadIdx.x][w];
+      R[3 * (size_t)r + threadIdx.x] -= v;
+      fc[3 * (size_t)r + threadIdx.x] += v;
     }
   }
   if (!TANGENT) return;
-  int s0r = rp[r], ma = mask[r];
-  int srr = S.pos[r], slc = srr >> 5, W = S.w[slc];
-  long long b0 = S.base[slc];
-  for (int e = e0; e < e1; ++e) {
-    int pk = cent[e], i = pk >> 5;
-    if (!con[i]) continue;
-    const double* kc = ck + 9 * (size_t)i;
-    double pa = cb_phi[(size_t)i * MAXCB + (pk & 31)];
-    int n = cb_n[i];
-    for (int eb = lane; eb < n; eb += 32) {
-      int cb = cb_idx[(size_t)i * MAXCB + eb];
-      int sl = find_slot(rp, col, r, cb);
-      if (sl < 0) continue;
-      long long slot = sliced_slot(b0, srr, sl - s0r);
-      int mb = mask[cb];
-      double pp = pa * cb_phi[(size_t)i * MAXCB + eb];
-      for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) {
-          if (((ma >> a) & 1) || ((mb >> b) & 1)) continue;
-          T* kv = K + sliced_entry(b0, W, slot, 3 * a + b);
-          *kv += (T)(pp * kc[3 * a + b]);
-        }
+  const size_t wsz = 9 * (size_t)mr + 64;
+  double* sph = smc + wi * wsz;  // phi_e phi_b of the current entry's columns, then their positions
+  int* spo = (int*)(sph + 32);
+  double* acc = sph + 64;
+  int s0r = rp[r], nb = rp[r + 1] - s0r;
+  if (threadIdx.x == 0) touched = 0;
+  bool mine = false;
+  const int k = lane % 9, cg = lane < 27 ? lane / 9 : 1 << 20;
+  for (int base = e0 + 32 * wi; base < e1; base += 32 * nw) {
+    int pk0 = base + lane < e1 ? cent[base + lane] : 0;
+    unsigned on = __ballot_sync(FULL, base + lane < e1 && con[pk0 >> 5] != 0);
+    if (on && !mine) {
+      for (int i = lane; i < 9 * nb; i += 32) acc[i] = 0.0;
+      mine = true;
     }
-    __syncwarp();
+    while (on) {
+      int pk = __shfl_sync(FULL, pk0, __ffs(on) - 1), i = pk >> 5;
+      on &= on - 1;
+      int n = cb_n[i];
+      double kc = lane < 27 ? ck[9 * (size_t)i + k] : 0.0;
+      __syncwarp();
+      if (lane < n) {
+        spo[lane] = find_slot(rp, col, r, cb_idx[(size_t)i * MAXCB + lane]) - s0r;
+        sph[lane] = cb_phi[(size_t)i * MAXCB + (pk & 31)] * cb_phi[(size_t)i * MAXCB + lane];
+      }
+      __syncwarp();
+      for (int c = cg; c < n; c += 3)
+        if (spo[c] >= 0) acc[9 * spo[c] + k] += sph[c] * kc;
+    }
+  }
+  // (the copies of the warps that met no corner in contact count as zero)
+  __syncthreads();
+  if (mine && lane == 0) atomicOr(&touched, 1 << wi);
+  __syncthreads();
+  int used = touched;
+  if (!used) return;
+  int ma = mask[r], srr = S.pos[r], slc = srr >> 5, W = S.w[slc];
+  long long b0 = S.base[slc];
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+    int mb = mask[col[s0r + i]];
+    long long slot = sliced_slot(b0, srr, i);
+    for (int a = 0; a < 3; ++a)
+      for (int b = 0; b < 3; ++b) {
+        double v = 0.0;
+        for (int w = 0; w < nw; ++w)
+          if ((used >> w) & 1) v += smc[w * wsz + 64 + 9 * i + 3 * a + b];
+        if (v == 0.0 || ((ma >> a) & 1) || ((mb >> b) & 1)) continue;
+        T* kv = K + sliced_entry(b0, W, slot, 3 * a + b);
+        *kv += (T)v;
+      }
   }
 }
 
@@ -1341,16 +1445,21 @@ void contact_terms(mpm_ctx* c, mpm_mesh* m, const mpm_material& mat, const mpm_r
       mat.pf, mat.pt, mat.mu, bi, du, cf, ck, con, ct, cdv, reac,
       grid_red(c, 3, grid_for(n8, 128))));
   if (couple && bsum)
-    MPM_LAUNCH_P(MPM_PROF_CONTACT, k_body_sums<<<1, 256, 0, st>>>(n8, cf, ck, ct, cdv, con, bsum));
+    MPM_LAUNCH_P(MPM_PROF_CONTACT, k_body_sums<<<1, BSUM_T, 0, st>>>(n8, cf, ck, ct, cdv, con, bsum));
   if (!m->nct) return;
   Sliced S = sliced_view(m);
-  MPM_LAUNCH_P(MPM_PROF_CONTACT, k_contact_rows<T, RES, TANGENT><<<grid_for(m->nct, 4), 128, 0, st>>>(
-      m->nct, ptr<int>(m->ct_row), ptr<int>(m->ct_ptr), ptr<int>(m->ct_ent), ptr<int>(m->cb_n),
+  // 128 threads per row, fewer where four copies of the longest row do not fit
+  size_t wb = TANGENT ? sizeof(double) * (9 * (size_t)m->maxrow + 64) : 0;
+  int nw = TANGENT ? (int)std::min<size_t>(4, (size_t)(200 * 1024) / wb) : 4;
+  auto kern = k_contact_rows<T, RES, TANGENT>;
+  MPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(nw * wb)));
+  MPM_LAUNCH_P(MPM_PROF_CONTACT, kern<<<m->nct, 32 * nw, nw * wb, st>>>(
+      m->maxrow, ptr<int>(m->ct_row), ptr<int>(m->ct_ptr), ptr<int>(m->ct_ent), ptr<int>(m->cb_n),
       ptr<int>(m->cb_idx), ptr<double>(m->cb_phi), cf, ck, con, R, fc, ptr<int>(m->row_ptr),
       ptr<int>(m->col), S, ptr<int>(m->dof_mask), K));
   if (TANGENT && couple && dyn->Kgb && dyn->Kbg)
-    MPM_LAUNCH_P(MPM_PROF_CONTACT, k_body_rows<<<grid_for(m->nct, 4), 128, 0, st>>>(
-        m->nct, ptr<int>(m->ct_row), ptr<int>(m->ct_ptr), ptr<int>(m->ct_ent),
+    MPM_LAUNCH_P(MPM_PROF_CONTACT, k_body_rows<<<m->nct, 64, 0, st>>>(
+        ptr<int>(m->ct_row), ptr<int>(m->ct_ptr), ptr<int>(m->ct_ent),
         ptr<double>(m->cb_phi), cf, ck, ct, cdv, con, 3LL * m->ndof, dyn->Kgb, dyn->Kbg));
 }
 
@@ -1553,14 +1662,17 @@ void assemble(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const mpm
       MPM_LAUNCH_P(MPM_PROF_TANGENT, k_tangent_mirror<<<grid_for(32LL * nd, 256), 256, 0, st>>>(nd, rp, col, S, (double*)K));
     if (inertia) {
       double c2 = 2.0 / (dyn->dt * dyn->dt);
+      size_t smem = 4 * sizeof(double) * (size_t)m->maxrow;
+      auto launch = [&](auto kern, auto* Kt) {
+        MPM_LAUNCH_P(MPM_PROF_TANGENT, kern<<<nd, 128, smem, st>>>(
+            P, pw, m->maxrow, ptr<long long>(m->src_ptr), ptr<uint64_t>(m->src_key),
+            ptr<unsigned short>(m->src_pos), ptr<double>(m->S), ptr<double>(m->pmass), c2, rp, col, S,
+            ptr<int>(m->dof_mask), Kt));
+      };
       if (mixed)
-        MPM_LAUNCH_P(MPM_PROF_TANGENT, k_mass_rows<float><<<grid_for(nd, 4), 128, 0, st>>>(
-            nd, P, ptr<long long>(m->src_ptr), ptr<uint64_t>(m->src_key), nsup, sidx, ptr<double>(m->S),
-            ptr<double>(m->pmass), c2, rp, col, S, ptr<int>(m->dof_mask), (float*)K));
+        launch(k_mass_rows<float>, (float*)K);
       else
-        MPM_LAUNCH_P(MPM_PROF_TANGENT, k_mass_rows<double><<<grid_for(nd, 4), 128, 0, st>>>(
-            nd, P, ptr<long long>(m->src_ptr), ptr<uint64_t>(m->src_key), nsup, sidx, ptr<double>(m->S),
-            ptr<double>(m->pmass), c2, rp, col, S, ptr<int>(m->dof_mask), (double*)K));
+        launch(k_mass_rows<double>, (double*)K);
     }
     int npad = 32 * m->nslice;
     if (npad > nd) {
