@@ -96,10 +96,10 @@ __device__ bool law_state(const Law& L, double E, double ys, const double* be6, 
   bt[5] = bt[7] = 0.5 * (bt[5] + bt[7]);
   jacobi3(bt, S.lam, S.Q);
   if (!(S.lam[0] > 0 && S.lam[1] > 0 && S.lam[2] > 0)) return false;
-  for (int a = 0; a < 3; ++a) S.eps[a] = 0.5 * log(S.lam[a]);
+  for (int a = 0; a < 3; ++a) S.eps[a] = 0.5 * log_stretch(S.lam[a]);
   principal_return(L, E, ys, S.eps, S.ta, S.dd, &S.gr);
-  S.mu = E / (2.0 * (1.0 + L.nu));
-  S.lm = E * L.nu / ((1.0 + L.nu) * (1.0 - 2.0 * L.nu));
+  S.mu = E * L.cmu;
+  S.lm = E * L.clm;
   S.kb = S.lm + 2.0 * S.mu / 3.0;
   double tr = S.eps[0] + S.eps[1] + S.eps[2], dn = 0.0;
   for (int a = 0; a < 3; ++a) {

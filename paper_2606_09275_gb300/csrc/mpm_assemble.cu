@@ -156,15 +156,14 @@ __device__ bool point_update_law(const Law& L, double E, double ys, const double
   jacobi3(bt, lam, Q);
   if (!(lam[0] > 0.0 && lam[1] > 0.0 && lam[2] > 0.0) || !isfinite(lam[0] + lam[1] + lam[2]))
     return false;
-  double eps[3] = {0.5 * log(lam[0]), 0.5 * log(lam[1]), 0.5 * log(lam[2])};
+  double eps[3] = {0.5 * log_stretch(lam[0]), 0.5 * log_stretch(lam[1]), 0.5 * log_stretch(lam[2])};
   double ta[3], dd[9], gr;
   principal_return(L, E, ys, eps, ta, dd, &gr);
-  double mu = E / (2.0 * (1.0 + L.nu));
-  double lm = E * L.nu / ((1.0 + L.nu) * (1.0 - 2.0 * L.nu));
-  double tt = ta[0] + ta[1] + ta[2];
+  double mu = E * L.cmu, lm = E * L.clm;
+  double tt = ta[0] + ta[1] + ta[2], tm = lm * tt / (3.0 * lm + 2.0 * mu), imu = 1.0 / mu;
   double bw[3];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) bw[a] = exp(2.0 * (ta[a] - lm * tt / (3.0 * lm + 2.0 * mu)) / (2.0 * mu));
+  for (int a = 0; a < 3; ++a) bw[a] = exp((ta[a] - tm) * imu);
   // tau = Q diag(ta) Q^T, b_e = Q diag(bw) Q^T
   const int ii[6] = {0, 1, 2, 0, 1, 0}, jj[6] = {0, 1, 2, 1, 2, 2};
 #pragma unroll
