@@ -14,56 +14,72 @@ namespace {
 
 // ------------------------------------------------------------------ kinematics
 
-// dF = I + sum_v du_v (x) grad S_vp; eight lanes per point, four points per warp
-__global__ void k_kinematics(int P, const int* __restrict__ nsup, const int* __restrict__ sidx,
-                             const double* __restrict__ dS, const double* __restrict__ du,
-                             double* dF) {
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  int w = (int)(t >> 3), sub = (int)(t & 7);
+// dF = I + sum_v du_v (x) grad S_vp, four lanes per point.  Bound by the FP64
+// rate: an FP64 instruction takes 16 SM cycles whatever the number of active
+// lanes, so a warp costs the longest support of its points (8, 12, 18 or 27
+// nodes in the interior, mixed within a cell).  Each block therefore deals its
+// points to the warps in order of support size (counted in shared memory, in
+// integers).  Per point 6 FP64 instructions instead of 10.5 with eight lanes
+// in point order; indentation, 1.9 M points: 1.35 -> 0.65 ms.
+constexpr int KIN_T = 256, KIN_P = KIN_T / 4;  // threads and points of a block
+__global__ void __launch_bounds__(KIN_T)
+    k_kinematics(int P, const int* __restrict__ nsup, const int* __restrict__ sidx, const double* __restrict__ dS,
+                 const double* __restrict__ du, double* dF) {
+  __shared__ int size[KIN_P], order[KIN_P];
+  const int w0 = blockIdx.x * KIN_P, np = min(KIN_P, P - w0), t = threadIdx.x;
+  if (t < np) size[t] = nsup[w0 + t];
+  __syncthreads();
+  {
+    // rank of point t / 4 among the block's, its four threads comparing a quarter each
+    int p = t >> 2, rank = 0;
+    if (p < np) {
+      int n = size[p];
+      for (int j = t & 3; j < np; j += 4) rank += size[j] < n || (size[j] == n && j < p);
+    }
+    rank += __shfl_xor_sync(0xffffffffu, rank, 1);
+    rank += __shfl_xor_sync(0xffffffffu, rank, 2);
+    if (p < np && (t & 3) == 0) order[rank] = p;
+  }
+  __syncthreads();
+  const int sub = t & 3;
+  bool in = (t >> 2) < np;
+  int p = in ? order[t >> 2] : 0, n = in ? size[p] : 0;
+  size_t w = (size_t)w0 + p;
   double a[9];
 #pragma unroll
   for (int i = 0; i < 9; ++i) a[i] = 0.0;
-  if (w < P) {
-    int n = nsup[w];
-    for (int k = sub; k < n; k += 8) {
-      size_t o = (size_t)w * MAXS + k;
-      int j = sidx[o];
-      double u0 = du[3 * (size_t)j], u1 = du[3 * (size_t)j + 1], u2 = du[3 * (size_t)j + 2];
-      double g0 = dS[3 * o], g1 = dS[3 * o + 1], g2 = dS[3 * o + 2];
-      a[0] += u0 * g0; a[1] += u0 * g1; a[2] += u0 * g2;
-      a[3] += u1 * g0; a[4] += u1 * g1; a[5] += u1 * g2;
-      a[6] += u2 * g0; a[7] += u2 * g1; a[8] += u2 * g2;
-    }
+  for (int k = sub; k < n; k += 4) {
+    size_t o = w * MAXS + k;
+    int j = sidx[o];
+    double u0 = du[3 * (size_t)j], u1 = du[3 * (size_t)j + 1], u2 = du[3 * (size_t)j + 2];
+    double g0 = dS[3 * o], g1 = dS[3 * o + 1], g2 = dS[3 * o + 2];
+    a[0] += u0 * g0; a[1] += u0 * g1; a[2] += u0 * g2;
+    a[3] += u1 * g0; a[4] += u1 * g1; a[5] += u1 * g2;
+    a[6] += u2 * g0; a[7] += u2 * g1; a[8] += u2 * g2;
   }
-  // reduce-scatter of a[0..7] over the 8 lanes of the point (lane sub ends
-  // with the sum of a[sub]: 7 FP64 additions instead of 24; the FP64 pipe
-  // bounds this kernel), a[8] by a butterfly
+  // reduce-scatter of a[0..7] over the 4 lanes (lane sub ends with the sums of
+  // a[2 sub'], a[2 sub' + 1] in bit-reversed order), a[8] by a butterfly
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    bool up = sub & 4;
+    bool up = sub & 2;
     double send = up ? a[i] : a[i + 4];
     double keep = up ? a[i + 4] : a[i];
-    a[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+    a[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
   }
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
-    bool up = sub & 2;
+    bool up = sub & 1;
     double send = up ? a[i] : a[i + 2];
     double keep = up ? a[i + 2] : a[i];
-    a[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
+    a[i] = keep + __shfl_xor_sync(0xffffffffu, send, 1);
   }
-  {
-    bool up = sub & 1;
-    double send = up ? a[0] : a[1];
-    double keep = up ? a[1] : a[0];
-    a[0] = keep + __shfl_xor_sync(0xffffffffu, send, 1);
-  }
-  a[8] += __shfl_xor_sync(0xffffffffu, a[8], 4);
   a[8] += __shfl_xor_sync(0xffffffffu, a[8], 2);
   a[8] += __shfl_xor_sync(0xffffffffu, a[8], 1);
-  if (w < P) {
-    dF[9 * (size_t)w + sub] = a[0] + ((sub % 4 == 0) ? 1.0 : 0.0);
-    if (sub == 0) dF[9 * (size_t)w + 8] = a[8] + 1.0;
+  if (in) {
+    int e = 2 * sub;  // entries e and e + 1; 0 and 4 lie on the diagonal
+    dF[9 * w + e] = a[0] + ((e & 3) == 0 ? 1.0 : 0.0);
+    dF[9 * w + e + 1] = a[1];
+    if (sub == 0) dF[9 * w + 8] = a[8] + 1.0;
   }
 }
 
@@ -307,6 +323,23 @@ __global__ void k_dS_to_float(int P, const int* __restrict__ nsup, const double*
 // gather: every lane sums a fixed set of sources in key order and the lanes
 // are combined by a fixed shuffle tree, so f_int and R are the same bit for
 // bit on every run (no floating-point atomics).
+// Bound by the FP64 rate and the L2: per row 9 multiply-adds per 32 sources,
+// 6 additions for the three sums over the lanes, and the ghost term only where
+// the row has one (its coefficients are tested as integers).  Indentation,
+// 1.9 M points: 1.85 ms with six shuffle trees of 5 additions and an FP64
+// compare per block, 1.21 so.
+__device__ inline double sum3_scatter(double f0, double f1, double f2, int lane) {
+  // lane 0 ends with the sum of f0 over the warp, lane 16 of f1, lane 8 of f2
+  bool up = lane & 16;
+  double a = (up ? f1 : f0) + __shfl_xor_sync(0xffffffffu, up ? f0 : f1, 16);
+  f2 += __shfl_xor_sync(0xffffffffu, f2, 16);
+  up = lane & 8;
+  a = (up ? f2 : a) + __shfl_xor_sync(0xffffffffu, up ? a : f2, 8);
+  a += __shfl_xor_sync(0xffffffffu, a, 4);
+  a += __shfl_xor_sync(0xffffffffu, a, 2);
+  return a + __shfl_xor_sync(0xffffffffu, a, 1);
+}
+
 __global__ void k_residual_rows(int nd, int P, double load, const long long* __restrict__ sptr,
                                 const uint64_t* __restrict__ skeys, const double* __restrict__ M,
                                 const double* __restrict__ dS, const int* __restrict__ rp,
@@ -325,30 +358,26 @@ __global__ void k_residual_rows(int nd, int P, double load, const long long* __r
     double2 m01 = m[0], m23 = m[1], m45 = m[2], m67 = m[3], m8x = m[4];
     const double* a = dS + 3 * ((size_t)w * MAXS + k);
     double a0 = a[0], a1 = a[1], a2 = a[2];
-    f0 += m01.x * a0 + m01.y * a1 + m23.x * a2;
-    f1 += m23.y * a0 + m45.x * a1 + m45.y * a2;
-    f2 += m67.x * a0 + m67.y * a1 + m8x.x * a2;
+    f0 = fma(m23.x, a2, fma(m01.y, a1, fma(m01.x, a0, f0)));
+    f1 = fma(m45.y, a2, fma(m45.x, a1, fma(m23.y, a0, f1)));
+    f2 = fma(m8x.x, a2, fma(m67.y, a1, fma(m67.x, a0, f2)));
   }
   double g0 = 0.0, g1 = 0.0, g2 = 0.0;
+  bool ghost = false;
   for (int s = rp[r] + lane; s < rp[r + 1]; s += 32) {
     double k = kg[s];
-    if (k != 0.0) {
+    if (__double_as_longlong(k) << 1) {
       int c = col[s];
+      ghost = true;
       g0 += k * du[3 * (size_t)c];
       g1 += k * du[3 * (size_t)c + 1];
       g2 += k * du[3 * (size_t)c + 2];
     }
   }
-  f0 = warp_sum(f0);
-  f1 = warp_sum(f1);
-  f2 = warp_sum(f2);
-  g0 = warp_sum(g0);
-  g1 = warp_sum(g1);
-  g2 = warp_sum(g2);
-  if (lane < 3) {
-    double f = lane == 0 ? f0 : (lane == 1 ? f1 : f2);
-    double g = lane == 0 ? g0 : (lane == 1 ? g1 : g2);
-    size_t i = 3 * (size_t)r + lane;
+  double f = sum3_scatter(f0, f1, f2, lane), g = 0.0;
+  if (__any_sync(0xffffffffu, ghost)) g = sum3_scatter(g0, g1, g2, lane);
+  if (lane == 0 || lane == 8 || lane == 16) {
+    size_t i = 3 * (size_t)r + (lane == 16 ? 1 : lane == 8 ? 2 : 0);
     fint[i] = f;
     R[i] = f - load * fext[i] + g;
   }
@@ -1619,7 +1648,7 @@ void assemble(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const mpm
       MPM_LAUNCH_P(MPM_PROF_FORCE, k_gx<double, double><<<grid_for(8LL * P, 256), 256, 0, st>>>(P, pw, nsup, dS, dFinv, (double*)gx));
     }
   } else {
-    MPM_LAUNCH_P(MPM_PROF_KINEMATICS, k_kinematics<<<grid_for(8LL * P, 256), 256, 0, st>>>(P, nsup, sidx, dS, du, dF));
+    MPM_LAUNCH_P(MPM_PROF_KINEMATICS, k_kinematics<<<grid_for(P, KIN_P), KIN_T, 0, st>>>(P, nsup, sidx, dS, du, dF));
     if (!K)
       MPM_LAUNCH_P(MPM_PROF_CONSTITUTIVE, k_constitutive<false, double><<<grid_for(P, 128), 128, 0, st>>>(
           P, L, ptr<double>(m->pE), ptr<double>(m->pys), ptr<double>(m->pbe), dF, V0, tau, dFinv, Mf,
