@@ -1436,7 +1436,7 @@ __global__ void k_norms(int n3, const double* __restrict__ R, const double* __re
 double norm_free(mpm_ctx* c, const mpm_mesh* m, const double* R) {
   double* slot = c->d_red + 16;
   MPM_CUDA(cudaMemsetAsync(slot, 0, 4 * sizeof(double), c->stream));
-  MPM_LAUNCH(k_norms<<<4 * 152, 256, 0, c->stream>>>(3 * m->ndof, R, nullptr, nullptr, nullptr, 0.0,
+  MPM_LAUNCH(k_norms<<<grid_strided(3 * m->ndof), 256, 0, c->stream>>>(3 * m->ndof, R, nullptr, nullptr, nullptr, 0.0,
                                           nullptr, ptr<int>(m->dof_mask), slot, grid_red(c, 4, 4 * 152)));
   MPM_CUDA(cudaMemcpyAsync(c->h_red + 16, slot, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   MPM_CUDA(cudaStreamSynchronize(c->stream));
@@ -1734,7 +1734,7 @@ void assemble(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const mpm
   if (want_norms) {
     double* slot = c->d_red + 16;
     MPM_CUDA(cudaMemsetAsync(slot, 0, 4 * sizeof(double), st));
-    MPM_LAUNCH(k_norms<<<4 * 152, 256, 0, st>>>(3 * nd, R, fint, ptr<double>(m->fext), fc, load, finert,
+    MPM_LAUNCH(k_norms<<<grid_strided(3 * nd), 256, 0, st>>>(3 * nd, R, fint, ptr<double>(m->fext), fc, load, finert,
                                      ptr<int>(m->dof_mask), slot, grid_red(c, 4, 4 * 152)));
     MPM_CUDA(cudaMemcpyAsync(c->h_red + 16, slot, 7 * sizeof(double), cudaMemcpyDeviceToHost, st));
     MPM_CUDA(cudaStreamSynchronize(st));

@@ -332,6 +332,13 @@ inline int grid_for(long long n, int block) {
   return (int)(g < 1 ? 1 : g);
 }
 
+// blocks of 256 threads of a grid-stride kernel over n entries: as many as
+// there is work for, at most 4 per SM
+inline int grid_strided(long long n) {
+  int g = grid_for(n, 256);
+  return g < 4 * 152 ? g : 4 * 152;
+}
+
 // ------------------------------------------------------------------ Morton codes
 
 __host__ __device__ inline uint64_t spread3(uint64_t v) {
@@ -744,24 +751,45 @@ __device__ inline double block_sum(double v, double* sh) {
 
 // ------------------------------------------------------------------ fixed-order grid sums
 //
-// Sums over a whole grid without floating-point atomics.  Each block reduces
-// its threads' values with the fixed shuffle tree of block_sum and stores the
+// Sums over a whole grid without floating-point atomics.  Each block adds its
+// threads' values in a fixed order and stores the
 // result in its own slot; the block that finishes last (elected by an integer
 // ticket) adds the slots in block order.  For a given launch shape the result
 // is the same bit for bit on every run, whatever order the blocks run in, so
 // the Newton path (its residual norms, line search, Krylov scalars) is
 // reproducible.  Every block of the grid must reach grid_sum (or none: a
 // kernel may return early only where all of its blocks do).
+// The values of a block are added up through shared memory by one warp per sum
+// (7 + 5 additions of a warp for 256 threads): an FP64 instruction costs 16 SM
+// cycles for every warp that executes it, and a shuffle tree in all 8 warps
+// took 45 (k_norms 23 -> 16 us at 744 k unknowns, 16 -> 6 at 2 k).
+// blockDim.x at most 256.
 template <int NV>
 __device__ inline void grid_sum(const double* v, double* const* out, GridRed g) {
-  __shared__ double gsh[32];
+  __shared__ double gsh[NV][256];
   __shared__ int glast;
+  const int t = threadIdx.x, w = t >> 5, l = t & 31, nw = blockDim.x >> 5;
+  auto block = [&](int i) {
+    double s = gsh[i][l];
+    for (int j = l + 32; j < (int)blockDim.x; j += 32) s += gsh[i][j];
+    return warp_sum(s);
+  };
 #pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    double s = block_sum(v[i], gsh);
-    if (threadIdx.x == 0) g.part[(size_t)i * gridDim.x + blockIdx.x] = s;
+  for (int i = 0; i < NV; ++i) gsh[i][t] = v[i];
+  __syncthreads();
+  if (gridDim.x == 1) {
+    for (int i = w; i < NV; i += nw) {
+      double s = block(i);
+      if (l == 0 && out[i]) *out[i] += s;
+    }
+    return;
   }
-  if (threadIdx.x == 0) {
+  for (int i = w; i < NV; i += nw) {
+    double s = block(i);
+    if (l == 0) g.part[(size_t)i * gridDim.x + blockIdx.x] = s;
+  }
+  __syncthreads();
+  if (t == 0) {
     __threadfence();
     glast = atomicAdd(g.ticket, 1u) == gridDim.x - 1;
   }
@@ -771,12 +799,15 @@ __device__ inline void grid_sum(const double* v, double* const* out, GridRed g) 
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
     double s = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
-      s += __ldcg(g.part + (size_t)i * gridDim.x + b);
-    s = block_sum(s, gsh);
-    if (threadIdx.x == 0 && out[i]) *out[i] += s;
+    for (int b = t; b < (int)gridDim.x; b += blockDim.x) s += __ldcg(g.part + (size_t)i * gridDim.x + b);
+    gsh[i][t] = s;
   }
-  if (threadIdx.x == 0) *g.ticket = 0u;
+  __syncthreads();
+  for (int i = w; i < NV; i += nw) {
+    double s = block(i);
+    if (l == 0 && out[i]) *out[i] += s;
+  }
+  if (t == 0) *g.ticket = 0u;
 }
 
 __device__ inline void grid_sum1(double v, double* out, GridRed g) {

@@ -181,7 +181,7 @@ void newton(mpm_ctx* c, mpm_mesh* m, const mpm_material* mat, const mpm_rigid& b
           if (sz.status) throw CudaError(sz.status, c->err);
         }
         MPM_CUDA(cudaMemsetAsync(dots, 0, 64 * sizeof(double), s));
-        int gb = std::min(grid_for(n3, 256), 4 * 152);
+        int gb = grid_strided(n3);
         for (int j = 0; j < nb; ++j) {
           const double* kr = dyn.Kbg + (size_t)fb[j] * n3;
           MPM_LAUNCH(k_dot<<<gb, 256, 0, s>>>(n3, kr, dx, dots + 7 * j, grid_red(c, 1, gb)));
