@@ -442,7 +442,7 @@ struct SubBox {
   double xi[3];  // centroid in the leaf's local coordinates
   double w;      // V_Kp / V_p
   double is;     // 1 / leaf size (a power of two, exact)
-  int K, s;
+  int K;
 };
 
 __device__ inline int warp_excl_scan(int v, int lane) {
@@ -456,71 +456,115 @@ __device__ inline int warp_excl_scan(int v, int lane) {
 
 constexpr int BW = 4;  // warps per block of the basis kernel
 
-constexpr int BH = 512;  // per-warp hash set of the basis kernel's node ids (at most MAXS distinct)
+constexpr int BH = 256;  // per-warp hash set of the basis kernel's node ids (at most MAXS distinct)
 
-__device__ inline unsigned basis_hash(int j) { return ((unsigned)j * 2654435761u) >> 23; }
+constexpr int BT = 16;  // sub-boxes whose corner values are tabulated at a time
+
+__device__ inline unsigned basis_hash(int j) { return ((unsigned)j * 2654435761u) >> 24; }
+
+// a positive normal float as a double, in integer instructions
+__device__ inline double widen(float f) {
+  unsigned b = __float_as_uint(f);
+  return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+
+// scratch of one warp of the basis kernel: the open boxes of the leaf walk,
+// then the node set, then the corner values
+union BasisTmp {
+  int open[MAXK][6];
+  struct {
+    int node[MAXE];  // node of an entry, then its rank
+    int hkey[BH];
+    int uid[MAXS], cnt[MAXS], next[MAXS];
+    unsigned char hslot[BH], rank[MAXS];
+  } set;
+  double val[BT * 8 * 4];
+};
 
 // Eq. (GIMP numerical), one warp per point (cell-sorted order):
-//  1. lane 0 cuts the domain into its leaf intersections (centre, volume);
+//  1. the domain is cut into its leaf intersections (centre, volume), the open
+//     boxes of a round one per lane;
 //  2. the (leaf corner, constraint entry) pairs are listed in a fixed order;
 //  3. the distinct independent nodes are found by a shared-memory hash set and
 //     ranked by id (support sorted by node id); the entries are grouped by
 //     node, each group keeping list order;
-//  4. lane k sums the contributions of support node k in list order, so the
-//     result does not depend on scheduling.
+//  4. every (sub-box, corner) value and gradient is computed once, by one lane,
+//     into shared memory; a lane then owns one of the four numbers of a support
+//     node and adds its weighted entries in list order, so the result does not
+//     depend on scheduling.
+// What bounds it: FP64 issue.  A warp's FP64 instruction takes its quarter of
+// the SM for 64 cycles whatever the number of active lanes, so each stage
+// spreads its FP64 work over the lanes: a bound of the domain, an axis of a
+// sub-box, a corner, a (node, number) pair.  A lane per node that recomputed its entries'
+// products took 20 instructions an entry, the longest group of 32 nodes long;
+// here an entry takes one fma, the longest group of 8 nodes long.  1.9 M points:
+// 26.1 ms so, 10.4 ms with the table and a lane per open box, sub-box and axis
+// of the domain, 8.8 ms with a lane per bound and per axis of a sub-box (some
+// 75 FP64 instructions a point, 7.5 ms of the FP64 pipe).
 __global__ void __launch_bounds__(32 * BW)
     k_basis(int P, Geo g, const double* __restrict__ px, const double* __restrict__ plp,
             const double* __restrict__ pE, const uint64_t* __restrict__ lkey,
             const int* __restrict__ llev, int nl, const int* __restrict__ corner,
             const int* __restrict__ cptr, const int* __restrict__ cidx,
             const double* __restrict__ cw, int* nsup, int* sidx, double* S, double* dS,
-            int* populated, unsigned long long* betaK, int* err) {
-  __shared__ SubBox sb[BW][MAXK];
-  __shared__ int e_node[BW][MAXE];
-  __shared__ short e_q[BW][MAXE];
-  __shared__ short e_ord[BW][MAXE];
-  __shared__ float e_w[BW][MAXE];  // constraint weights are products of 1/2 and 1/4: exact
-  __shared__ unsigned char e_rk[BW][MAXE];
-  __shared__ int sup[BW][MAXS];
-  __shared__ int hkey[BW][BH];
-  __shared__ unsigned char hslot[BW][BH];
-  __shared__ int uid[BW][MAXS];
-  __shared__ unsigned char urank[BW][MAXS];
-  __shared__ int ucnt[BW][MAXS], ubase[BW][MAXS], ustart[BW][MAXS];
-  __shared__ int nsub_s[BW], nu_s[BW];
+            int* active, int* populated, unsigned long long* betaK, int* err) {
+  __shared__ SubBox sb_s[BW][MAXK];
+  __shared__ __align__(16) BasisTmp tmp_s[BW];
+  __shared__ float e_w_s[BW][MAXE];  // constraint weights are sums of products of 1/2 and 1/4: exact
+  __shared__ unsigned short e_ord_s[BW][MAXE];
+  __shared__ unsigned short ustart_s[BW][MAXS + 1];
+  __shared__ unsigned char e_q_s[BW][MAXE];  // 8 sub-box + corner, below 8 MAXK = 216
+  __shared__ int nu_s[BW];
   int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int w = blockIdx.x * BW + wi;
   if (w >= P) return;
-  // 1. the domain cut into its leaf intersections.  Every cut face is a leaf
-  // face, an integer in grid units, so lane 0 walks the leaves in integer
-  // arithmetic: a bound is either the domain's own (code -1) or a face.
-  // The walk's FP64 work (volumes, centroids) then runs one sub-box per
-  // lane: a warp's FP64 instruction costs the same pipe time whatever the
-  // number of active lanes.
-  double Lo[3], Hi[3];
-  double Vp = domain_box(px + 3 * (size_t)w, plp + 3 * (size_t)w, g, Lo, Hi);
-  if (lane == 0) {
-    int n = 0;
-    if (!(Hi[0] > Lo[0]) || !(Hi[1] > Lo[1]) || !(Hi[2] > Lo[2])) {
-      atomicOr(err, EB_DOMAIN);
-      n = -1;
-    } else {
-      int fLo[3], fHi[3];
-      bool iHi[3];
-      for (int d = 0; d < 3; ++d) {
-        fLo[d] = (int)floor(Lo[d]);
-        fHi[d] = (int)floor(Hi[d]);
-        iHi[d] = Hi[d] == (double)fHi[d];
+  SubBox* sb = sb_s[wi];
+  BasisTmp& tmp = tmp_s[wi];
+  float* e_w = e_w_s[wi];
+  unsigned char* e_q = e_q_s[wi];
+  unsigned short *e_ord = e_ord_s[wi], *ustart = ustart_s[wi];
+  const unsigned all = 0xffffffffu;
+  // 1. the domain's bounds, one of the six per lane (lanes beyond the sixth
+  // repeat them), then its leaf intersections.  Every cut face is a leaf face,
+  // an integer in grid units, so the walk runs in integer arithmetic: a bound
+  // is either the domain's own (code -1) or a face.
+  double bd, Vp;  // lane 2 d + side: bound of axis d
+  int fLo[3], fHi[3];
+  unsigned iHi;   // bit 2 d + 1: the upper bound of axis d is an integer
+  {
+    int d = (lane % 6) >> 1, side = lane & 1;
+    double x = px[3 * (size_t)w + d], l = plp[3 * (size_t)w + d];
+    double v = snap_grid((side ? x + l : x - l) * g.scale), N = (double)g.N;
+    double len = __shfl_xor_sync(all, v, 1) - v;  // of use in the even lanes
+    bd = side ? (v > N ? N : v) : (v < 0.0 ? 0.0 : v);
+    double fl = floor(bd);
+    int f = (int)fl;
+    iHi = __ballot_sync(all, bd == fl);
+    bool empty = !(__shfl_xor_sync(all, bd, 1) > bd) && !side;
+    for (int i = 0; i < 3; ++i) {
+      fLo[i] = __shfl_sync(all, f, 2 * i);
+      fHi[i] = __shfl_sync(all, f, 2 * i + 1);
+    }
+    Vp = __shfl_sync(all, len, 0) * __shfl_sync(all, len, 2) * __shfl_sync(all, len, 4);
+    if (__any_sync(all, empty)) {
+      if (lane == 0) {
+        atomicOr(err, EB_DOMAIN);
+        nsup[w] = 0;
       }
-      int st[3 * MAXK + 8][6];
-      int ns = 1;
-      for (int d = 0; d < 6; ++d) st[0][d] = -1;
-      while (ns > 0) {
-        --ns;
-        int a[3], b[3], kh[3], e[3], q[3];
+      return;
+    }
+  }
+  int nsub = 0;
+  {
+    int a[3] = {-1, -1, -1}, b[3] = {-1, -1, -1};
+    int nopen = 1;
+    while (nopen > 0) {
+      // an open box yields a sub-box and up to three more open boxes
+      bool on = lane < nopen, gt[3] = {false, false, false};
+      int kh[3], e[3];
+      if (on) {
+        int q[3];
         for (int d = 0; d < 3; ++d) {
-          a[d] = st[ns][d];
-          b[d] = st[ns][3 + d];
           q[d] = a[d] < 0 ? fLo[d] : a[d];
           q[d] = q[d] > g.N - 1 ? g.N - 1 : (q[d] < 0 ? 0 : q[d]);
         }
@@ -528,7 +572,8 @@ __global__ void __launch_bounds__(32 * BW)
         int s = 1 << (g.D - llev[K]);
         int ka[3];
         demorton(lkey[K], ka);
-        bool gt[3];
+        SubBox& o = sb[nsub + lane];
+        int* cd = reinterpret_cast<int*>(o.xi);  // bound codes until step 1b
         for (int d = 0; d < 3; ++d) {
           kh[d] = ka[d] + s;
           if (b[d] < 0) {
@@ -536,89 +581,87 @@ __global__ void __launch_bounds__(32 * BW)
             // floor(Hi) < kh; Hi > kh iff floor(Hi) > kh, or equal and Hi
             // is not an integer
             e[d] = fHi[d] < kh[d] ? -1 : kh[d];
-            gt[d] = fHi[d] > kh[d] || (!iHi[d] && fHi[d] == kh[d]);
+            gt[d] = fHi[d] > kh[d] || (!((iHi >> (2 * d + 1)) & 1u) && fHi[d] == kh[d]);
           } else {
             e[d] = b[d] < kh[d] ? b[d] : kh[d];
             gt[d] = b[d] > kh[d];
           }
-        }
-        if (n >= MAXK || ns + 3 > 3 * MAXK + 8) {
-          atomicOr(err, EB_SUPPORT);
-          n = -1;
-          break;
-        }
-        SubBox& o = sb[wi][n++];
-        int* cd = reinterpret_cast<int*>(o.xi);  // bound codes until step 1b
-        for (int d = 0; d < 3; ++d) {
           cd[d] = a[d];
           cd[3 + d] = e[d];
         }
         o.K = K;
-        o.s = s;
-        if (gt[0]) {
-          int* r = st[ns++];
-          r[0] = kh[0]; r[1] = a[1]; r[2] = a[2]; r[3] = b[0]; r[4] = b[1]; r[5] = b[2];
-        }
-        if (gt[1]) {
-          int* r = st[ns++];
-          r[0] = a[0]; r[1] = kh[1]; r[2] = a[2]; r[3] = e[0]; r[4] = b[1]; r[5] = b[2];
-        }
-        if (gt[2]) {
-          int* r = st[ns++];
-          r[0] = a[0]; r[1] = a[1]; r[2] = kh[2]; r[3] = e[0]; r[4] = e[1]; r[5] = b[2];
-        }
       }
+      nsub += nopen;
+      int kids = (gt[0] ? 1 : 0) + (gt[1] ? 1 : 0) + (gt[2] ? 1 : 0);
+      int at = warp_excl_scan(kids, lane);
+      nopen = __shfl_sync(all, at + kids, 31);
+      if (nsub + nopen > MAXK) {  // every open box yields a sub-box
+        if (lane == 0) {
+          atomicOr(err, EB_SUPPORT);
+          nsup[w] = 0;
+        }
+        return;
+      }
+      __syncwarp();
+      if (gt[0]) {
+        int* r = tmp.open[at++];
+        r[0] = kh[0]; r[1] = a[1]; r[2] = a[2]; r[3] = b[0]; r[4] = b[1]; r[5] = b[2];
+      }
+      if (gt[1]) {
+        int* r = tmp.open[at++];
+        r[0] = a[0]; r[1] = kh[1]; r[2] = a[2]; r[3] = e[0]; r[4] = b[1]; r[5] = b[2];
+      }
+      if (gt[2]) {
+        int* r = tmp.open[at++];
+        r[0] = a[0]; r[1] = a[1]; r[2] = kh[2]; r[3] = e[0]; r[4] = e[1]; r[5] = b[2];
+      }
+      __syncwarp();
+      if (lane < nopen)
+        for (int d = 0; d < 3; ++d) {
+          a[d] = tmp.open[lane][d];
+          b[d] = tmp.open[lane][3 + d];
+        }
     }
-    nsub_s[wi] = n;
   }
-  __syncwarp();
-  // 1b. one lane per sub-box: volume fraction, centroid in leaf coordinates
-  if (lane < nsub_s[wi]) {
-    SubBox& o = sb[wi][lane];
+  // 1b. a sub-box and axis per lane, ten sub-boxes at a time: the sides'
+  // lengths and the centroid in leaf coordinates; then a sub-box per lane: its
+  // volume fraction
+  for (int s0 = 0; s0 < nsub; s0 += 10) {
+    int i = s0 + lane / 3, d = lane % 3;
+    bool on = lane < 30 && i < nsub;
+    SubBox& o = sb[on ? i : 0];
     const int* cd = reinterpret_cast<const int*>(o.xi);
-    int ca[3], ce[3];
-    for (int d = 0; d < 3; ++d) {
-      ca[d] = cd[d];
-      ce[d] = cd[3 + d];
-    }
-    int ka[3];
-    demorton(lkey[o.K], ka);
-    double vol = 1.0, xi[3];
+    double lo = __shfl_sync(all, bd, 2 * d), hi = __shfl_sync(all, bd, 2 * d + 1);
+    int ca = cd[d], ce = cd[3 + d], K = o.K, ka[3];
+    demorton(lkey[K], ka);
     // the leaf size is a power of two: multiplying by its exact reciprocal
-    // equals the division and keeps the FP64 pipe (slow on this part) free
-    double is = ldexp(1.0, llev[o.K] - g.D);
-    for (int d = 0; d < 3; ++d) {
-      double a = ca[d] < 0 ? Lo[d] : (double)ca[d];
-      double e = ce[d] < 0 ? Hi[d] : (double)ce[d];
-      vol *= e - a;
-      xi[d] = (0.5 * (a + e) - (double)ka[d]) * is;
+    // equals the division
+    double is = __hiloint2double((1023 + llev[K] - g.D) << 20, 0);
+    double a = ca < 0 ? lo : (double)ca, e = ce < 0 ? hi : (double)ce;
+    double xi = (0.5 * (a + e) - (double)(d == 0 ? ka[0] : (d == 1 ? ka[1] : ka[2]))) * is;
+    double len = e - a;
+    double v1 = __shfl_down_sync(all, len, 1), v2 = __shfl_down_sync(all, len, 2);
+    __syncwarp();
+    if (on) o.xi[d] = xi;
+    if (on && d == 0) {
+      o.is = is;
+      o.w = len * v1 * v2 / Vp;
+      populated[K] = 1;
+      atomicMax(betaK + K, (unsigned long long)__double_as_longlong(pE[w]));
     }
-    for (int d = 0; d < 3; ++d) o.xi[d] = xi[d];
-    o.is = is;
-    o.w = vol / Vp;
   }
   __syncwarp();
-  int nsub = nsub_s[wi];
-  if (nsub < 0) {
-    if (lane == 0) nsup[w] = 0;
-    return;
-  }
-  if (lane < nsub) {
-    int K = sb[wi][lane].K;
-    populated[K] = 1;
-    atomicMax(betaK + K, (unsigned long long)__double_as_longlong(pE[w]));
-  }
   // 2. list the (corner, constraint) entries in pair order
   int npair = 8 * nsub;
   int per = (npair + 31) / 32;
   int q0 = lane * per, q1 = min(q0 + per, npair);
   int len = 0;
   for (int q = q0; q < q1; ++q) {
-    int node = corner[8 * (size_t)sb[wi][q >> 3].K + (q & 7)];
+    int node = corner[8 * (size_t)sb[q >> 3].K + (q & 7)];
     len += cptr[node + 1] - cptr[node];
   }
   int off = warp_excl_scan(len, lane);
-  int total = __shfl_sync(0xffffffffu, off + len, 31);
+  int total = __shfl_sync(all, off + len, 31);
   if (total > MAXE) {
     if (lane == 0) {
       atomicOr(err, EB_SUPPORT);
@@ -628,28 +671,28 @@ __global__ void __launch_bounds__(32 * BW)
   }
   int pos = off;
   for (int q = q0; q < q1; ++q) {
-    int node = corner[8 * (size_t)sb[wi][q >> 3].K + (q & 7)];
+    int node = corner[8 * (size_t)sb[q >> 3].K + (q & 7)];
     for (int t = cptr[node]; t < cptr[node + 1]; ++t) {
-      e_node[wi][pos] = cidx[t];
-      e_q[wi][pos] = (short)q;
-      e_w[wi][pos] = (float)cw[t];
+      tmp.set.node[pos] = cidx[t];
+      e_q[pos] = (unsigned char)q;
+      e_w[pos] = (float)cw[t];
       ++pos;
     }
   }
-  __syncwarp();
   // 3. distinct nodes (hash set), ranked by id, entries grouped by node
-  for (int i = lane; i < BH; i += 32) hkey[wi][i] = -1;
+  for (int i = lane; i < BH; i += 32) tmp.set.hkey[i] = -1;
+  for (int u = lane; u < MAXS; u += 32) tmp.set.cnt[u] = 0;
   if (lane == 0) nu_s[wi] = 0;
   __syncwarp();
   for (int e = lane; e < total; e += 32) {
-    int j = e_node[wi][e];
+    int j = tmp.set.node[e];
     unsigned h = basis_hash(j);
     for (int probe = 0; probe < BH; ++probe) {
-      int prev = atomicCAS(&hkey[wi][h], -1, j);
+      int prev = atomicCAS(&tmp.set.hkey[h], -1, j);
       if (prev == -1) {
         int slot = atomicAdd(&nu_s[wi], 1);
-        if (slot < MAXS) uid[wi][slot] = j;
-        hslot[wi][h] = (unsigned char)min(slot, 255);
+        if (slot < MAXS) tmp.set.uid[slot] = j;
+        tmp.set.hslot[h] = (unsigned char)min(slot, 255);
         break;
       }
       if (prev == j) break;
@@ -666,29 +709,30 @@ __global__ void __launch_bounds__(32 * BW)
     return;
   }
   for (int u = lane; u < ns; u += 32) {
-    int j = uid[wi][u], r = 0;
-    for (int u2 = 0; u2 < ns; ++u2) r += uid[wi][u2] < j ? 1 : 0;
-    urank[wi][u] = (unsigned char)r;
-    sup[wi][r] = j;
+    int j = tmp.set.uid[u], r = 0;
+    for (int u2 = 0; u2 < ns; ++u2) r += tmp.set.uid[u2] < j ? 1 : 0;
+    tmp.set.rank[u] = (unsigned char)r;
+    sidx[(size_t)w * MAXS + r] = j;
+    active[j] = 1;
   }
-  for (int u = lane; u < MAXS; u += 32) ucnt[wi][u] = 0;
   __syncwarp();
   // rank of every entry (hash lookup) and the count per rank
   for (int e = lane; e < total; e += 32) {
-    int j = e_node[wi][e];
+    int j = tmp.set.node[e];
     unsigned h = basis_hash(j);
-    while (hkey[wi][h] != j) h = (h + 1) & (BH - 1);
-    int r = urank[wi][hslot[wi][h]];
-    e_rk[wi][e] = (unsigned char)r;
-    atomicAdd(&ucnt[wi][r], 1);
+    while (tmp.set.hkey[h] != j) h = (h + 1) & (BH - 1);
+    int r = tmp.set.rank[tmp.set.hslot[h]];
+    tmp.set.node[e] = r;
+    atomicAdd(&tmp.set.cnt[r], 1);
   }
   __syncwarp();
   {
-    int c0 = lane < ns ? ucnt[wi][lane] : 0, c1 = lane + 32 < ns ? ucnt[wi][lane + 32] : 0;
+    int c0 = lane < ns ? tmp.set.cnt[lane] : 0, c1 = lane + 32 < ns ? tmp.set.cnt[lane + 32] : 0;
     int x0 = warp_excl_scan(c0, lane), x1 = warp_excl_scan(c1, lane);
-    int t0 = __shfl_sync(0xffffffffu, x0 + c0, 31);
-    if (lane < ns) ubase[wi][lane] = ustart[wi][lane] = x0;
-    if (lane + 32 < ns) ubase[wi][lane + 32] = ustart[wi][lane + 32] = t0 + x1;
+    int t0 = __shfl_sync(all, x0 + c0, 31);
+    if (lane < ns) tmp.set.next[lane] = ustart[lane] = x0;
+    if (lane + 32 < ns) tmp.set.next[lane + 32] = ustart[lane + 32] = t0 + x1;
+    if (lane == 0) ustart[ns] = total;
   }
   __syncwarp();
   // stable grouping: chunks of 32 entries in list order, positions inside a
@@ -696,53 +740,50 @@ __global__ void __launch_bounds__(32 * BW)
   for (int c0 = 0; c0 < total; c0 += 32) {
     int e = c0 + lane;
     bool valid = e < total;
-    int r = valid ? (int)e_rk[wi][e] : -1 - lane;
-    unsigned grp = __match_any_sync(0xffffffffu, r);
+    int r = valid ? tmp.set.node[e] : -1 - lane;
+    unsigned grp = __match_any_sync(all, r);
     int before = __popc(grp & ((1u << lane) - 1u));
-    int pos = valid ? ubase[wi][r] + before : 0;
+    int at = valid ? tmp.set.next[r] + before : 0;
     __syncwarp();
     if (valid) {
-      e_ord[wi][pos] = (short)e;
-      if (before == 0) ubase[wi][r] += __popc(grp);
+      e_ord[at] = (unsigned short)e;
+      if (before == 0) tmp.set.next[r] += __popc(grp);
     }
     __syncwarp();
   }
   // 4. values and gradients of S_vp
-  for (int k = lane; k < ns; k += 32) {
-    int j = sup[wi][k];
-    double s0 = 0.0, g0 = 0.0, g1 = 0.0, g2 = 0.0;
-    for (int t = ustart[wi][k]; t < ustart[wi][k] + ucnt[wi][k]; ++t) {
-      int e = e_ord[wi][t];
-      int q = e_q[wi][e];
-      const SubBox& o = sb[wi][q >> 3];
-      int c = q & 7;
+  for (int b0 = 0; b0 < nsub; b0 += BT) {
+    int b1 = min(b0 + BT, nsub);
+    __syncwarp();
+    for (int i = lane; i < 8 * (b1 - b0); i += 32) {
+      const SubBox& o = sb[b0 + (i >> 3)];
+      int c = i & 7;
       double f0 = (c & 1) ? o.xi[0] : 1.0 - o.xi[0];
       double f1 = (c & 2) ? o.xi[1] : 1.0 - o.xi[1];
       double f2 = (c & 4) ? o.xi[2] : 1.0 - o.xi[2];
-      double inv = o.is;
-      double d0 = (c & 1) ? inv : -inv, d1 = (c & 2) ? inv : -inv, d2 = (c & 4) ? inv : -inv;
-      double ww = e_w[wi][e] * o.w;
-      s0 += ww * (f0 * f1 * f2);
-      g0 += ww * (d0 * f1 * f2);
-      g1 += ww * (f0 * d1 * f2);
-      g2 += ww * (f0 * f1 * d2);
+      double v = o.w, vs = v * o.is;
+      double f01 = f0 * f1, f02 = f0 * f2, f12 = f1 * f2;
+      double* t = tmp.val + 4 * i;
+      t[0] = v * (f01 * f2);
+      t[1] = ((c & 1) ? vs : -vs) * f12;
+      t[2] = ((c & 2) ? vs : -vs) * f02;
+      t[3] = ((c & 4) ? vs : -vs) * f01;
     }
-    size_t o = (size_t)w * MAXS + k;
-    sidx[o] = j;
-    S[o] = s0;
-    dS[3 * o] = g0 * g.scale;
-    dS[3 * o + 1] = g1 * g.scale;
-    dS[3 * o + 2] = g2 * g.scale;
+    __syncwarp();
+    int n = lane & 3;  // S and the three components of dS
+    for (int k = lane >> 2; k < ns; k += 8) {
+      size_t o = (size_t)w * MAXS + k;
+      double* out = n == 0 ? S + o : dS + 3 * o + (n - 1);
+      double a = b0 ? *out : 0.0;
+      for (int t = ustart[k]; t < ustart[k + 1]; ++t) {
+        int e = e_ord[t], q = (int)e_q[e] - 8 * b0;
+        if (nsub > BT && (q < 0 || q >= 8 * BT)) continue;
+        a = fma(widen(e_w[e]), tmp.val[4 * q + n], a);
+      }
+      *out = n > 0 && b1 == nsub ? a * g.scale : a;
+    }
   }
   if (lane == 0) nsup[w] = ns;
-}
-
-__global__ void k_mark_active(int P, const int* __restrict__ nsup, const int* __restrict__ sidx,
-                              int* active) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)P * MAXS) return;
-  int w = (int)(i / MAXS), k = (int)(i % MAXS);
-  if (k < nsup[w]) active[sidx[i]] = 1;
 }
 
 __global__ void k_number_dofs(int nn, const int* __restrict__ active, const int* __restrict__ pos,
@@ -1596,9 +1637,11 @@ void build_mesh(mpm_ctx* c, mpm_mesh* m, const mpm_domain& dom, const mpm_rigid&
   double* betaK = grow<double>(c, m->betaK, nl);
   MPM_CUDA(cudaMemsetAsync(pop, 0, sizeof(int) * nl, st));
   MPM_CUDA(cudaMemsetAsync(betaK, 0, sizeof(double) * nl, st));
+  int* active = grow<int>(c, c->tmp[0], nn);
+  MPM_CUDA(cudaMemsetAsync(active, 0, sizeof(int) * nn, st));
   MPM_LAUNCH_P(MPM_PROF_BASIS, k_basis<<<grid_for(P, BW), 32 * BW, 0, st>>>(P, g, ptr<double>(m->px), ptr<double>(m->plp),
                                                ptr<double>(m->pE), lkey, llev, nl, corner, cptr, cidx,
-                                               cw, nsup, sidx, S, dS, pop,
+                                               cw, nsup, sidx, S, dS, active, pop,
                                                (unsigned long long*)betaK, d_err));
   {
     int e = check_device_error(c, "GIMP basis");
@@ -1606,10 +1649,7 @@ void build_mesh(mpm_ctx* c, mpm_mesh* m, const mpm_domain& dom, const mpm_rigid&
   }
   // active nodes -> dofs (Morton order)
   {
-    int* active = grow<int>(c, c->tmp[0], nn);
     int* pos = grow<int>(c, c->tmp[1], nn);
-    MPM_CUDA(cudaMemsetAsync(active, 0, sizeof(int) * nn, st));
-    MPM_LAUNCH(k_mark_active<<<grid_for((long long)P * MAXS, 256), 256, 0, st>>>(P, nsup, sidx, active));
     cub_exclusive_sum_int(c, active, pos, nn);
     int nd = read_total(c, pos, active, nn);
     m->ndof = nd;
