@@ -144,7 +144,8 @@ __global__ void k_corner_ids(int n, const uint64_t* __restrict__ key, const int*
 // Sec. 3.1: n hangs when it lies on the boundary of a leaf without being one of
 // its vertices; K_n is the largest such leaf (ties: lowest Morton key)
 __global__ void k_hang(int nn, const uint64_t* __restrict__ nkey, const uint64_t* __restrict__ lkey,
-                       const int* __restrict__ llev, int nl, Geo g, int* hang, int* owner) {
+                       const int* __restrict__ llev, int nl, Geo g, int* hang, int* owner,
+                       int* nhang) {
   int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= nn) return;
   int X[3];
@@ -172,6 +173,8 @@ __global__ void k_hang(int nn, const uint64_t* __restrict__ nkey, const uint64_t
   }
   hang[n] = best >= 0 ? 1 : 0;
   owner[n] = best;
+  unsigned on = __activemask(), hs = __ballot_sync(on, best >= 0);
+  if (hs && (threadIdx.x & 31) == __ffs(on) - 1) atomicAdd(nhang, __popc(hs));
 }
 
 struct NodeView {
@@ -798,14 +801,6 @@ __global__ void k_number_dofs(int nn, const int* __restrict__ active, const int*
   }
 }
 
-__global__ void k_sidx_to_dof(int P, const int* __restrict__ nsup, const int* __restrict__ node_dof,
-                              int* sidx) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)P * MAXS) return;
-  int w = (int)(i / MAXS), k = (int)(i % MAXS);
-  if (k < nsup[w]) sidx[i] = node_dof[sidx[i]];
-}
-
 struct Planes {
   int n;
   int axis[8];
@@ -1039,23 +1034,44 @@ __global__ void k_ghost_rows(int nd, int P, const long long* __restrict__ sptr,
 
 // ------------------------------------------------------------------ block pattern
 
-// sum over the points of (support size)^2: the (source, column) pairs of the
-// tangent gather, for the benchmark's operation counts (integer, exact)
-__global__ void k_support_pairs(int P, const int* __restrict__ nsup, unsigned long long* out) {
-  int w = blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned long long v = w < P ? (unsigned long long)nsup[w] * (unsigned long long)nsup[w] : 0ULL;
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0 && v) atomicAdd(out, v);
-}
+// Counts of a mesh kept on the device until the build's last synchronisation:
+// the sum over the points of (support size)^2, i.e. the (source, column) pairs
+// of the tangent gather, for the benchmark's operation counts (integer, exact);
+// the largest support, the longest row and the number of hanging nodes.
+struct MeshCounts {
+  unsigned long long npair;
+  int maxs, maxrow, nhang;
+};
 
-// source keys: row dof << 32 | source << 6 | local index (points, then ghost faces)
-__global__ void k_src_keys_points(int P, const int* __restrict__ nsup, const int* __restrict__ sidx,
-                                  const int* __restrict__ off, uint64_t* keys) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)P * MAXS) return;
-  int w = (int)(i / MAXS), k = (int)(i % MAXS);
-  if (k >= nsup[w]) return;
-  keys[off[w] + k] = ((uint64_t)(uint32_t)sidx[i] << 32) | ((uint64_t)(uint32_t)w << 6) | (uint32_t)k;
+// one warp per point: its support from node ids to dofs, and the point's
+// source keys: row dof << 32 | source << 6 | local index (points, then ghost
+// faces).  With these bits the keys of the points, and of the faces after them,
+// are listed in ascending order of their lower 32 bits: a stable sort by the
+// row alone (3 passes of 8 bits at 260 k rows instead of 8) orders them fully.
+__global__ void k_point_sources(int P, const int* __restrict__ nsup, const int* __restrict__ node_dof,
+                                const int* __restrict__ off, int* sidx, uint64_t* keys,
+                                MeshCounts* mc) {
+  __shared__ int ns[32];
+  int wi = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  int w = blockIdx.x * nw + wi;
+  int n = w < P ? nsup[w] : 0;
+  int o = n ? off[w] : 0;
+  for (int k = lane; k < n; k += 32) {
+    size_t i = (size_t)w * MAXS + k;
+    int r = node_dof[sidx[i]];
+    sidx[i] = r;
+    keys[o + k] = ((uint64_t)(uint32_t)r << 32) | ((uint64_t)(uint32_t)w << 6) | (uint32_t)k;
+  }
+  if (lane == 0) ns[wi] = n;
+  __syncthreads();
+  if (wi == 0) {
+    n = lane < nw ? ns[lane] : 0;
+    int mx = __reduce_max_sync(0xffffffffu, n), sq = warp_sum_int(n * n);
+    if (lane == 0 && sq) {
+      atomicAdd(&mc->npair, (unsigned long long)sq);
+      if (mx > *(volatile int*)&mc->maxs) atomicMax(&mc->maxs, mx);
+    }
+  }
 }
 
 __global__ void k_src_keys_faces(int nf, int P, const int* __restrict__ gn, const int* __restrict__ gdof,
@@ -1077,77 +1093,182 @@ __global__ void k_src_ptr(long long n, const uint64_t* __restrict__ keys, int nd
   if (i == n - 1 || (uint32_t)(keys[i + 1] >> 32) != r) ptr[r + 1] = i + 1;
 }
 
-__device__ inline int hash_insert(int* h, int key) {
-  unsigned s = ((unsigned)key * 2654435761u) & (HASH - 1);
-  for (int probe = 0; probe < HASH; ++probe) {
-    int prev = atomicCAS(h + s, -1, key);
-    if (prev == -1) return 1;
-    if (prev == key) return 0;
-    s = (s + 1) & (HASH - 1);
+// Block pattern: the columns of row r are the union of the supports of every
+// source (point or ghost face) touching r.  One warp per row collects them in
+// a hash set in shared memory and ranks them.  What bounds it is the latency
+// of the chain key -> support -> insertion over some 200 sources a row, and the
+// insertions' shared-memory traffic.  So a warp takes 32 keys and support sizes
+// at once, 8 supports in flight, and reads a slot before it tries to claim it
+// (some 40 of 41 insertions find their column there).  Rows of at most PSHORT
+// columns (125 where the leaf size does not change) use a set of 512 slots
+// (3 KB a warp, 44 warps to the SM; 2048 slots leave room for 18) and leave
+// their sorted columns in a staging row, which a copy takes to its place once
+// the row lengths are known; the others are collected again then, by the kernel
+// with the large set.  Two traversals, source by source, of a 2048-slot set took
+// 2 x 5.63 ms for 260 k rows and 51 M sources; now 2.10 ms and the copy 0.08 ms.
+constexpr int PSHORT = 256;            // longest row of the small set, and a staging row
+constexpr int PHASH = 2 * PSHORT;      // its slots
+constexpr int PPROBE = 64;             // its longest probe sequence; a row beyond it is a long one
+constexpr int PW = 4;                  // warps per block of the pattern kernels
+constexpr int PLW = 2;                 // the same of the long rows' kernel
+
+struct PatternSrc {
+  int P;
+  const long long* sptr;
+  const uint64_t* keys;
+  const int *nsup, *sidx, *gn, *gdof;
+};
+
+// 1: added, 0: there already, -1: no slot within `probes`
+template <int H>
+__device__ inline int set_insert(volatile int* h, int key, int probes) {
+  unsigned s = ((unsigned)key * 2654435761u) >> 16 & (H - 1);
+  for (int i = 0; i < probes; ++i) {
+    int v = h[s];
+    if (v == -1) v = atomicCAS((int*)h + s, -1, key);
+    if (v == -1) return 1;
+    if (v == key) return 0;
+    s = (s + 1) & (H - 1);
   }
   return -1;
 }
 
-constexpr int PW = 2;  // warps per block of the pattern kernel
+// the set of row r's columns in h[H]; their number, or -1 when more than `limit`
+// or out of slots
+template <int H>
+__device__ int pattern_collect(const PatternSrc& p, int r, int* h, int limit, int probes, int lane) {
+  const unsigned all = 0xffffffffu;
+  for (int i = lane; i < H; i += 32) h[i] = -1;
+  __syncwarp();
+  int cnt = 0;
+  bool bad = false;
+  long long s1 = p.sptr[r + 1];
+  for (long long s0 = p.sptr[r]; s0 < s1; s0 += 32) {
+    int m = (int)min(32LL, s1 - s0), n = 0;
+    long long base = 0;  // of the lane's source, in sidx or (from P on) gdof
+    if (lane < m) {
+      int sid = (int)((uint32_t)p.keys[s0 + lane] >> 6);
+      n = sid < p.P ? p.nsup[sid] : p.gn[sid - p.P];
+      base = sid < p.P ? (long long)sid * MAXS : -1 - (long long)(sid - p.P) * MAXG;
+    }
+    for (int t = 0; t < m; t += 8) {
+      int v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        int nu = __shfl_sync(all, n, (t + u) & 31);  // 0 past the last source
+        long long b = __shfl_sync(all, base, (t + u) & 31);
+        const int* q = b >= 0 ? p.sidx + b : p.gdof + (-1 - b);
+        v[u] = lane < nu ? q[lane] : -1;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (v[u] < 0) continue;
+        int rv = set_insert<H>(h, v[u], probes);
+        cnt += rv > 0;
+        bad |= rv < 0;
+      }
+    }
+    // supports of more than 32 nodes
+    for (unsigned more = __ballot_sync(all, n > 32); more; more &= more - 1) {
+      int t = __ffs(more) - 1;
+      int nu = __shfl_sync(all, n, t);
+      long long b = __shfl_sync(all, base, t);
+      const int* q = b >= 0 ? p.sidx + b : p.gdof + (-1 - b);
+      for (int l = lane + 32; l < nu; l += 32) {
+        int rv = set_insert<H>(h, q[l], probes);
+        cnt += rv > 0;
+        bad |= rv < 0;
+      }
+      __syncwarp();
+    }
+    if (__any_sync(all, bad) || __reduce_add_sync(all, cnt) > limit) return -1;
+  }
+  __syncwarp();
+  return warp_sum_int(cnt);
+}
 
-// one warp per row: the columns of row r are the union of the supports of
-// every source (point or ghost face) touching r; count, then write sorted
+// the set's cnt members in ascending order to out, by way of the list lst (its
+// length a multiple of 4, 16-byte aligned)
+template <int H>
+__device__ void pattern_sorted(const int* h, int cnt, int* lst, int* out, int lane) {
+  int at = 0;
+  for (int i = lane; i < H; i += 32) {
+    int v = h[i];
+    unsigned b = __ballot_sync(0xffffffffu, v >= 0);
+    if (v >= 0) lst[at + __popc(b & ((1u << lane) - 1u))] = v;
+    at += __popc(b);
+  }
+  if (lane < ((4 - (cnt & 3)) & 3)) lst[cnt + lane] = 0x7fffffff;
+  __syncwarp();
+  for (int e0 = 0; e0 < cnt; e0 += 128) {
+    int v[4], rk[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      int e = e0 + 32 * j + lane;
+      v[j] = e < cnt ? lst[e] : 0;
+      rk[j] = 0;
+    }
+    for (int t = 0; t < cnt; t += 4) {
+      int4 x = *reinterpret_cast<const int4*>(lst + t);
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        rk[j] += (x.x < v[j]) + (x.y < v[j]) + (x.z < v[j]) + (x.w < v[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (e0 + 32 * j + lane < cnt) out[rk[j]] = v[j];
+  }
+}
+
+// lengths of the rows and the sorted columns of the short ones in their staging
+// rows; -1 for a long row
 __global__ void __launch_bounds__(32 * PW)
-    k_pattern_rows(int ndof, int P, int mode, const long long* __restrict__ sptr,
-                   const uint64_t* __restrict__ keys, const int* __restrict__ nsup,
-                   const int* __restrict__ sidx, const int* __restrict__ gn,
-                   const int* __restrict__ gdof, int* rowcnt, const int* __restrict__ row_ptr,
-                   int* col, int* err) {
-  __shared__ int h[PW][HASH];
-  __shared__ int lst[PW][MAXROW];
+    k_pattern_rows(int ndof, PatternSrc p, int* rowcnt, int* stage) {
+  __shared__ int h[PW][PHASH];
+  __shared__ __align__(16) int lst[PW][PSHORT];
   int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int r = blockIdx.x * PW + wi;
   if (r >= ndof) return;
-  for (int i = lane; i < HASH; i += 32) h[wi][i] = -1;
-  __syncwarp();
-  int cnt = 0, bad = 0;
-  for (long long i = sptr[r]; i < sptr[r + 1]; ++i) {
-    uint32_t sid = (uint32_t)keys[i] >> 6;
-    int n;
-    const int* base;
-    if ((int)sid < P) {
-      n = nsup[sid];
-      base = sidx + (size_t)sid * MAXS;
-    } else {
-      n = gn[sid - P];
-      base = gdof + (size_t)(sid - P) * MAXG;
+  int cnt = pattern_collect<PHASH>(p, r, h[wi], PSHORT, PPROBE, lane);
+  if (lane == 0) rowcnt[r] = cnt;
+  if (cnt > 0) pattern_sorted<PHASH>(h[wi], cnt, lst[wi], stage + (size_t)r * PSHORT, lane);
+}
+
+// the long rows.  row_ptr null: their lengths (columns to the staging row where
+// they fit it after all); else the columns of those that did not fit it
+__global__ void __launch_bounds__(32 * PLW)
+    k_pattern_long(int ndof, PatternSrc p, int* rowcnt, int* stage, const int* __restrict__ row_ptr,
+                   int* col, int* err) {
+  __shared__ int h[PLW][HASH];
+  __shared__ __align__(16) int lst[PLW][MAXROW];
+  int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int r0 = 32 * (blockIdx.x * PLW + wi); r0 < ndof; r0 += 32 * PLW * gridDim.x) {
+    int n = r0 + lane < ndof ? rowcnt[r0 + lane] : 0;
+    unsigned todo = __ballot_sync(0xffffffffu, row_ptr ? n > PSHORT : n < 0);
+    for (; todo; todo &= todo - 1) {
+      int r = r0 + __ffs(todo) - 1;
+      int cnt = pattern_collect<HASH>(p, r, h[wi], MAXROW, HASH, lane);
+      if (!row_ptr && lane == 0) {
+        rowcnt[r] = max(cnt, 0);
+        if (cnt < 0) atomicOr(err, EB_ROW);
+      }
+      if (row_ptr && cnt > 0)
+        pattern_sorted<HASH>(h[wi], cnt, lst[wi], col + row_ptr[r], lane);
+      else if (!row_ptr && cnt > 0 && cnt <= PSHORT)
+        pattern_sorted<HASH>(h[wi], cnt, lst[wi], stage + (size_t)r * PSHORT, lane);
+      __syncwarp();
     }
-    for (int l = lane; l < n; l += 32) {
-      int rv = hash_insert(h[wi], base[l]);
-      if (rv > 0) ++cnt;
-      if (rv < 0) bad = 1;
-    }
   }
-  cnt = warp_sum_int(cnt);
-  bad = __any_sync(0xffffffffu, bad);
-  if (cnt > MAXROW || bad) {
-    if (lane == 0) atomicOr(err, EB_ROW);
-    if (mode == 0 && lane == 0) rowcnt[r] = 0;
-    return;
-  }
-  if (mode == 0) {
-    if (lane == 0) rowcnt[r] = cnt;
-    return;
-  }
-  __syncwarp();
-  // compact the occupied slots, then rank
-  int mine = 0;
-  for (int i = lane * (HASH / 32); i < (lane + 1) * (HASH / 32); ++i) mine += h[wi][i] >= 0;
-  int off = warp_excl_scan(mine, lane);
-  for (int i = lane * (HASH / 32); i < (lane + 1) * (HASH / 32); ++i)
-    if (h[wi][i] >= 0) lst[wi][off++] = h[wi][i];
-  __syncwarp();
-  int b = row_ptr[r];
-  for (int e = lane; e < cnt; e += 32) {
-    int v = lst[wi][e], rk = 0;
-    for (int e2 = 0; e2 < cnt; ++e2) rk += lst[wi][e2] < v;
-    col[b + rk] = v;
-  }
+}
+
+// staging rows to their place, one warp per row
+__global__ void k_pattern_write(int ndof, const int* __restrict__ row_ptr, const int* __restrict__ stage,
+                                int* col) {
+  int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (r >= ndof) return;
+  int b = row_ptr[r], n = row_ptr[r + 1] - b;
+  if (n > PSHORT) return;
+  for (int i = lane; i < n; i += 32) col[b + i] = stage[(size_t)r * PSHORT + i];
 }
 
 // ------------------------------------------------------------------ gravity, contact candidates
@@ -1366,16 +1487,21 @@ __global__ void k_slice_order(int nd, int npad, const int* __restrict__ rp, int*
   row[w0 + rank] = r;
 }
 
-// width of each slice of 32 storage rows: longest row, rounded up to 4 blocks
-__global__ void k_slice_width(int nd, int ns, const int* __restrict__ rp, const int* __restrict__ row, int* w) {
+// width of each slice of 32 storage rows: longest row, rounded up to 4 blocks;
+// the longest row of all
+__global__ void k_slice_width(int nd, int ns, const int* __restrict__ rp, const int* __restrict__ row, int* w,
+                              int* maxrow) {
   int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= ns) return;
   int m = 0;
-  for (int sr = 32 * s; sr < 32 * s + 32; ++sr) {
-    int r = row[sr];
-    if (r < nd) m = max(m, rp[r + 1] - rp[r]);
+  if (s < ns) {
+    for (int sr = 32 * s; sr < 32 * s + 32; ++sr) {
+      int r = row[sr];
+      if (r < nd) m = max(m, rp[r + 1] - rp[r]);
+    }
+    w[s] = (m + 3) & ~3;
   }
-  w[s] = (m + 3) & ~3;
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(maxrow, m);
 }
 
 __global__ void k_slice_slots(int ns, const int* __restrict__ w, int* slots) {
@@ -1450,12 +1576,6 @@ void tree_balance(mpm_ctx* c, mpm_mesh* m) {
   throw CudaError(MPM_ERR_BALANCE, "octree balance did not settle");
 }
 
-int bits_for(long long v) {
-  int b = 1;
-  while ((1LL << b) <= v) ++b;
-  return b;
-}
-
 }  // namespace
 
 // ------------------------------------------------------------------ the build
@@ -1508,6 +1628,8 @@ void build_mesh(mpm_ctx* c, mpm_mesh* m, const mpm_domain& dom, const mpm_rigid&
   int* d_err = c->d_err;
   if (body.kind == 3) tri_setup(c, m, body);
   const Body bv = body_view(m, body);
+  MeshCounts* mc = (MeshCounts*)(c->d_red + 50);
+  MPM_CUDA(cudaMemsetAsync(mc, 0, sizeof(MeshCounts), st));
 
   // ---- a1: uniform tree at depth_min, then Sec. 5 refinement + balance
   {
@@ -1582,7 +1704,7 @@ void build_mesh(mpm_ctx* c, mpm_mesh* m, const mpm_domain& dom, const mpm_rigid&
     uint64_t* ck = grow<uint64_t>(c, c->tmp[3], 8 * (size_t)nl);
     uint64_t* alt = grow<uint64_t>(c, c->tmp[4], 8 * (size_t)nl);
     MPM_LAUNCH(k_corner_keys<<<grid_for(nl, 256), 256, 0, st>>>(nl, lkey, llev, g.D, ck));
-    cub_sort_u64(c, ck, alt, 8 * nl, 3 * (g.D + 1));
+    ck = cub_sort_u64(c, ck, alt, 8 * nl, 0, 3 * (g.D + 1));
     uint64_t* nkey = grow<uint64_t>(c, m->node_key, 8 * (size_t)nl);
     int nn = cub_unique_u64(c, ck, nkey, 8 * nl);
     m->nnode = nn;
@@ -1590,7 +1712,7 @@ void build_mesh(mpm_ctx* c, mpm_mesh* m, const mpm_domain& dom, const mpm_rigid&
     MPM_LAUNCH(k_corner_ids<<<grid_for(nl, 256), 256, 0, st>>>(nl, lkey, llev, g.D, nkey, nn, corner));
     int* hang = grow<int>(c, m->hang, nn);
     int* owner = grow<int>(c, m->owner, nn);
-    MPM_LAUNCH(k_hang<<<grid_for(nn, 256), 256, 0, st>>>(nn, nkey, lkey, llev, nl, g, hang, owner));
+    MPM_LAUNCH(k_hang<<<grid_for(nn, 256), 256, 0, st>>>(nn, nkey, lkey, llev, nl, g, hang, owner, &mc->nhang));
     NodeView v{nkey, lkey, llev, corner, hang, owner, g.D};
     int* cnt = grow<int>(c, c->tmp[0], nn + 1);
     int* cptr = grow<int>(c, m->cptr, nn + 1);
@@ -1656,7 +1778,6 @@ void build_mesh(mpm_ctx* c, mpm_mesh* m, const mpm_domain& dom, const mpm_rigid&
     int* node_dof = grow<int>(c, m->node_dof, nn);
     int* dof_node = grow<int>(c, m->dof_node, nd);
     MPM_LAUNCH(k_number_dofs<<<grid_for(nn, 256), 256, 0, st>>>(nn, active, pos, node_dof, dof_node));
-    MPM_LAUNCH(k_sidx_to_dof<<<grid_for((long long)P * MAXS, 256), 256, 0, st>>>(P, nsup, node_dof, sidx));
     Planes pl{};
     pl.n = dom.nbc;
     for (int b = 0; b < dom.nbc; ++b) {
@@ -1700,30 +1821,34 @@ void build_mesh(mpm_ctx* c, mpm_mesh* m, const mpm_domain& dom, const mpm_rigid&
     long long total = npt + (long long)nf * MAXG;
     uint64_t* keys = grow<uint64_t>(c, m->src_key, total);
     uint64_t* alt = grow<uint64_t>(c, c->tmp[3], total);
-    MPM_LAUNCH(k_src_keys_points<<<grid_for((long long)P * MAXS, 256), 256, 0, st>>>(P, nsup, sidx, off, keys));
+    // rows below 2^bits - 1: the unused face slots' row of ones sorts last.  An
+    // odd number of passes starts in the scratch buffer, to end in the keys
+    int bits = bits_for(nd);
+    bool odd = ((bits + 7) / 8) & 1;
+    uint64_t *first = odd ? alt : keys, *second = odd ? keys : alt;
+    MPM_LAUNCH(k_point_sources<<<grid_for(P, 8), 256, 0, st>>>(P, nsup, node_dof, off, sidx, first, mc));
     if (nf) {
       // unused face slots keep an out-of-range row so that they sort last
-      MPM_CUDA(cudaMemsetAsync(keys + npt, 0xff, sizeof(uint64_t) * (size_t)nf * MAXG, st));
+      MPM_CUDA(cudaMemsetAsync(first + npt, 0xff, sizeof(uint64_t) * (size_t)nf * MAXG, st));
       MPM_LAUNCH(k_src_keys_faces<<<grid_for((long long)nf * MAXG, 256), 256, 0, st>>>(
-          nf, P, ptr<int>(m->gn), ptr<int>(m->gdof), npt, keys));
+          nf, P, ptr<int>(m->gn), ptr<int>(m->gdof), npt, first));
     }
-    cub_sort_u64(c, keys, alt, (int)total, 64);
+    uint64_t* sorted = cub_sort_u64(c, first, second, (int)total, 32, 32 + bits);
+    if (sorted != keys)
+      MPM_CUDA(cudaMemcpyAsync(keys, sorted, sizeof(uint64_t) * (size_t)total, cudaMemcpyDeviceToDevice, st));
     long long* sptr = grow<long long>(c, m->src_ptr, nd + 1);
     MPM_CUDA(cudaMemsetAsync(sptr, 0, sizeof(long long) * (nd + 1), st));
     MPM_LAUNCH(k_src_ptr<<<grid_for(total, 256), 256, 0, st>>>(total, keys, nd, sptr));
     m->nsrc = total;
-    {
-      unsigned long long* np2 = (unsigned long long*)(c->d_red + 50);
-      MPM_CUDA(cudaMemsetAsync(np2, 0, sizeof(unsigned long long), st));
-      MPM_LAUNCH(k_support_pairs<<<grid_for(P, 256), 256, 0, st>>>(P, nsup, np2));
-      MPM_CUDA(cudaMemcpyAsync(&m->npair, np2, sizeof(long long), cudaMemcpyDeviceToHost, st));
-    }
     int* rowcnt = grow<int>(c, m->rowcnt, nd + 1);
     int* rp = grow<int>(c, m->row_ptr, nd + 1);
     MPM_CUDA(cudaMemsetAsync(rowcnt + nd, 0, sizeof(int), st));
-    MPM_LAUNCH_P(MPM_PROF_PATTERN, k_pattern_rows<<<grid_for(nd, PW), 32 * PW, 0, st>>>(nd, P, 0, sptr, keys, nsup, sidx,
-                                                         ptr<int>(m->gn), ptr<int>(m->gdof), rowcnt,
-                                                         nullptr, nullptr, d_err));
+    PatternSrc ps{P, sptr, keys, nsup, sidx, ptr<int>(m->gn), ptr<int>(m->gdof)};
+    int* stage = grow<int>(c, c->tmp[3], (size_t)nd * PSHORT);  // the sort's scratch is free again
+    int lblocks = std::min(grid_for(nd, 32 * PLW), 152 * 9);
+    MPM_LAUNCH_P(MPM_PROF_PATTERN, k_pattern_rows<<<grid_for(nd, PW), 32 * PW, 0, st>>>(nd, ps, rowcnt, stage));
+    MPM_LAUNCH_P(MPM_PROF_PATTERN, k_pattern_long<<<lblocks, 32 * PLW, 0, st>>>(nd, ps, rowcnt, stage, nullptr,
+                                                                               nullptr, d_err));
     cub_exclusive_sum_int(c, rowcnt, rp, nd + 1);
     int nnzb = read_total(c, rp, rowcnt, nd + 1);
     {
@@ -1732,16 +1857,9 @@ void build_mesh(mpm_ctx* c, mpm_mesh* m, const mpm_domain& dom, const mpm_rigid&
     }
     m->nnzb = nnzb;
     int* col = grow<int>(c, m->col, nnzb);
-    MPM_LAUNCH_P(MPM_PROF_PATTERN, k_pattern_rows<<<grid_for(nd, PW), 32 * PW, 0, st>>>(nd, P, 1, sptr, keys, nsup, sidx,
-                                                         ptr<int>(m->gn), ptr<int>(m->gdof), rowcnt,
-                                                         rp, col, d_err));
-    // longest row (for the solver's launch shapes)
-    std::vector<int> h(nd + 1);
-    MPM_CUDA(cudaMemcpyAsync(h.data(), rp, sizeof(int) * (nd + 1), cudaMemcpyDeviceToHost, st));
-    MPM_CUDA(cudaStreamSynchronize(st));
-    int mr = 0;
-    for (int r = 0; r < nd; ++r) mr = std::max(mr, h[r + 1] - h[r]);
-    m->maxrow = mr;
+    MPM_LAUNCH_P(MPM_PROF_PATTERN, k_pattern_write<<<grid_for(nd, 8), 256, 0, st>>>(nd, rp, stage, col));
+    MPM_LAUNCH_P(MPM_PROF_PATTERN, k_pattern_long<<<lblocks, 32 * PLW, 0, st>>>(nd, ps, rowcnt, stage, rp, col,
+                                                                               d_err));
     // sliced storage of the stiffness
     int ns = (nd + 31) / 32;
     m->nslice = ns;
@@ -1751,7 +1869,7 @@ void build_mesh(mpm_ctx* c, mpm_mesh* m, const mpm_domain& dom, const mpm_rigid&
     int* srow = grow<int>(c, m->srow, 32 * (size_t)ns);
     int* rpos = grow<int>(c, m->spos, 32 * (size_t)ns);
     MPM_LAUNCH(k_slice_order<<<(32 * ns + SLICE_WINDOW - 1) / SLICE_WINDOW, SLICE_WINDOW, 0, st>>>(nd, 32 * ns, rp, srow, rpos));
-    MPM_LAUNCH(k_slice_width<<<grid_for(ns, 256), 256, 0, st>>>(nd, ns, rp, srow, sw));
+    MPM_LAUNCH(k_slice_width<<<grid_for(ns, 256), 256, 0, st>>>(nd, ns, rp, srow, sw, &mc->maxrow));
     MPM_LAUNCH(k_slice_slots<<<grid_for(ns, 256), 256, 0, st>>>(ns, sw, slots));
     MPM_CUDA(cudaMemsetAsync(slots + ns, 0, sizeof(int), st));
     cub_exclusive_sum_int(c, slots, spos, ns + 1);
@@ -1823,7 +1941,8 @@ void build_mesh(mpm_ctx* c, mpm_mesh* m, const mpm_domain& dom, const mpm_rigid&
       uint64_t* keys = grow<uint64_t>(c, c->tmp[4], nk);
       uint64_t* alt = grow<uint64_t>(c, c->tmp[5], nk);
       MPM_LAUNCH(k_ct_keys<<<grid_for(nk, 256), 256, 0, st>>>(8 * nc, ptr<int>(m->cb_n), ptr<int>(m->cb_idx), keys));
-      cub_sort_u64(c, keys, alt, (int)nk, 64);
+      // listed in ascending order of the lower 32 bits: sorted by the row alone
+      keys = cub_sort_u64(c, keys, alt, (int)nk, 32, 32 + bits_for(nd));
       int* cflag = grow<int>(c, c->tmp[6], nk + 1);
       int* cpos = grow<int>(c, c->tmp[7], nk + 1);
       MPM_LAUNCH(k_ct_flag<<<grid_for(nk, 256), 256, 0, st>>>(nk, keys, cflag));
@@ -1837,23 +1956,14 @@ void build_mesh(mpm_ctx* c, mpm_mesh* m, const mpm_domain& dom, const mpm_rigid&
   }
 
   // FP32 copies of the basis for the mixed-precision path are made on demand
-  // by the assembly; count the largest support
-  {
-    std::vector<int> h(P);
-    MPM_CUDA(cudaMemcpyAsync(h.data(), nsup, sizeof(int) * P, cudaMemcpyDeviceToHost, st));
-    MPM_CUDA(cudaStreamSynchronize(st));
-    int mx = 0;
-    for (int v : h) mx = std::max(mx, v);
-    m->maxs = mx;
-  }
-  int nh = 0;
-  {
-    std::vector<int> h(nn);
-    MPM_CUDA(cudaMemcpyAsync(h.data(), ptr<int>(m->hang), sizeof(int) * nn, cudaMemcpyDeviceToHost, st));
-    MPM_CUDA(cudaStreamSynchronize(st));
-    for (int v : h) nh += v;
-  }
-  m->nhang = nh;
+  // by the assembly
+  MeshCounts* h = (MeshCounts*)c->h_red;
+  MPM_CUDA(cudaMemcpyAsync(h, mc, sizeof(MeshCounts), cudaMemcpyDeviceToHost, st));
+  MPM_CUDA(cudaStreamSynchronize(st));
+  m->npair = (long long)h->npair;
+  m->maxs = h->maxs;
+  m->maxrow = h->maxrow;
+  m->nhang = h->nhang;
   m->built = 1;
 }
 

@@ -13,15 +13,16 @@ void cub_exclusive_sum_int(mpm_ctx* c, const int* in, int* out, int n) {
   MPM_CUDA(cub::DeviceScan::ExclusiveSum(tmp, bytes, in, out, n, c->stream));
 }
 
-void cub_sort_u64(mpm_ctx* c, uint64_t* keys, uint64_t* alt, int n, int end_bit) {
+// stable sort by the bits [begin_bit, end_bit) of the keys in `keys`, each pass
+// of 8 bits moving them between `keys` and `alt`; returns the one that holds
+// the result
+uint64_t* cub_sort_u64(mpm_ctx* c, uint64_t* keys, uint64_t* alt, int n, int begin_bit, int end_bit) {
   cub::DoubleBuffer<uint64_t> db(keys, alt);
   size_t bytes = 0;
-  MPM_CUDA(cub::DeviceRadixSort::SortKeys(nullptr, bytes, db, n, 0, end_bit, c->stream));
+  MPM_CUDA(cub::DeviceRadixSort::SortKeys(nullptr, bytes, db, n, begin_bit, end_bit, c->stream));
   void* tmp = grow_bytes(c, c->cub_tmp, bytes);
-  MPM_CUDA(cub::DeviceRadixSort::SortKeys(tmp, bytes, db, n, 0, end_bit, c->stream));
-  if (db.Current() != keys)
-    MPM_CUDA(cudaMemcpyAsync(keys, db.Current(), sizeof(uint64_t) * (size_t)n,
-                             cudaMemcpyDeviceToDevice, c->stream));
+  MPM_CUDA(cub::DeviceRadixSort::SortKeys(tmp, bytes, db, n, begin_bit, end_bit, c->stream));
+  return db.Current();
 }
 
 void cub_sort_pairs_int(mpm_ctx* c, const int* kin, int* kout, const int* vin, int* vout, int n,

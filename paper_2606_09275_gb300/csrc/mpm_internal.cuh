@@ -929,7 +929,13 @@ void point_update(mpm_ctx* c, const mpm_mesh* m, const mpm_material& mat, const 
 
 // CUB wrappers (mpm_cub.cu)
 void cub_exclusive_sum_int(mpm_ctx* c, const int* in, int* out, int n);
-void cub_sort_u64(mpm_ctx* c, uint64_t* keys, uint64_t* tmp, int n, int end_bit);
+// bits that hold the numbers 0..v
+inline int bits_for(long long v) {
+  int b = 1;
+  while ((1LL << b) <= v) ++b;
+  return b;
+}
+uint64_t* cub_sort_u64(mpm_ctx* c, uint64_t* keys, uint64_t* alt, int n, int begin_bit, int end_bit);
 void cub_sort_pairs_int(mpm_ctx* c, const int* kin, int* kout, const int* vin, int* vout, int n,
                         int end_bit);
 int cub_unique_u64(mpm_ctx* c, const uint64_t* in, uint64_t* out, int n);

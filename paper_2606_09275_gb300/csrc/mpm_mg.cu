@@ -1099,7 +1099,8 @@ void mg_structure(mpm_ctx* c, mpm_mesh* m) {
       uint64_t* keys = grow<uint64_t>(c, c->tmp[4], n8);
       uint64_t* alt = grow<uint64_t>(c, c->tmp[5], n8);
       MPM_LAUNCH(k_mg_tkeys<<<grid_for(n8, 256), 256, 0, st>>>(nd, ptr<int>(G.p_idx), keys));
-      cub_sort_u64(c, keys, alt, (int)n8, 64);
+      // listed in ascending order of the lower 35 bits: sorted by the row alone
+      keys = cub_sort_u64(c, keys, alt, (int)n8, 35, 35 + bits_for(L.nrow));
       int* tptr = grow<int>(c, G.t_ptr, L.nrow + 1);
       int* tmax = (int*)(c->d_red + 8);
       MPM_CUDA(cudaMemsetAsync(tmax, 0, sizeof(int), st));

@@ -30,3 +30,18 @@ def test_domains_of_up_to_27_leaves(length):
     assert np.max(np.abs(np.where(mask[..., None], mesh.export("dS") - dS, 0))) < 1e-13 * scale
     if length > 1.5:
         assert nsup.max() == 64
+
+
+@pytest.mark.parametrize("length, longest", [(0.5, 125), (1.5, 294), (1.9, 256)])
+def test_rows_around_256_columns(length, longest):
+    """Rows beyond 256 columns take the pattern builder's large set, whole numbers throughout."""
+    from paper_2606_09275_gb300 import mpm
+    cfg = inputs.workload("column", beta=0.4, points=dict(spacing=length / 8, jitter=0.02, seed=4, ys=1e4))
+    pts = inputs.make_points(cfg)
+    om = oracle.Model(cfg, pts)
+    om.build(nosplit=True)
+    mesh = mpm.octree_build(mpm.Context(), cfg, mpm.Points(pts), nosplit=True)
+    rp, col = om.pattern()
+    assert np.array_equal(mesh.export("row_ptr"), rp)
+    assert np.array_equal(mesh.export("col"), col)
+    assert np.diff(rp).max() == longest
