@@ -305,8 +305,8 @@ __global__ void k_mg_rap1(int nd, int R, int S, const float* __restrict__ pw,
 // (1) k_mg_kp, one warp per fine row i: (K P)_iJ = sum_j K_ij P_jJ for the
 //     4 x 4 x 4 level-1 nodes J = c_i + (-1..2) around the level-1 cell c_i
 //     of dof i (every P_jJ of a column j of the row lands there), the
-//     columns j taken in row order, accumulated in shared memory and written
-//     out as kp[i][9][64];
+//     columns j taken in row order, cell by cell, accumulated in shared memory
+//     and written out as kp[i][9][64];
 // (2) k_mg_ptkp, one warp per level-1 row a: A_ab = sum_i P_ia (K P)_ib over
 //     the fine dofs i of the transpose of P, in dof order, lanes over the
 //     125 stencil offsets b - a.
@@ -323,18 +323,23 @@ __host__ __device__ constexpr int kp_warps() {
 template <class T>
 struct KpShared {
   static constexpr int NW = kp_warps<T>();
-  T tab[NW][KP_NS * 9];     // (K P)_i, [slot][9]
-  T sv[NW][32][9];          // a chunk of 32 blocks K_ij (masked)
-  int ss[NW][32][8];        // their P_j entries: slot (-1: none) ...
-  float sw[NW][32][8];      // ... and weight
+  T tab[NW][KP_NS * 9];                // (K P)_i, [slot][9]
+  alignas(16) T sv[NW][32][3][4];      // a chunk of 32 blocks K_ij (masked), rows padded to 4
+  alignas(16) float sw[NW][32][8];     // the weights of their dof's 8 cell corners
 };
 
+// What bounds it: shared-memory instructions.  The columns of a row are in
+// Morton order, so those of one level-1 cell follow each other and go to the
+// same 8 corners: a lane owns a (corner, block row) pair and sums its three
+// entries over such a run in registers, two loads a column, before it adds them
+// to the table.  A term at a time straight into the table took 15 accesses a
+// column, the weights read from P 64 bytes a column: 3.01 ms for the 248 k rows
+// of the indentation block, 1.14 ms now (reading K takes 0.17).
 template <class T>
 __global__ void __launch_bounds__(32 * kp_warps<T>())
     k_mg_kp(int nd, int D, int d1, const int* __restrict__ dof_node, const uint64_t* __restrict__ nkey,
-            const float* __restrict__ pw, const int* __restrict__ pidx, const int* __restrict__ fmask,
-            const int* __restrict__ rp, const int* __restrict__ col, Sliced SK, const T* __restrict__ K,
-            const int* __restrict__ xyz, T* kp, int* kpc, int* err) {
+            const int* __restrict__ fmask, const int* __restrict__ rp, const int* __restrict__ col,
+            Sliced SK, const T* __restrict__ K, T* kp, int* kpc, int* err) {
   __shared__ KpShared<T> sh;
   int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int i = blockIdx.x * kp_warps<T>() + wi;
@@ -344,52 +349,77 @@ __global__ void __launch_bounds__(32 * kp_warps<T>())
   int X[3], ci[3];
   demorton(nkey[dof_node[i]], X);
   int shf = D - d1, n = 1 << d1;
+  float h = 1.0f / (float)(1 << shf);
   for (int d = 0; d < 3; ++d) ci[d] = min(X[d] >> shf, n - 1);
   if (lane == 0) kpc[i] = pack3(ci[0], ci[1], ci[2]);
   int mi = fmask[i];
   int s0 = rp[i], nb = rp[i + 1] - s0;
   int si = SK.pos[i], sl = si >> 5, W = SK.w[sl];
   long long b0 = SK.base[sl];
+  int q = lane / 3, c = lane - 3 * q;  // the lane's corner and block row (lanes below 24)
   bool bad = false;
   for (int base = 0; base < nb; base += 32) {
     int idx = base + lane, cnt = min(32, nb - base);
+    int cell = -1;  // of the lane's column, around the cell of i
     __syncwarp();
     if (idx < nb) {
       int j = col[s0 + idx];
       int mj = fmask[j];
       long long slot = sliced_slot(b0, si, idx);
 #pragma unroll
-      for (int e = 0; e < 9; ++e) {
-        int ca = e / 3, ck = e - 3 * (e / 3);
-        sh.sv[wi][lane][e] = (((mi >> ca) & 1) || ((mj >> ck) & 1)) ? (T)0 : K[sliced_entry(b0, W, slot, e)];
-      }
+      for (int a = 0; a < 3; ++a) {
+        T v[4];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        int b = pidx[8 * (size_t)j + q];
-        int s = -1;
-        if (b >= 0) {
-          int cb[3];
-          unpack3(xyz[b], cb);
-          int o0 = cb[0] - ci[0] + 1, o1 = cb[1] - ci[1] + 1, o2 = cb[2] - ci[2] + 1;
-          if ((unsigned)o0 < 4u && (unsigned)o1 < 4u && (unsigned)o2 < 4u)
-            s = o0 + 4 * (o1 + 4 * o2);
-          else
-            bad = true;
-          sh.sw[wi][lane][q] = pw[8 * (size_t)j + q];
-        }
-        sh.ss[wi][lane][q] = s;
+        for (int k = 0; k < 3; ++k)
+          v[k] = (((mi >> a) & 1) || ((mj >> k) & 1)) ? (T)0 : K[sliced_entry(b0, W, slot, 3 * a + k)];
+        v[3] = (T)0;
+        st4(sh.sv[wi][lane][a], v);
       }
+      demorton(nkey[dof_node[j]], X);
+      float t[3];
+      cell = 0;
+      for (int d = 0; d < 3; ++d) {
+        int cj = min(X[d] >> shf, n - 1), o = cj - ci[d] + 1;
+        t[d] = (float)(X[d] - (cj << shf)) * h;
+        // the corners with a weight lie in the 4 x 4 x 4 nodes
+        if (o < 0 || o > 3 || (o == 3 && t[d] != 0.0f)) bad = true;
+        cell |= (o & 7) << (3 * d);
+      }
+      float w[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        w[k] = ((k & 1) ? t[0] : 1.0f - t[0]) * ((k & 2) ? t[1] : 1.0f - t[1]) *
+               ((k & 4) ? t[2] : 1.0f - t[2]);
+      st4(sh.sw[wi][lane], w);
+      st4(sh.sw[wi][lane] + 4, w + 4);
     }
+    int before = __shfl_up_sync(0xffffffffu, cell, 1);
+    unsigned start = __ballot_sync(0xffffffffu, idx < nb && (lane == 0 || cell != before));
     __syncwarp();
-    // column by column (a fixed order per accumulator): the 8 x 9 (entry,
-    // component) terms of a column go to distinct accumulators
-    for (int u = 0; u < cnt; ++u) {
-      for (int t = lane; t < 72; t += 32) {
-        int q = t / 9, e = t - 9 * (t / 9);
-        int s = sh.ss[wi][u][q];
-        if (s >= 0) tab[9 * s + e] += (T)sh.sw[wi][u][q] * sh.sv[wi][u][e];
+    // run by run of columns of the same cell (a fixed order per accumulator)
+    for (int u = 0; u < cnt;) {
+      unsigned rest = u < 31 ? start >> (u + 1) : 0u;
+      int u1 = rest ? u + __ffs(rest) : cnt;
+      int o = __shfl_sync(0xffffffffu, cell, u);
+      if (lane < 24) {
+        T a0 = (T)0, a1 = (T)0, a2 = (T)0;
+        for (; u < u1; ++u) {
+          T v[4], w = (T)sh.sw[wi][u][q];
+          ld4(sh.sv[wi][u][c], v);
+          a0 += w * v[0];
+          a1 += w * v[1];
+          a2 += w * v[2];
+        }
+        int o0 = (o & 7) + (q & 1), o1 = ((o >> 3) & 7) + ((q >> 1) & 1), o2 = (o >> 6) + (q >> 2);
+        if (o0 < 4 && o1 < 4 && o2 < 4) {
+          T* p = tab + 9 * (o0 + 4 * (o1 + 4 * o2)) + 3 * c;
+          p[0] += a0;
+          p[1] += a1;
+          p[2] += a2;
+        }
       }
-      __syncwarp();
+      u = u1;
+      __syncwarp();  // the next run's lanes may add to the same nodes
     }
   }
   if (bad) atomicOr(err, EB_ROW);
@@ -519,6 +549,141 @@ __global__ void k_mg_rapu(int nrow_f, int Rc, int Sc, int n1c, const int* __rest
   }
 }
 
+// One axis of the trilinear interpolation, gathered: five values of the finer
+// nodes i - 2 .. i + 2 to the coarse nodes they interpolate from; i an even node
+// (three of them) or an odd one (four).  Halves to the nearest integer.
+__device__ inline void gather_axis(const long long* v, bool odd, long long* o) {
+  auto h = [](long long x) { return (x + 1) >> 1; };
+  if (odd) {
+    o[0] = h(v[0]);
+    o[1] = h(v[0]) + v[1] + h(v[2]);
+    o[2] = h(v[2]) + v[3] + h(v[4]);
+    o[3] = h(v[4]);
+  } else {
+    o[0] = v[0] + h(v[1]);
+    o[1] = h(v[1]) + v[2] + h(v[3]);
+    o[2] = h(v[3]) + v[4];
+    o[3] = 0;
+  }
+}
+
+// The same product gathered, for stencils of radius 2 on both levels: one block
+// per coarse row a, in the fixed point of the scattered product.  Over the rows
+// i of the finer nodes 2 a + {-1, 0, 1}^3, the 5 x 5 x 5 blocks of a row are
+// interpolated an axis at a time, a thread per line, to the 4 x 4 x 4 coarse
+// nodes around i, and added to the row of a in shared memory; the next row's
+// loads are in flight meanwhile.  What bounds it: shared-memory and integer
+// issue, and on levels of a few hundred rows the chain of 27 rows.  The
+// scattered form sends every one of the 27 x 422 x 9 terms of a coarse row to
+// L2 as a 64-bit atomic (2.38, 0.46, 0.17 and 0.13 ms on the levels below the
+// 33 k rows of the indentation block's level 1, and its conversion pass); a
+// thread per entry summing its up to 27 terms in three nested loops took 1.88,
+// 0.32, 0.13 and 0.13 ms; this form takes 0.27, 0.05, 0.03
+// and 0.03.
+constexpr int RG = 256;  // threads per block, at least 225
+template <class T>
+__global__ void __launch_bounds__(RG)
+    k_mg_rapg(const int* __restrict__ xyz_c, int n1f, const int* __restrict__ gid_f,
+              const int* __restrict__ fmask, const T* __restrict__ Af, T* A,
+              const unsigned long long* __restrict__ bnd) {
+  constexpr int S = 125, NE = 9 * S;
+  __shared__ long long acc[NE];        // the row of a, [z][y][x][9] around a
+  __shared__ long long bx[4 * 225];    // after x: [x'][z][y][9]
+  __shared__ long long by[4 * 180];    // after y: [y'][x'][z][9]
+  __shared__ int node[343];            // rows of the finer nodes 2 a + {-3..3}^3, -1: none
+  __shared__ unsigned char mask[343];  // their Dirichlet components
+  int t = threadIdx.x, a = blockIdx.x;
+  double B = __longlong_as_double((long long)*bnd) * 27.0;
+  int ex = !(B > 0.0) || !isfinite(B) ? 0 : 60 - ilogb(B);  // as fixed_scale
+  int ca[3];
+  unpack3(xyz_c[a], ca);
+  for (int f = t; f < 343; f += RG) {
+    int x = 2 * ca[0] + f % 7 - 3, y = 2 * ca[1] + (f / 7) % 7 - 3, z = 2 * ca[2] + f / 49 - 3;
+    bool in = x >= 0 && y >= 0 && z >= 0 && x < n1f && y < n1f && z < n1f;
+    int j = in ? gid_f[x + n1f * (y + n1f * z)] : -1;
+    node[f] = j;
+    mask[f] = j >= 0 ? (unsigned char)fmask[j] : (unsigned char)7;
+  }
+  for (int f = t; f < NE; f += RG) acc[f] = 0;
+  __syncthreads();
+  // the thread's lines: (y, z, e), (x', z, e) and (x', y', e)
+  int e = t % 9, yz = t / 9;
+  bool onx = t < 225, ony = t < 180, onz = t < 144;
+  int ex3 = e / 3, ec3 = e % 3;
+  int line_x = 45 * yz + e;                                        // of a row of Af, 9 a step
+  int mask_x = 7 * (yz % 5) + 49 * (yz / 5);                       // of the node i - (2, 2, 2)
+  int line_y = 225 * (yz / 5) + 45 * (yz % 5) + e;                 // of bx, 9 a step
+  int line_z = 180 * (yz / 4) + 45 * (yz % 4) + e;                 // of by, 9 a step
+  int line_a = 9 * (yz % 4 + 5 * (yz / 4)) + e;                    // of acc, 225 a step
+  T next[5];
+  auto center = [](int q) { return 2 + q % 3 + 7 * (2 + (q / 3) % 3 + 7 * (2 + q / 9)); };
+  auto fetch = [&](int q) {
+    if (q >= 27 || !onx) return;
+    int i = node[center(q)];
+    if (i < 0) return;
+    const T* p = Af + (size_t)i * NE + line_x;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) next[k] = p[9 * k];
+  };
+  fetch(0);
+  for (int q = 0; q < 27; ++q) {
+    int ctr = center(q);
+    if (node[ctr] < 0) {  // the same for the whole block
+      fetch(q + 1);
+      continue;
+    }
+    int dx = q % 3 - 1, dy = (q / 3) % 3 - 1, dz = q / 9 - 1;
+    int w = abs(dx) + abs(dy) + abs(dz);  // P_ia = 2^-w
+    long long v[5], o[4];
+    if (onx) {
+      bool off = (mask[ctr] >> ex3) & 1;
+      const unsigned char* mj = mask + ctr - 114 + mask_x;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        if constexpr (sizeof(T) == 4)
+          v[k] = __float2ll_rn(scalbnf(next[k], ex - w));
+        else
+          v[k] = __double2ll_rn(scalbn(next[k], ex - w));
+        if (off || ((mj[k] >> ec3) & 1)) v[k] = 0;
+      }
+      gather_axis(v, dx != 0, o);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) bx[225 * k + t] = o[k];
+    }
+    fetch(q + 1);
+    __syncthreads();
+    if (ony) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) v[k] = bx[line_y + 9 * k];
+      gather_axis(v, dy != 0, o);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) by[180 * k + t] = o[k];
+    }
+    __syncthreads();
+    if (onz) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) v[k] = by[line_z + 9 * k];
+      gather_axis(v, dz != 0, o);
+      // the first coarse node of an axis: -1 around an even or the upper odd
+      // node, -2 around the lower; the fourth, of odd nodes only, ends at +2
+      int b = (dx >= 0 ? 1 : 0) + 5 * (dy >= 0 ? 1 : 0) + 25 * (dz >= 0 ? 1 : 0);
+      bool in = (yz % 4 < 3 || dx != 0) && (yz / 4 < 3 || dy != 0);
+      if (in) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (k < 3 || dz != 0) acc[9 * b + line_a + 225 * k] += o[k];
+      }
+    }
+  }
+  __syncthreads();
+  for (int f = t; f < NE; f += RG) {
+    if constexpr (sizeof(T) == 4)
+      A[(size_t)a * NE + f] = scalbnf(__ll2float_rn(acc[f]), -ex);
+    else
+      A[(size_t)a * NE + f] = scalbn((double)acc[f], -ex);
+  }
+}
+
 // ---------------------------------------------------------------- smoother inverses
 
 // w times the inverse of D + diag(l1 sums of the off-diagonal blocks), 12 per row
@@ -545,20 +710,29 @@ __device__ inline void store_inv(const double* a, T* o, int* err, double w) {
   o[11] = (T)0;
 }
 
-// also the largest l1 norm of a row (all 9 entries of every block), the bound
-// of the level-1 Galerkin product (a maximum of non-negative doubles, by the
-// ordering of their bit patterns: the same whatever the order)
+// maximum over the warp of non-negative doubles, by the ordering of their bit
+// patterns (the same whatever the order), added to *out by one lane
+__device__ inline void warp_max_to(unsigned long long* out, double v) {
+  unsigned long long x = (unsigned long long)__double_as_longlong(v);
+  unsigned hi = (unsigned)(x >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+  unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)x : 0u);
+  if ((threadIdx.x & 31) == 0) atomicMax(out, ((unsigned long long)mh << 32) | ml);
+}
+
+// Also the largest l1 norm of a row (all 9 entries of every block), the bound
+// of the level-1 Galerkin product, and (amax non-null) the largest |K|, which
+// scales the FP16 copy: one pass over K.  It is bound by that read: the
+// diagonal block, found at a different slot in every lane, is picked out in the
+// matrix precision (it occurs once; padding slots repeat its column with zeros),
+// not summed in FP64 in 32 divergent turns (0.39 ms, and 0.26 for a pass of its
+// own for the largest entry; 0.20 ms together now, 248 k rows).
 template <class T>
 __global__ void k_mg_dinv_fine(int nd, int npad, Sliced SK, const T* __restrict__ K, T* Dinv, int* err,
-                               double w, unsigned long long* bnd) {
-  int sr = blockIdx.x * blockDim.x + threadIdx.x;  // storage row
+                               double w, unsigned long long* bnd, unsigned* amax) {
+  int sr = blockIdx.x * blockDim.x + threadIdx.x;  // storage row; npad is a multiple of 32
   if (sr >= npad) return;
   int r = SK.row[sr];
   T* o = Dinv + 12 * (size_t)r;
-  if (r >= nd) {
-    for (int e = 0; e < 12; ++e) o[e] = (T)0;
-    return;
-  }
   // the row in the access pattern of the SpMV: four slots per 16-byte load
   int sl = sr >> 5, ln = sr & 31, W = SK.w[sl];
   long long b0 = SK.base[sl];
@@ -566,8 +740,7 @@ __global__ void k_mg_dinv_fine(int nd, int npad, Sliced SK, const T* __restrict_
   const int* cb = SK.scol + b0;
   size_t plane = (size_t)32 * W;
   // (the l1 sums, a smoother parameter, accumulate in the matrix precision)
-  double a[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-  T s[3] = {0, 0, 0};
+  T dg[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, s[3] = {0, 0, 0}, mx = 0;
   for (int k4 = 0; k4 < (W >> 2); ++k4) {
     size_t off = ((size_t)k4 * 32 + ln) * 4;
     int4 c = *reinterpret_cast<const int4*>(cb + off);
@@ -577,44 +750,100 @@ __global__ void k_mg_dinv_fine(int nd, int npad, Sliced SK, const T* __restrict_
     for (int e = 0; e < 9; ++e) ld4(Kb + e * plane + off, v[e]);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      if (cc[j] == r) {
+      bool on = cc[j] == r;
 #pragma unroll
-        for (int e = 0; e < 9; ++e) a[e] += (double)v[e][j];
-      } else {
-#pragma unroll
-        for (int e = 0; e < 9; ++e) s[e / 3] += v[e][j] < (T)0 ? -v[e][j] : v[e][j];
+      for (int e = 0; e < 9; ++e) {
+        T av = v[e][j] < (T)0 ? -v[e][j] : v[e][j];
+        dg[e] = on ? dg[e] + v[e][j] : dg[e];
+        s[e / 3] += on ? (T)0 : av;
+        mx = av > mx ? av : mx;
       }
     }
   }
-  double l1 = (double)s[0] + (double)s[1] + (double)s[2];
-  for (int e = 0; e < 9; ++e) l1 += fabs(a[e]);
-  atomicMax(bnd, (unsigned long long)__double_as_longlong(l1));
+  if (r >= nd) {
+    for (int e = 0; e < 9; ++e) dg[e] = (T)0;
+    s[0] = s[1] = s[2] = (T)0;
+  }
+  double a[9], l1 = (double)s[0] + (double)s[1] + (double)s[2];
+  for (int e = 0; e < 9; ++e) {
+    a[e] = (double)dg[e];
+    l1 += fabs(a[e]);
+  }
+  warp_max_to(bnd, l1);
+  if (sizeof(T) == 4 && amax) {
+    unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint((float)mx));
+    if ((threadIdx.x & 31) == 0) atomicMax(amax, m);
+  }
+  if (r >= nd) {
+    for (int e = 0; e < 12; ++e) o[e] = (T)0;
+    return;
+  }
   for (int d = 0; d < 3; ++d) a[4 * d] += (double)s[d];
   store_inv<T>(a, o, err, w);
 }
 
+// a + b with the rounding error kept in e (FP32; an FP64 sum takes it as it is)
+__device__ inline void add_kept(float& a, float& e, float b) {
+  float s = a + b, z = s - a;
+  e += (a - (s - z)) + (b - z);
+  a = s;
+}
+__device__ inline void add_kept(double& a, double&, double b) { a += b; }
+
+// Level operators: eight lanes per row read it coalesced and sum its l1 parts
+// (FP32 entries in FP32 with the errors kept, so that no FP64 is spent per
+// entry), then a thread per row, the first warp's, inverts.  A thread per row
+// for the whole walk took 0.18 ms for 33 k rows and 0.11 ms, pure latency, on
+// each of the small levels; 0.04 and 0.012 ms now.
+constexpr int DR = 32;  // rows per block of 256 threads
 template <class T>
-__global__ void k_mg_dinv(int nrow, int npad, int S, int R, const T* __restrict__ A, T* Dinv, int* err,
-                          double w, unsigned long long* bnd) {
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= npad) return;
+__global__ void __launch_bounds__(8 * DR)
+    k_mg_dinv(int nrow, int npad, int S, int R, const T* __restrict__ A, T* Dinv, int* err, double w,
+              unsigned long long* bnd) {
+  __shared__ double ls[DR][3];
+  int S1 = 2 * R + 1, center = R + S1 * (R + S1 * R);
+  {
+    int r = blockIdx.x * DR + (threadIdx.x >> 3), l = threadIdx.x & 7;
+    const T* row = A + (size_t)r * S * 9;
+    T s[3] = {0, 0, 0}, c[3] = {0, 0, 0};
+    if (r < nrow)
+      for (int o = l; o < S; o += 8) {
+        if (o == center) continue;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+          T v = row[9 * o + e];
+          add_kept(s[e / 3], c[e / 3], v < (T)0 ? -v : v);
+        }
+      }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) {
+        T so = __shfl_xor_sync(0xffffffffu, s[d], o), co = __shfl_xor_sync(0xffffffffu, c[d], o);
+        add_kept(s[d], c[d], so);
+        c[d] += co;
+      }
+      if (l == 0) ls[threadIdx.x >> 3][d] = (double)s[d] + (double)c[d];
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x >= DR) return;
+  int r = blockIdx.x * DR + threadIdx.x;  // npad is a multiple of 32: r < npad
   T* o = Dinv + 12 * (size_t)r;
+  double a[9], l1 = 0.0;
+  const double* sd = ls[threadIdx.x];
+  if (r < nrow) {
+    const T* row = A + (size_t)r * S * 9;
+    for (int e = 0; e < 9; ++e) a[e] = (double)row[9 * center + e];
+    l1 = sd[0] + sd[1] + sd[2];
+    for (int e = 0; e < 9; ++e) l1 += fabs(a[e]);
+  }
+  warp_max_to(bnd, l1);
   if (r >= nrow) {
     for (int e = 0; e < 12; ++e) o[e] = (T)0;
     return;
   }
-  int S1 = 2 * R + 1, center = R + S1 * (R + S1 * R);
-  const T* row = A + (size_t)r * S * 9;
-  double a[9], s[3] = {0, 0, 0};
-  for (int e = 0; e < 9; ++e) a[e] = (double)row[9 * center + e];
-  for (int oo = 0; oo < S; ++oo) {
-    if (oo == center) continue;
-    for (int e = 0; e < 9; ++e) s[e / 3] += fabs((double)row[9 * oo + e]);
-  }
-  double l1 = s[0] + s[1] + s[2];
-  for (int e = 0; e < 9; ++e) l1 += fabs(a[e]);
-  atomicMax(bnd, (unsigned long long)__double_as_longlong(l1));
-  for (int d = 0; d < 3; ++d) a[4 * d] += s[d];
+  for (int d = 0; d < 3; ++d) a[4 * d] += sd[d];
   store_inv<T>(a, o, err, w);
 }
 
@@ -624,14 +853,18 @@ __global__ void k_mg_dinv(int nrow, int npad, int S, int R, const T* __restrict_
 // direction the coarse space does not resolve (interpolation columns that
 // coincide on a thin active region): its row and column are dropped, which
 // leaves the pseudo-inverse on the rest and keeps the V-cycle positive
-// definite (the smoother part alone is).
+// definite (the smoother part alone is).  In place: at step k the columns up to
+// k hold the inverse's, the others the matrix's, so a step is one fma an entry
+// of n3 x n3 rather than of n3 x 2 n3 (0.63 ms at n3 = 81, bound by the one SM's
+// FP64 pipe; 0.28 now).
 template <class T>
 __global__ void k_mg_dense(int nrow, int S, int R, const int* __restrict__ xyz, int n1,
                            const int* __restrict__ gid, const T* __restrict__ A, T* Cinv) {
-  extern __shared__ double M[];  // [n3][2 n3]
+  extern __shared__ double M[];  // [n3][n3], then the pivot's column [n3]
   __shared__ double dmax;
-  int n3 = 3 * nrow, w2 = 2 * n3;
-  for (int u = threadIdx.x; u < n3 * w2; u += blockDim.x) M[u] = 0.0;
+  int n3 = 3 * nrow;
+  double* pc = M + n3 * n3;
+  for (int u = threadIdx.x; u < n3 * n3; u += blockDim.x) M[u] = 0.0;
   __syncthreads();
   int S1 = 2 * R + 1;
   for (int u = threadIdx.x; u < nrow * S; u += blockDim.x) {
@@ -643,58 +876,40 @@ __global__ void k_mg_dense(int nrow, int S, int R, const int* __restrict__ xyz, 
     int b = gid[cb[0] + n1 * (cb[1] + n1 * cb[2])];
     if (b < 0) continue;
     const T* blk = A + ((size_t)a * S + o) * 9;
-    for (int e = 0; e < 9; ++e) M[(3 * a + e / 3) * w2 + 3 * b + e % 3] = (double)blk[e];
+    for (int e = 0; e < 9; ++e) M[(3 * a + e / 3) * n3 + 3 * b + e % 3] = (double)blk[e];
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     double d = 0.0;
-    for (int i = 0; i < n3; ++i) d = fmax(d, M[i * w2 + i]);
+    for (int i = 0; i < n3; ++i) d = fmax(d, M[i * n3 + i]);
     dmax = d;
   }
-  for (int i = threadIdx.x; i < n3; i += blockDim.x) M[i * w2 + n3 + i] = 1.0;
   __syncthreads();
   double tiny = 1e-12 * dmax;
+  int wi = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   for (int k = 0; k < n3; ++k) {
-    double piv = M[k * w2 + k];
+    double piv = M[k * n3 + k];
+    bool drop = !(piv > tiny) || !isfinite(piv);
+    for (int i = threadIdx.x; i < n3; i += blockDim.x) pc[i] = M[i * n3 + k];
     __syncthreads();
-    if (!(piv > tiny) || !isfinite(piv)) {
-      // drop direction k: zero its row and column in both halves
-      for (int j = threadIdx.x; j < w2; j += blockDim.x) M[k * w2 + j] = 0.0;
-      for (int i = threadIdx.x; i < n3; i += blockDim.x) {
-        M[i * w2 + k] = 0.0;
-        M[i * w2 + n3 + k] = 0.0;
-      }
-      __syncthreads();
-      continue;
-    }
-    for (int j = threadIdx.x; j < w2; j += blockDim.x) M[k * w2 + j] /= piv;
-    __syncthreads();
-    for (int u = threadIdx.x; u < n3 * w2; u += blockDim.x) {
-      int i = u / w2, j = u - w2 * i;
-      if (i == k || j == k) continue;
-      M[u] -= M[i * w2 + k] * M[k * w2 + j];
+    // the pivot's row divided, its column started from the identity's
+    for (int j = threadIdx.x; j < n3; j += blockDim.x) {
+      M[k * n3 + j] = drop ? 0.0 : (j == k ? 1.0 : M[k * n3 + j]) / piv;
+      if (j != k) M[j * n3 + k] = 0.0;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < n3; i += blockDim.x)
-      if (i != k) M[i * w2 + k] = 0.0;
+    if (drop) continue;
+    for (int i = wi; i < n3; i += nw) {
+      if (i == k) continue;
+      double f = pc[i];
+      for (int j = lane; j < n3; j += 32) M[i * n3 + j] = fma(-f, M[k * n3 + j], M[i * n3 + j]);
+    }
     __syncthreads();
   }
-  for (int u = threadIdx.x; u < n3 * n3; u += blockDim.x) {
-    int i = u / n3, j = u - n3 * i;
-    Cinv[u] = (T)M[i * w2 + n3 + j];
-  }
+  for (int u = threadIdx.x; u < n3 * n3; u += blockDim.x) Cinv[u] = (T)M[u];
 }
 
 // ---------------------------------------------------------------- FP16 smoothing copy
-
-// largest |K| (as ordered bits of a non-negative float)
-__global__ void k_absmax(long long n, const float* __restrict__ K, unsigned* out) {
-  float m = 0.f;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    m = fmaxf(m, fabsf(K[i]));
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(m));
-}
 
 // FP16 copy of K scaled by 2^e (the largest |entry| maps below 2^14, clear of
 // the FP16 limit 65504); scaling by a power of two keeps the copy exactly as
@@ -1152,16 +1367,15 @@ void mg_numeric(mpm_ctx* c, mpm_mesh* m, const T* K, bool coarse) {
   unsigned long long* bnd = grow<unsigned long long>(c, G.bound, 16);
   MPM_CUDA(cudaMemsetAsync(bnd, 0, 16 * sizeof(unsigned long long), st));
   T* fD = grow<T>(c, G.fDinv, 12 * (size_t)npad);
-  MPM_LAUNCH_P(MPM_PROF_MG_SETUP, k_mg_dinv_fine<T><<<grid_for(npad, 256), 256, 0, st>>>(nd, npad, SK, K, fD, c->d_err, kSmoothW, bnd));
+  unsigned* amax = (unsigned*)(c->d_red + 10);
+  MPM_CUDA(cudaMemsetAsync(amax, 0, sizeof(unsigned), st));
+  MPM_LAUNCH_P(MPM_PROF_MG_SETUP, k_mg_dinv_fine<T><<<grid_for(npad, 256), 256, 0, st>>>(nd, npad, SK, K, fD, c->d_err, kSmoothW, bnd, amax));
   grow<T>(c, G.fr, 4 * (size_t)npad);
   grow<T>(c, G.fx, 4 * (size_t)npad);
   if constexpr (sizeof(T) == 4) {
     // FP16 copy of the fine matrix for the V-cycle's two fine-level products
     long long n9 = 9LL * m->nslot;
-    unsigned* amax = (unsigned*)(c->d_red + 10);
     float* ksc = (float*)(c->d_red + 11);
-    MPM_CUDA(cudaMemsetAsync(amax, 0, sizeof(unsigned), st));
-    MPM_LAUNCH_P(MPM_PROF_MG_SETUP, k_absmax<<<4 * 152, 256, 0, st>>>(n9, K, amax));
     MPM_LAUNCH_P(MPM_PROF_MG_SETUP, k_to_half<<<grid_for(32LL * m->nslice, 256), 256, 0, st>>>(m->nslice, SK, K, amax, grow<__half>(c, G.fKh, n9), ksc));
   }
   if (!coarse) return;
@@ -1179,11 +1393,14 @@ void mg_numeric(mpm_ctx* c, mpm_mesh* m, const T* K, bool coarse) {
       int* kpc = grow<int>(c, G.kpc, nd);
       constexpr int NW = kp_warps<T>();
       MPM_LAUNCH_P(MPM_PROF_MG_RAP, k_mg_kp<T><<<(nd + NW - 1) / NW, 32 * NW, 0, st>>>(
-          nd, m->g.D, L.d, ptr<int>(m->dof_node), ptr<uint64_t>(m->node_key), ptr<float>(G.p_w),
-          ptr<int>(G.p_idx), ptr<int>(m->dof_mask), ptr<int>(m->row_ptr), ptr<int>(m->col), SK, K,
-          ptr<int>(L.xyz), kp, kpc, c->d_err));
+          nd, m->g.D, L.d, ptr<int>(m->dof_node), ptr<uint64_t>(m->node_key), ptr<int>(m->dof_mask),
+          ptr<int>(m->row_ptr), ptr<int>(m->col), SK, K, kp, kpc, c->d_err));
       MPM_LAUNCH_P(MPM_PROF_MG_RAP, k_mg_ptkp<T><<<grid_for(L.nrow, 8), 256, 0, st>>>(
           L.nrow, ptr<int>(L.xyz), ptr<int>(G.t_ptr), ptr<int>(G.t_idx), ptr<float>(G.t_w), kpc, kp, A));
+    } else if (l > 0 && L.R == 2 && G.lev[l - 1].R == 2) {
+      MGLevel& F = G.lev[l - 1];
+      MPM_LAUNCH_P(MPM_PROF_MG_RAP, k_mg_rapg<T><<<L.nrow, RG, 0, st>>>(
+          ptr<int>(L.xyz), F.n1, ptr<int>(F.gid), ptr<int>(F.mask), ptr<T>(F.A), A, bnd + l));
     } else {
     ACC* acc = grow<ACC>(c, G.acc, nA);
     MPM_CUDA(cudaMemsetAsync(acc, 0, sizeof(ACC) * nA, st));
@@ -1203,7 +1420,7 @@ void mg_numeric(mpm_ctx* c, mpm_mesh* m, const T* K, bool coarse) {
     MPM_LAUNCH_P(MPM_PROF_MG_RAP, (k_mg_from_fixed<T, ACC><<<4 * 152, 256, 0, st>>>((long long)nA, acc, bnd + l, cnt, A)));
     }
     MPM_LAUNCH_P(MPM_PROF_MG_SETUP, k_mg_fix_masked<T><<<grid_for(L.nrow, 128), 128, 0, st>>>(L.nrow, L.S, L.R, ptr<int>(L.mask), A));
-    MPM_LAUNCH_P(MPM_PROF_MG_SETUP, k_mg_dinv<T><<<grid_for(L.npad, 128), 128, 0, st>>>(L.nrow, L.npad, L.S, L.R, A,
+    MPM_LAUNCH_P(MPM_PROF_MG_SETUP, k_mg_dinv<T><<<grid_for(L.npad, DR), 8 * DR, 0, st>>>(L.nrow, L.npad, L.S, L.R, A,
                                                                    grow<T>(c, L.Dinv, 12 * (size_t)L.npad), c->d_err, kSmoothW,
                                                                    bnd + l + 1));
     // level vectors: padding rows stay zero
@@ -1214,9 +1431,9 @@ void mg_numeric(mpm_ctx* c, mpm_mesh* m, const T* K, bool coarse) {
   MGLevel& C = G.lev[G.nlev - 1];
   int n3 = G.n3c;
   T* Ci = grow<T>(c, G.cinv, (size_t)std::max(n3 * n3, 1));
-  size_t dsm = sizeof(double) * (size_t)n3 * 2 * n3;
+  size_t dsm = sizeof(double) * (size_t)n3 * (n3 + 1);
   MPM_CUDA(cudaFuncSetAttribute(k_mg_dense<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm));
-  MPM_LAUNCH_P(MPM_PROF_MG_SETUP, k_mg_dense<T><<<1, 256, dsm, st>>>(C.nrow, C.S, C.R, ptr<int>(C.xyz), C.n1, ptr<int>(C.gid),
+  MPM_LAUNCH_P(MPM_PROF_MG_SETUP, k_mg_dense<T><<<1, 1024, dsm, st>>>(C.nrow, C.S, C.R, ptr<int>(C.xyz), C.n1, ptr<int>(C.gid),
                                                 ptr<T>(C.A), Ci));
   G.prec = sizeof(T) == 4 ? MPM_MIXED : MPM_FP64;
   G.num_gen = m->gen;
