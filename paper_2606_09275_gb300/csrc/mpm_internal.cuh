@@ -391,6 +391,97 @@ __device__ inline double snap_grid(double v) {
   return fabs(v - r) < 1e-9 ? r : v;
 }
 
+// bounds of a GIMP domain in finest-grid units as integers: floor of the lower
+// and upper bound of each axis, and whether the upper one is an integer
+struct DomainCells {
+  int lo[3], hi[3];
+  bool whole[3];
+};
+
+// One open box of the walk over a domain's leaf intersections, in integer
+// arithmetic: every cut face is a leaf face, an integer in grid units, so a
+// bound is either the domain's own (code -1) or a face.  The box [a, b) is cut
+// at the leaf K of its lower corner: its part in K ends at e; up to three more
+// boxes stay open, that of axis d if gt[d], with the bounds child() gives.
+struct LeafCut {
+  int K, s, kh[3], e[3];
+  bool gt[3];
+  __device__ void cut(const Geo& g, const uint64_t* __restrict__ lkey, const int* __restrict__ llev,
+                      int nl, const DomainCells& c, const int* a, const int* b) {
+    int q[3], ka[3];
+    for (int d = 0; d < 3; ++d) {
+      q[d] = a[d] < 0 ? c.lo[d] : a[d];
+      q[d] = q[d] > g.N - 1 ? g.N - 1 : (q[d] < 0 ? 0 : q[d]);
+    }
+    K = locate(lkey, nl, q[0], q[1], q[2]);
+    s = 1 << (g.D - llev[K]);
+    demorton(lkey[K], ka);
+    for (int d = 0; d < 3; ++d) {
+      kh[d] = ka[d] + s;
+      if (b[d] < 0) {
+        // the domain's upper bound against the face kh: Hi < kh iff
+        // floor(Hi) < kh; Hi > kh iff floor(Hi) > kh, or equal and Hi is not
+        // an integer
+        e[d] = c.hi[d] < kh[d] ? -1 : kh[d];
+        gt[d] = c.hi[d] > kh[d] || (!c.whole[d] && c.hi[d] == kh[d]);
+      } else {
+        e[d] = b[d] < kh[d] ? b[d] : kh[d];
+        gt[d] = b[d] > kh[d];
+      }
+    }
+  }
+  __device__ void child(int d, const int* a, const int* b, int* r) const {
+    for (int k = 0; k < 3; ++k) {
+      r[k] = k == d ? kh[k] : a[k];
+      r[3 + k] = k < d ? e[k] : b[k];
+    }
+  }
+};
+
+__device__ inline int warp_excl_scan(int v, int lane) {
+  int x = v;
+  for (int o = 1; o < 32; o <<= 1) {
+    int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  return x - v;
+}
+
+// the leaf intersections of a warp's domain, the open boxes of a round one per
+// lane: put(n, K, a, e) for intersection n, in the leaf K, with the bound codes
+// a and e; `open` holds MAXK boxes in shared memory.  Returns their number, or
+// -1 above MAXK.
+template <class Put>
+__device__ int warp_cut_domain(const Geo& g, const uint64_t* __restrict__ lkey, const int* __restrict__ llev,
+                               int nl, const DomainCells& c, int (*open)[6], int lane, Put put) {
+  int a[3] = {-1, -1, -1}, b[3] = {-1, -1, -1};
+  int n = 0;
+  for (int nopen = 1; nopen > 0;) {
+    LeafCut l;
+    l.gt[0] = l.gt[1] = l.gt[2] = false;
+    if (lane < nopen) {
+      l.cut(g, lkey, llev, nl, c, a, b);
+      put(n + lane, l.K, a, l.e);
+    }
+    n += nopen;
+    int kids = (l.gt[0] ? 1 : 0) + (l.gt[1] ? 1 : 0) + (l.gt[2] ? 1 : 0);
+    int at = warp_excl_scan(kids, lane);
+    nopen = __shfl_sync(0xffffffffu, at + kids, 31);
+    if (n + nopen > MAXK) return -1;  // every open box yields an intersection
+    __syncwarp();
+    for (int d = 0; d < 3; ++d)
+      if (l.gt[d]) l.child(d, a, b, open[at++]);
+    __syncwarp();
+    if (lane < nopen)
+      for (int d = 0; d < 3; ++d) {
+        a[d] = open[lane][d];
+        b[d] = open[lane][3 + d];
+      }
+  }
+  __syncwarp();
+  return n;
+}
+
 // ------------------------------------------------------------------ rigid body geometry
 
 __device__ inline double body_rxy(const mpm_rigid& b, const double* lo, const double* hi) {
