@@ -1634,9 +1634,11 @@ void assemble(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const mpm
     MPM_CUDA(cudaMemsetAsync(dyn->Kgb, 0, sizeof(double) * 18 * (size_t)nd, st));
     MPM_CUDA(cudaMemsetAsync(dyn->Kbg, 0, sizeof(double) * 18 * (size_t)nd, st));
   }
-  // grid-sum partials for every reduction below, sized once; a clean ticket
+  // grid-sum partials for every reduction below, sized once; a clean ticket,
+  // norms and reaction (slots 14 to 22)
   grid_red(c, 4, std::max(4096, grid_for(8LL * m->ncand, 128)));
-  MPM_CUDA(cudaMemsetAsync(c->d_ticket, 0, sizeof(unsigned), st));
+  MPM_CUDA(cudaMemsetAsync(c->d_red + 14, 0, 9 * sizeof(double), st));
+  if (out) out->clean = false;
   if (K && reuse) {
     // Newton's tangent at the increment of the last residual evaluation: its
     // dF, dF^-1, tau and spectral state are still in place, R is complete
@@ -1661,7 +1663,7 @@ void assemble(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const mpm
       MPM_LAUNCH_P(MPM_PROF_CONSTITUTIVE, k_constitutive<true, double><<<grid_for(P, 128), 128, 0, st>>>(
           P, L, ptr<double>(m->pE), ptr<double>(m->pys), ptr<double>(m->pbe), dF, V0, tau, dFinv, Mf,
           (double*)Aalg, nullptr, c->d_err));
-    MPM_CUDA(cudaMemsetAsync(fc, 0, sizeof(double) * 3 * nd, st));
+    if (contact) MPM_CUDA(cudaMemsetAsync(fc, 0, sizeof(double) * 3 * nd, st));
     MPM_LAUNCH_P(MPM_PROF_RESIDUAL, k_residual_rows<<<grid_for(nd, 8), 256, 0, st>>>(
         nd, P, load, ptr<long long>(m->src_ptr), ptr<uint64_t>(m->src_key), Mf, dS, rp, col,
         ptr<double>(m->kg), du, ptr<double>(m->fext), fint, R));
@@ -1722,7 +1724,6 @@ void assemble(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const mpm
     if (couple) body_out(c, mat, body, load, dyn, bsum, out, true);
     return;
   }
-  MPM_CUDA(cudaMemsetAsync(reac, 0, 3 * sizeof(double), st));
   if (contact) {
     if (!K)
       contact_terms<double, true, false>(c, m, mat, body, du, R, fc, reac, (double*)nullptr, dyn, bsum);
@@ -1733,11 +1734,11 @@ void assemble(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const mpm
   }
   if (want_norms) {
     double* slot = c->d_red + 16;
-    MPM_CUDA(cudaMemsetAsync(slot, 0, 4 * sizeof(double), st));
-    MPM_LAUNCH(k_norms<<<grid_strided(3 * nd), 256, 0, st>>>(3 * nd, R, fint, ptr<double>(m->fext), fc, load, finert,
+    MPM_LAUNCH(k_norms<<<grid_strided(3 * nd), 256, 0, st>>>(3 * nd, R, fint, ptr<double>(m->fext), contact ? fc : nullptr, load, finert,
                                      ptr<int>(m->dof_mask), slot, grid_red(c, 4, 4 * 152)));
-    MPM_CUDA(cudaMemcpyAsync(c->h_red + 16, slot, 7 * sizeof(double), cudaMemcpyDeviceToHost, st));
+    MPM_CUDA(cudaMemcpyAsync(c->h_red + 16, slot, 8 * sizeof(double), cudaMemcpyDeviceToHost, st));
     MPM_CUDA(cudaStreamSynchronize(st));
+    out->clean = *(const int*)(c->h_red + 23) == 0;
     out->fint_norm = sqrt(c->h_red[17]);
     out->fextc_norm = sqrt(c->h_red[18]);
     out->finert_norm = sqrt(c->h_red[19]);

@@ -121,15 +121,14 @@ extern "C" int mpm_create(mpm_ctx** out, void* stream) {
     int coop = 0;
     MPM_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device));
     if (coop) MPM_CUDA(cudaDeviceGetAttribute(&c->coop_sms, cudaDevAttrMultiProcessorCount, c->device));
-    MPM_CUDA(cudaMallocAsync((void**)&c->d_err, sizeof(int), c->stream));
-    MPM_CUDA(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
     MPM_CUDA(cudaMallocAsync((void**)&c->d_red, 64 * sizeof(double), c->stream));
+    MPM_CUDA(cudaMemsetAsync(c->d_red, 0, 64 * sizeof(double), c->stream));
+    c->d_ticket = (unsigned*)(c->d_red + 14);
+    c->d_err = (int*)(c->d_red + 23);
     // CUDA graphs for the V-cycle (MPM_GRAPHS=0 in the environment: plain
     // launches, for comparison)
     const char* eg = getenv("MPM_GRAPHS");
     if (!(eg && eg[0] == '0')) MPM_CUDA(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
-    MPM_CUDA(cudaMallocAsync((void**)&c->d_ticket, 16, c->stream));
-    MPM_CUDA(cudaMemsetAsync(c->d_ticket, 0, 16, c->stream));
     grid_red(c, 4, 4096);
     MPM_CUDA(cudaMallocHost((void**)&c->h_red, 64 * sizeof(double)));
     MPM_CUDA(cudaMallocHost((void**)&c->h_int, 64 * sizeof(int)));
@@ -188,9 +187,7 @@ extern "C" int mpm_destroy(mpm_ctx* c) {
   } catch (...) {
   }
   for (cudaEvent_t e : c->evpool) cudaEventDestroy(e);
-  if (c->d_err) cudaFreeAsync(c->d_err, c->stream);
   if (c->d_red) cudaFreeAsync(c->d_red, c->stream);
-  if (c->d_ticket) cudaFreeAsync(c->d_ticket, c->stream);
   cudaStreamSynchronize(c->stream);
   if (c->h_red) cudaFreeHost(c->h_red);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
@@ -469,7 +466,7 @@ extern "C" int mpm_assemble(mpm_ctx* c, const mpm_mesh* m, const mpm_material* m
     AsmOut o{};
     bool host_out = reaction || fint_norms;
     assemble(c, m, *mat, body ? *body : nob, du, load, precision, R, K, &o, host_out);
-    int st = check_device_error(c, "mpm_assemble");
+    int st = assembly_error(c, o, "mpm_assemble");
     if (st) return st;
     if (reaction)
       for (int d = 0; d < 3; ++d) reaction[d] = o.reaction[d];
@@ -496,7 +493,7 @@ extern "C" int mpm_assemble_body(mpm_ctx* c, const mpm_mesh* m, const mpm_materi
     dyn.Kbg = Kbg;
     AsmOut o{};
     assemble(c, m, *mat, *body, du, load, precision, R, K, &o, true, false, &dyn);
-    int st = check_device_error(c, "mpm_assemble_body");
+    int st = assembly_error(c, o, "mpm_assemble_body");
     if (st) return st;
     if (reaction)
       for (int d = 0; d < 3; ++d) reaction[d] = o.reaction[d];

@@ -158,8 +158,11 @@ struct mpm_ctx {
   cudaStream_t cap_stream = nullptr;  // private stream on which CUDA graphs are captured
   int device = 0;
   int coop_sms = 0;            // SMs, where cooperative launches are supported (else 0)
+  // device reduction slots (64 doubles).  Those of an assembly follow each other:
+  // the grid sums' ticket (14, 15), the norms (16-19), the reaction (20-22) and
+  // the error word (23), so that one memset starts them and one copy reads them
+  double* d_red = nullptr;
   int* d_err = nullptr;        // device error word
-  double* d_red = nullptr;     // device reduction slots (64 doubles)
   // fixed-order grid sums (mpm::GridRed): per-block partials and the ticket
   // that elects the last block; the ticket is zero between launches
   mpm::Buf part;
@@ -969,7 +972,13 @@ struct AsmOut {
   double reaction[3];
   double fint_norm, fextc_norm, finert_norm;
   double Rb[6], Kbb[36];  // a free body's residual and its derivative in q
+  bool clean;             // the error word came with the norms and was zero
 };
+// check_device_error after an assembly, without a second copy and
+// synchronisation where its norms brought a zero error word along
+inline int assembly_error(mpm_ctx* c, const AsmOut& o, const char* where) {
+  return o.clean ? (int)MPM_OK : check_device_error(c, where);
+}
 // a time step's inertia and a free body's equations: dt > 0 adds the Newmark
 // inertia (needs the build's point velocities); q is the body's increment;
 // with `body` the assembly forms the body's residual (AsmOut.Rb, with its

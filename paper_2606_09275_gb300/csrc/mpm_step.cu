@@ -140,7 +140,7 @@ void newton(mpm_ctx* c, mpm_mesh* m, const mpm_material* mat, const mpm_rigid& b
     tm.start();
     assemble(c, m, *mat, bd, du, prm->load, prec, R, nullptr, &o, true, false, dp);
     st.ms_assemble += tm.stop();
-    status = check_device_error(c, "assembly");
+    status = assembly_error(c, o, "assembly");
     if (status) throw CudaError(status, c->err);
     double rn = body_norm(sqrt(c->h_red[16]), o);
     bool conv = false;
@@ -218,7 +218,7 @@ void newton(mpm_ctx* c, mpm_mesh* m, const mpm_material* mat, const mpm_rigid& b
         AsmOut ot{};
         assemble(c, m, *mat, bd, trial, prm->load, prec, Rt, nullptr, &ot, true, false, dp ? &dt_ : nullptr);
         double r1 = body_norm(sqrt(c->h_red[16]), ot);
-        int es = check_device_error(c, "line search");
+        int es = assembly_error(c, ot, "line search");
         if (es) r1 = INFINITY;
         ilast = e;
         if (best < 0.0 || r1 < best) {
@@ -238,7 +238,7 @@ void newton(mpm_ctx* c, mpm_mesh* m, const mpm_material* mat, const mpm_rigid& b
         rn = best;
       } else {
         assemble(c, m, *mat, bd, du, prm->load, prec, R, nullptr, &o, true, false, dp);
-        status = check_device_error(c, "assembly");
+        status = assembly_error(c, o, "assembly");
         if (status) throw CudaError(status, c->err);
         rn = body_norm(sqrt(c->h_red[16]), o);
       }
