@@ -121,35 +121,51 @@ __device__ void tangent_rotate(const double* Q, const double* lam, const double*
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       int s = (i == j) ? i : (i + j == 1 ? 3 : (i + j == 3 ? 4 : 5));
-      taum[3 * i + j] = (R)tau6[s];
+      taum[3 * i + j] = v0 * (R)tau6[s];
     }
-  for (int i = 0; i < 3; ++i)
-    for (int k = 0; k < 3; ++k)
-      for (int m = 0; m < 3; ++m) {
-        R o[4];
+  // A_ijkm for a pair (k, m) is Q B Q^T, B symmetric in the eigenbasis: B_aa =
+  // sum_c d_ac q_kc q_mc, B_ac = theta_ac (lam_c q_ka q_mc + lam_a q_kc q_ma).
+  // Some 80 multiply-adds a pair, where the sums written out entry by entry took
+  // 750 (FP64: the law and this for the punch of depths 3 to 6 50 us, 96 so;
+  // this alone for the rolling sphere 28 and 71 us)
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          R s = (R)0;
+  for (int k = 0; k < 3; ++k)
 #pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            R qia = q[3 * i + a];
+    for (int m = 0; m < 3; ++m) {
+      R B[3][3];
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              s += d[3 * a + c] * qia * q[3 * j + a] * q[3 * k + c] * q[3 * m + c];
-              if (a != c)
-                s += th[3 * a + c] * qia * q[3 * j + c] *
-                     (lr[c] * q[3 * k + a] * q[3 * m + c] + lr[a] * q[3 * k + c] * q[3 * m + a]);
-            }
-          }
-          if (j == k) s -= taum[3 * i + m];
-          o[j] = v0 * s;
-        }
-        o[3] = (R)0;
-        st4(Aout + (i * 9 + k * 3 + m) * 4, o);
+      for (int a = 0; a < 3; ++a) {
+        R s = d[3 * a] * (q[3 * k] * q[3 * m]);
+        s += d[3 * a + 1] * (q[3 * k + 1] * q[3 * m + 1]);
+        s += d[3 * a + 2] * (q[3 * k + 2] * q[3 * m + 2]);
+        B[a][a] = v0 * s;
       }
+#pragma unroll
+      for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int c = a + 1; c < 3; ++c)
+          B[a][c] = B[c][a] = v0 * (th[3 * a + c] * (lr[c] * (q[3 * k + a] * q[3 * m + c]) +
+                                                     lr[a] * (q[3 * k + c] * q[3 * m + a])));
+      R o[3][4];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        R t[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) t[c] = q[3 * i] * B[0][c] + q[3 * i + 1] * B[1][c] + q[3 * i + 2] * B[2][c];
+#pragma unroll
+        for (int j = i; j < 3; ++j)
+          o[i][j] = o[j][i] = t[0] * q[3 * j] + t[1] * q[3 * j + 1] + t[2] * q[3 * j + 2];
+        o[i][3] = (R)0;
+      }
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        o[i][k] -= taum[3 * i + m];
+        st4(Aout + (i * 9 + k * 3 + m) * 4, o[i]);
+      }
+    }
 }
 
-template <bool TANGENT, class TA>
+template <bool TANGENT, class TA, bool SAVE = false>
 __device__ bool point_update_law(const Law& L, double E, double ys, const double* be, const double* dF,
                                  double* tau6, double* be_new, double V0, TA* Aout, double* save = nullptr) {
   double b[9] = {be[0], be[3], be[5], be[3], be[1], be[4], be[5], be[4], be[2]};
@@ -159,15 +175,12 @@ __device__ bool point_update_law(const Law& L, double E, double ys, const double
 #pragma unroll
     for (int j = 0; j < 3; ++j)
       t[3 * i + j] = dF[3 * i] * b[j] + dF[3 * i + 1] * b[3 + j] + dF[3 * i + 2] * b[6 + j];
+  // dF b dF^T is symmetric: its upper half
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j)
-      bt[3 * i + j] = t[3 * i] * dF[3 * j] + t[3 * i + 1] * dF[3 * j + 1] + t[3 * i + 2] * dF[3 * j + 2];
-  // symmetrise before the rotations
-  bt[1] = bt[3] = 0.5 * (bt[1] + bt[3]);
-  bt[2] = bt[6] = 0.5 * (bt[2] + bt[6]);
-  bt[5] = bt[7] = 0.5 * (bt[5] + bt[7]);
+    for (int j = i; j < 3; ++j)
+      bt[3 * i + j] = bt[3 * j + i] = t[3 * i] * dF[3 * j] + t[3 * i + 1] * dF[3 * j + 1] + t[3 * i + 2] * dF[3 * j + 2];
   double lam[3], Q[9];
   jacobi3(bt, lam, Q);
   if (!(lam[0] > 0.0 && lam[1] > 0.0 && lam[2] > 0.0) || !isfinite(lam[0] + lam[1] + lam[2]))
@@ -189,7 +202,7 @@ __device__ bool point_update_law(const Law& L, double E, double ys, const double
     be_new[s] = Q[3 * i] * bw[0] * Q[3 * j] + Q[3 * i + 1] * bw[1] * Q[3 * j + 1] + Q[3 * i + 2] * bw[2] * Q[3 * j + 2];
   }
   if (TANGENT) tangent_rotate<TA>(Q, lam, dd, gr, tau6, V0, Aout);
-  if (save) {
+  if constexpr (SAVE) {
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
       save[i] = Q[i];
@@ -208,8 +221,13 @@ __device__ inline double det3(const double* a) {
 }
 
 // also M = V0 tau dF^-T (row-major, 12 per point, the last 3 unused), so that
-// the internal force of support k is M grad S_k (k_residual_rows)
-template <bool TANGENT, class TA>
+// the internal force of support k is M grad S_k (k_residual_rows).  SAVE: the
+// spectral state for a tangent at the same increment (k_tangent_state), of use
+// to a Newton iteration only.  Bound by FP64 issue, some
+// 500 instructions a point: 1.9 M points take 1.73 ms (1.90 with the state always
+// saved, a division per principal direction and rotation, and all nine entries
+// of dF b dF^T), with the FP32 tangent 2.04 (2.51).
+template <bool TANGENT, class TA, bool SAVE>
 __global__ void k_constitutive(int P, Law L, const double* __restrict__ E, const double* __restrict__ ys,
                                const double* __restrict__ be, const double* __restrict__ dF,
                                const double* __restrict__ V0, double* tau, double* dFinv,
@@ -222,9 +240,8 @@ __global__ void k_constitutive(int P, Law L, const double* __restrict__ E, const
   double det = det3(f);
   double t6[6], bn[6];
   bool ok = det > 0.0 && isfinite(det) &&
-            point_update_law<TANGENT, TA>(L, E[w], ys[w], be + 6 * (size_t)w, f, t6, bn, V0[w],
-                                          Aalg + 108 * (size_t)w,
-                                          lawst ? lawst + 22 * (size_t)w : nullptr);
+            point_update_law<TANGENT, TA, SAVE>(L, E[w], ys[w], be + 6 * (size_t)w, f, t6, bn, V0[w],
+                                                Aalg + 108 * (size_t)w, lawst + 22 * (size_t)w);
   if (!ok) {
     atomicOr(err, EB_NAN);
 #pragma unroll
@@ -248,14 +265,16 @@ __global__ void k_constitutive(int P, Law L, const double* __restrict__ E, const
   double fi[9];
 #pragma unroll
   for (int e = 0; e < 9; ++e) fi[e] = o[e];
-  double tm[9] = {t6[0], t6[3], t6[5], t6[3], t6[1], t6[4], t6[5], t6[4], t6[2]};
-  double v0 = V0[w];
+  double v0 = V0[w], u6[6];
+#pragma unroll
+  for (int s = 0; s < 6; ++s) u6[s] = v0 * t6[s];
+  double tm[9] = {u6[0], u6[3], u6[5], u6[3], u6[1], u6[4], u6[5], u6[4], u6[2]};
   double* M = Mf + 12 * (size_t)w;
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int l = 0; l < 3; ++l)
-      M[3 * i + l] = v0 * (tm[3 * i] * fi[3 * l] + tm[3 * i + 1] * fi[3 * l + 1] + tm[3 * i + 2] * fi[3 * l + 2]);
+      M[3 * i + l] = tm[3 * i] * fi[3 * l] + tm[3 * i + 1] * fi[3 * l + 1] + tm[3 * i + 2] * fi[3 * l + 2];
 }
 
 // the tangent of the state the last residual evaluation left (same increment):
@@ -1579,7 +1598,7 @@ void body_out(mpm_ctx* c, const mpm_material& mat, const mpm_rigid& body, double
 
 void assemble(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const mpm_rigid& body,
               const double* du, double load, int precision, double* R, void* K, AsmOut* out,
-              bool want_norms, bool reuse, const Dyn* dyn) {
+              bool want_norms, bool reuse, const Dyn* dyn, bool save_state) {
   mpm_mesh* m = const_cast<mpm_mesh*>(mc);
   cudaStream_t st = c->stream;
   int P = m->np, nd = m->ndof;
@@ -1587,7 +1606,7 @@ void assemble(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const mpm
   double* dF = grow<double>(c, m->dF, 9 * (size_t)P);
   double* dFinv = grow<double>(c, m->dFinv, 9 * (size_t)P);
   double* tau = grow<double>(c, m->tau, 6 * (size_t)P);
-  double* lawst = grow<double>(c, m->lawst, 22 * (size_t)P);
+  double* lawst = save_state || reuse ? grow<double>(c, m->lawst, 22 * (size_t)P) : nullptr;
   double* Mf = grow<double>(c, m->Mf, 12 * (size_t)P);
   const int* nsup = ptr<int>(m->nsup);
   const int* sidx = ptr<int>(m->sidx);
@@ -1651,18 +1670,20 @@ void assemble(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const mpm
     }
   } else {
     MPM_LAUNCH_P(MPM_PROF_KINEMATICS, k_kinematics<<<grid_for(P, KIN_P), KIN_T, 0, st>>>(P, nsup, sidx, dS, du, dF));
-    if (!K)
-      MPM_LAUNCH_P(MPM_PROF_CONSTITUTIVE, k_constitutive<false, double><<<grid_for(P, 128), 128, 0, st>>>(
+    if (!K) {
+      auto kern = save_state ? k_constitutive<false, double, true> : k_constitutive<false, double, false>;
+      MPM_LAUNCH_P(MPM_PROF_CONSTITUTIVE, kern<<<grid_for(P, 128), 128, 0, st>>>(
           P, L, ptr<double>(m->pE), ptr<double>(m->pys), ptr<double>(m->pbe), dF, V0, tau, dFinv, Mf,
           nullptr, lawst, c->d_err));
+    }
     else if (mixed)
-      MPM_LAUNCH_P(MPM_PROF_CONSTITUTIVE, k_constitutive<true, float><<<grid_for(P, 128), 128, 0, st>>>(
+      MPM_LAUNCH_P(MPM_PROF_CONSTITUTIVE, (k_constitutive<true, float, false><<<grid_for(P, 128), 128, 0, st>>>(
           P, L, ptr<double>(m->pE), ptr<double>(m->pys), ptr<double>(m->pbe), dF, V0, tau, dFinv, Mf,
-          (float*)Aalg, nullptr, c->d_err));
+          (float*)Aalg, nullptr, c->d_err)));
     else
-      MPM_LAUNCH_P(MPM_PROF_CONSTITUTIVE, k_constitutive<true, double><<<grid_for(P, 128), 128, 0, st>>>(
+      MPM_LAUNCH_P(MPM_PROF_CONSTITUTIVE, (k_constitutive<true, double, false><<<grid_for(P, 128), 128, 0, st>>>(
           P, L, ptr<double>(m->pE), ptr<double>(m->pys), ptr<double>(m->pbe), dF, V0, tau, dFinv, Mf,
-          (double*)Aalg, nullptr, c->d_err));
+          (double*)Aalg, nullptr, c->d_err)));
     if (contact) MPM_CUDA(cudaMemsetAsync(fc, 0, sizeof(double) * 3 * nd, st));
     MPM_LAUNCH_P(MPM_PROF_RESIDUAL, k_residual_rows<<<grid_for(nd, 8), 256, 0, st>>>(
         nd, P, load, ptr<long long>(m->src_ptr), ptr<uint64_t>(m->src_key), Mf, dS, rp, col,

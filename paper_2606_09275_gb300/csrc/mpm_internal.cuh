@@ -995,7 +995,7 @@ struct Dyn {
 // left at the same increment (dF, tau and the spectral state); R untouched
 void assemble(mpm_ctx* c, const mpm_mesh* m, const mpm_material& mat, const mpm_rigid& body,
               const double* du, double load, int precision, double* R, void* K, AsmOut* out,
-              bool want_norms, bool reuse = false, const Dyn* dyn = nullptr);
+              bool want_norms, bool reuse = false, const Dyn* dyn = nullptr, bool save_state = false);
 double norm_free(mpm_ctx* c, const mpm_mesh* m, const double* R);
 void blocks_export(mpm_ctx* c, const mpm_mesh* m, const void* K, int precision, double* out);
 

@@ -138,7 +138,7 @@ void newton(mpm_ctx* c, mpm_mesh* m, const mpm_material* mat, const mpm_rigid& b
     };
     AsmOut o{};
     tm.start();
-    assemble(c, m, *mat, bd, du, prm->load, prec, R, nullptr, &o, true, false, dp);
+    assemble(c, m, *mat, bd, du, prm->load, prec, R, nullptr, &o, true, false, dp, true);
     st.ms_assemble += tm.stop();
     status = assembly_error(c, o, "assembly");
     if (status) throw CudaError(status, c->err);
@@ -216,7 +216,8 @@ void newton(mpm_ctx* c, mpm_mesh* m, const mpm_material* mat, const mpm_rigid& b
         dt_.Kgb = dt_.Kbg = nullptr;
         for (int j = 0; j < 6; ++j) dt_.q[j] = dyn.q[j] + etas[e] * dq[j];
         AsmOut ot{};
-        assemble(c, m, *mat, bd, trial, prm->load, prec, Rt, nullptr, &ot, true, false, dp ? &dt_ : nullptr);
+        assemble(c, m, *mat, bd, trial, prm->load, prec, Rt, nullptr, &ot, true, false, dp ? &dt_ : nullptr,
+                 true);
         double r1 = body_norm(sqrt(c->h_red[16]), ot);
         int es = assembly_error(c, ot, "line search");
         if (es) r1 = INFINITY;
@@ -237,7 +238,7 @@ void newton(mpm_ctx* c, mpm_mesh* m, const mpm_material* mat, const mpm_rigid& b
         o = obest;
         rn = best;
       } else {
-        assemble(c, m, *mat, bd, du, prm->load, prec, R, nullptr, &o, true, false, dp);
+        assemble(c, m, *mat, bd, du, prm->load, prec, R, nullptr, &o, true, false, dp, true);
         status = assembly_error(c, o, "assembly");
         if (status) throw CudaError(status, c->err);
         rn = body_norm(sqrt(c->h_red[16]), o);
