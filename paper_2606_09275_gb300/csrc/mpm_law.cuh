@@ -272,11 +272,10 @@ __device__ inline void principal_return(const Law& L, double E, double ys, const
   *gr = 2.0 * mu;
   if (L.model == 1) {
     // von Mises: q = sqrt(3/2)|s|, radial return onto q = ys
-    double c = 1.224744871391589 * 2.0 * mu, q = c * dn;
+    double q = 1.224744871391589 * 2.0 * mu * dn;
     if (q <= ys) return;
-    // one division (nine FP64 instructions) for ys / q and the direction dev / dn
-    double iq = 1.0 / q, g = 2.0 * mu * (ys * iq), id = c * iq;
-    double nn[3] = {dev[0] * id, dev[1] * id, dev[2] * id};
+    double fac = ys / q, g = 2.0 * mu * fac;
+    double nn[3] = {dev[0] / dn, dev[1] / dn, dev[2] / dn};
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       ta[a] = kb * tr + g * dev[a];
