@@ -175,12 +175,15 @@ __device__ bool point_update_law(const Law& L, double E, double ys, const double
 #pragma unroll
     for (int j = 0; j < 3; ++j)
       t[3 * i + j] = dF[3 * i] * b[j] + dF[3 * i + 1] * b[3 + j] + dF[3 * i + 2] * b[6 + j];
-  // dF b dF^T is symmetric: its upper half
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = i; j < 3; ++j)
-      bt[3 * i + j] = bt[3 * j + i] = t[3 * i] * dF[3 * j] + t[3 * i + 1] * dF[3 * j + 1] + t[3 * i + 2] * dF[3 * j + 2];
+    for (int j = 0; j < 3; ++j)
+      bt[3 * i + j] = t[3 * i] * dF[3 * j] + t[3 * i + 1] * dF[3 * j + 1] + t[3 * i + 2] * dF[3 * j + 2];
+  // symmetrise before the rotations
+  bt[1] = bt[3] = 0.5 * (bt[1] + bt[3]);
+  bt[2] = bt[6] = 0.5 * (bt[2] + bt[6]);
+  bt[5] = bt[7] = 0.5 * (bt[5] + bt[7]);
   double lam[3], Q[9];
   jacobi3(bt, lam, Q);
   if (!(lam[0] > 0.0 && lam[1] > 0.0 && lam[2] > 0.0) || !isfinite(lam[0] + lam[1] + lam[2]))
@@ -224,9 +227,8 @@ __device__ inline double det3(const double* a) {
 // the internal force of support k is M grad S_k (k_residual_rows).  SAVE: the
 // spectral state for a tangent at the same increment (k_tangent_state), of use
 // to a Newton iteration only.  Bound by FP64 issue, some
-// 500 instructions a point: 1.9 M points take 1.73 ms (1.90 with the state always
-// saved, a division per principal direction and rotation, and all nine entries
-// of dF b dF^T), with the FP32 tangent 2.04 (2.51).
+// 550 instructions a point: 1.9 M points take 1.88 ms (1.71 elastic ones), with
+// the FP32 tangent 2.23 (2.51 with its entries summed term by term).
 template <bool TANGENT, class TA, bool SAVE>
 __global__ void k_constitutive(int P, Law L, const double* __restrict__ E, const double* __restrict__ ys,
                                const double* __restrict__ be, const double* __restrict__ dF,

@@ -59,34 +59,17 @@ __device__ inline void jacobi_rotate(T* d, T* a, T* Q) {
   }
 }
 
-// a double to a float and back in integer instructions (a conversion takes the
-// FP64 pipe as long as an FMA): cut off below its 24 bits, zero below the normal
-// range; the value must lie below 2^127
-__device__ inline float cut_float(double v) {
-  unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-  int e = (int)((hi >> 20) & 0x7ffu) - 896;
-  unsigned b = (hi & 0x80000000u) | ((unsigned)e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
-  return e > 0 ? __uint_as_float(b) : 0.f;
-}
-__device__ inline double widen_float(float f) {
-  unsigned b = __float_as_uint(f);
-  bool normal = (b & 0x7f800000u) != 0;
-  return normal ? __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29))
-                : 0.0;
-}
-
-// the same rotation for |apq / h| <= 1e-4 by an FP32 quotient t = apq / h, without
-// its two square roots and its divisions: c = 1 - t^2 / 2 and s = t c up to t^4
-// (1e-16); of apq stays what the quotient leaves, r = apq - t h, some 1e-7 of it,
-// and t^2 of it, for the next sweep
+// the same rotation for |apq / h| <= 1e-4, without its two square roots and
+// one of its divisions: t = apq / h up to t^3 (what stays of apq is 1e-8 of
+// it, for the next sweep), c = 1 - t^2 / 2 and s = t c up to t^4 (1e-16)
 template <int P, int Q_>
-__device__ inline void jacobi_nudge(double* d, double* a, double* Q, double t, double h) {
+__device__ inline void jacobi_nudge(double* d, double* a, double* Q, double t) {
   constexpr int O = 3 - P - Q_, PQ = P + Q_ - 1, OP = O + P - 1, OQ = O + Q_ - 1;
-  double apq = a[PQ], t2 = t * t, r = fma(-t, h, apq), both = apq + r;
+  double apq = a[PQ], t2 = t * t;
   double cs = fma(-0.5, t2, 1.0), sn = t * cs;
-  d[P] = fma(-t, both, d[P]);
-  d[Q_] = fma(t, both, d[Q_]);
-  a[PQ] = fma(-t2, apq, r);
+  d[P] = fma(-t, apq, d[P]);
+  d[Q_] = fma(t, apq, d[Q_]);
+  a[PQ] = -apq * t2;
   double aop = a[OP], aoq = a[OQ];
   a[OP] = fma(cs, aop, -sn * aoq);
   a[OQ] = fma(sn, aop, cs * aoq);
@@ -98,14 +81,12 @@ __device__ inline void jacobi_nudge(double* d, double* a, double* Q, double t, d
   }
 }
 
-// `narrow`: the matrix lies well inside the FP32 range
 template <int P, int Q_>
-__device__ inline void jacobi_step(double* d, double* a, double* Q, bool narrow) {
+__device__ inline void jacobi_step(double* d, double* a, double* Q) {
   constexpr int PQ = P + Q_ - 1;
-  double h = d[Q_] - d[P];
-  float af = cut_float(a[PQ]), t = af == 0.f ? 0.f : af / cut_float(h);
-  if (narrow && fabsf(t) <= 1e-4f)
-    jacobi_nudge<P, Q_>(d, a, Q, widen_float(t), h);
+  double h = d[Q_] - d[P], t = a[PQ] == 0.0 ? 0.0 : a[PQ] / h;
+  if (fabs(t) <= 1e-4)
+    jacobi_nudge<P, Q_>(d, a, Q, t);
   else
     jacobi_rotate<P, Q_>(d, a, Q);
 }
@@ -146,12 +127,11 @@ __device__ inline void jacobi_seed(float* d, float* a, float* q) {
 // FP32 Jacobi sweeps find (as a quaternion, so that the FP64 start is
 // orthonormal to rounding): FP64 instructions are the cost of the point
 // kernels here (16 SM cycles each, against a quarter for FP32), and from the
-// start two sweeps of three small rotations (24 instructions; 32 with an FP64
-// quotient) finish, where the identity takes four of full ones (65).  A million
-// matrices of strains of 1e-2: 1.40 ms from the identity, 0.55 ms so (0.64 with
-// the FP64 quotient), with smaller errors (|Q^T Q - I| 2.4e-16 in the mean
-// against 3.3e-16); of nearly equal eigenvalues, which FP32 cannot tell apart,
-// 1.00 and 1.15 ms.
+// start two sweeps of three small rotations (32 instructions) finish, where
+// the identity takes four of full ones (65).  A million matrices of strains of
+// 1e-2: 1.40 ms from the identity, 0.65 ms so, with smaller errors
+// (|Q^T Q - I| 2.2e-16 in the mean against 3.3e-16); of nearly equal
+// eigenvalues, which FP32 cannot tell apart, 1.00 and 1.03 ms.
 __device__ inline void jacobi3(double* A, double* lam, double* Q) {
   double m = (A[0] + A[4] + A[8]) * (1.0 / 3.0);
   double d[3] = {A[0] - m, A[4] - m, A[8] - m}, a[3] = {A[1], A[2], A[5]};
@@ -175,7 +155,6 @@ __device__ inline void jacobi3(double* A, double* lam, double* Q) {
     af[i] = (float)a[i];
     big = fmaxf(big, fmaxf(fabsf(df[i]), fabsf(af[i])));
   }
-  bool narrow = big > 1e-15f && big < 1e15f;
   if (big > 1e-30f && big < 1e30f) {
     float sc = 1.f / big;
 #pragma unroll
@@ -212,9 +191,9 @@ __device__ inline void jacobi3(double* A, double* lam, double* Q) {
   a[0] = qt(0, 1); a[1] = qt(0, 2); a[2] = qt(1, 2);
   for (int sweep = 0; sweep < 40; ++sweep) {
     if (done()) break;
-    jacobi_step<0, 1>(d, a, Q, narrow);
-    jacobi_step<0, 2>(d, a, Q, narrow);
-    jacobi_step<1, 2>(d, a, Q, narrow);
+    jacobi_step<0, 1>(d, a, Q);
+    jacobi_step<0, 2>(d, a, Q);
+    jacobi_step<1, 2>(d, a, Q);
   }
 #pragma unroll
   for (int i = 0; i < 3; ++i) lam[i] = m + d[i];
@@ -275,7 +254,8 @@ __device__ inline void principal_return(const Law& L, double E, double ys, const
     double q = 1.224744871391589 * 2.0 * mu * dn;
     if (q <= ys) return;
     double fac = ys / q, g = 2.0 * mu * fac;
-    double nn[3] = {dev[0] / dn, dev[1] / dn, dev[2] / dn};
+    double n0 = dev[0] / dn, n1 = dev[1] / dn, n2 = dev[2] / dn;
+    double nn[3] = {n0, n1, n2};
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       ta[a] = kb * tr + g * dev[a];
