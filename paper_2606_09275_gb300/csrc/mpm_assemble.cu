@@ -348,7 +348,8 @@ __global__ void k_dS_to_float(int P, const int* __restrict__ nsup, const double*
 // 6 additions for the three sums over the lanes, and the ghost term only where
 // the row has one (its coefficients are tested as integers).  Indentation,
 // 1.9 M points: 1.85 ms with six shuffle trees of 5 additions and an FP64
-// compare per block, 1.21 so.
+// compare per block, 1.20 so, 1.03 with the loads of two sources of a lane under
+// way at once (of four 1.17).
 __device__ inline double sum3_scatter(double f0, double f1, double f2, int lane) {
   // lane 0 ends with the sum of f0 over the warp, lane 16 of f1, lane 8 of f2
   bool up = lane & 16;
@@ -361,6 +362,8 @@ __device__ inline double sum3_scatter(double f0, double f1, double f2, int lane)
   return a + __shfl_xor_sync(0xffffffffu, a, 1);
 }
 
+constexpr int RS = 2;
+
 __global__ void k_residual_rows(int nd, int P, double load, const long long* __restrict__ sptr,
                                 const uint64_t* __restrict__ skeys, const double* __restrict__ M,
                                 const double* __restrict__ dS, const int* __restrict__ rp,
@@ -371,17 +374,31 @@ __global__ void k_residual_rows(int nd, int P, double load, const long long* __r
   if (r >= nd) return;
   double f0 = 0.0, f1 = 0.0, f2 = 0.0;
   long long q1 = sptr[r + 1];
-  for (long long q = sptr[r] + lane; q < q1; q += 32) {
-    uint32_t sid = (uint32_t)skeys[q];
-    int w = (int)(sid >> 6), k = (int)(sid & 63);
-    if (w >= P) continue;  // ghost-face source
-    const double2* m = reinterpret_cast<const double2*>(M + 12 * (size_t)w);
-    double2 m01 = m[0], m23 = m[1], m45 = m[2], m67 = m[3], m8x = m[4];
-    const double* a = dS + 3 * ((size_t)w * MAXS + k);
-    double a0 = a[0], a1 = a[1], a2 = a[2];
-    f0 = fma(m23.x, a2, fma(m01.y, a1, fma(m01.x, a0, f0)));
-    f1 = fma(m45.y, a2, fma(m45.x, a1, fma(m23.y, a0, f1)));
-    f2 = fma(m8x.x, a2, fma(m67.y, a1, fma(m67.x, a0, f2)));
+  // RS sources of a lane at a time, all their loads under way before the sums
+  for (long long q = sptr[r] + lane; q < q1; q += 32 * RS) {
+    double2 m[RS][5];
+    double a[RS][3];
+    bool on[RS];
+#pragma unroll
+    for (int u = 0; u < RS; ++u) {
+      uint32_t sid = q + 32 * u < q1 ? (uint32_t)skeys[q + 32 * u] : 0xffffffffu;
+      int w = (int)(sid >> 6), k = (int)(sid & 63);
+      on[u] = w < P;  // else a ghost-face source
+      if (!on[u]) continue;
+      const double2* mp = reinterpret_cast<const double2*>(M + 12 * (size_t)w);
+      const double* ap = dS + 3 * ((size_t)w * MAXS + k);
+#pragma unroll
+      for (int i = 0; i < 5; ++i) m[u][i] = mp[i];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) a[u][i] = ap[i];
+    }
+#pragma unroll
+    for (int u = 0; u < RS; ++u) {
+      if (!on[u]) continue;
+      f0 = fma(m[u][1].x, a[u][2], fma(m[u][0].y, a[u][1], fma(m[u][0].x, a[u][0], f0)));
+      f1 = fma(m[u][2].y, a[u][2], fma(m[u][2].x, a[u][1], fma(m[u][1].y, a[u][0], f1)));
+      f2 = fma(m[u][4].x, a[u][2], fma(m[u][3].y, a[u][1], fma(m[u][3].x, a[u][0], f2)));
+    }
   }
   double g0 = 0.0, g1 = 0.0, g2 = 0.0;
   bool ghost = false;
