@@ -1052,9 +1052,9 @@ __global__ void k_src_ptr(long long n, const uint64_t* __restrict__ keys, int nd
 
 // Block pattern: the columns of row r are the union of the supports of every
 // source (point or ghost face) touching r.  One warp per row collects them in
-// a hash set in shared memory and ranks them.  What bounds it is the latency
-// of the chain key -> support -> insertion over some 200 sources a row, and the
-// insertions' shared-memory traffic.  So a warp takes 32 keys and support sizes
+// a hash set in shared memory and ranks them.  Taken source by source it
+// waits on the chain key -> support -> insertion, some 200 times a row; so a warp
+// takes 32 keys and support sizes
 // at once, 8 supports in flight, and reads a slot before it tries to claim it
 // (some 40 of 41 insertions find their column there).  Rows of at most PSHORT
 // columns (125 where the leaf size does not change) use a set of 512 slots
@@ -1062,7 +1062,8 @@ __global__ void k_src_ptr(long long n, const uint64_t* __restrict__ keys, int nd
 // their sorted columns in a staging row, which a copy takes to its place once
 // the row lengths are known; the others are collected again then, by the kernel
 // with the large set.  Two traversals, source by source, of a 2048-slot set took
-// 2 x 5.63 ms for 260 k rows and 51 M sources; now 2.10 ms and the copy 0.08 ms.
+// 2 x 5.63 ms for 260 k rows and 51 M sources; now 2.10 ms, bound by
+// instruction issue (87 % of the slots), and the copy 0.08 ms.
 constexpr int PSHORT = 256;            // longest row of the small set, and a staging row
 constexpr int PHASH = 2 * PSHORT;      // its slots
 constexpr int PPROBE = 64;             // its longest probe sequence; a row beyond it is a long one
