@@ -59,6 +59,10 @@ __device__ inline unsigned long long rk_ld_acquire(const unsigned long long* p) 
 __device__ inline void rk_st(unsigned long long* p, unsigned long long v) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
+__device__ inline void rk_st_release(unsigned long long* p, unsigned long long v) {
+  asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ inline void rk_fence() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
 // loads of a vector that other SMs write during the launch (past the L1)
 __device__ inline void ld4_cg(const float* p, float* v) {
@@ -105,6 +109,13 @@ struct RkShared {
 // shows that they were read), the coordinator its message when the next sum
 // is complete; a set comes round again RK_NBUF sums later, and at least every
 // third sum is fenced, so nobody meets a stale value.
+//
+// A fenced sum hands the vectors that the blocks stored before it to all of
+// them: every worker fences and posts slot 0 (release); the coordinator's lanes
+// that saw the slots fence (acquire) and meet at its barrier; each lane that
+// answers stores the second word of its message with release, which covers
+// what the other lanes saw; the workers load that word with acquire and meet
+// at their barrier.
 struct RkGrid {
   unsigned long long* slot;
   int G, me, k;
@@ -141,7 +152,7 @@ __device__ inline void rk_sum(RkGrid& g, RkShared& sh, const double* v, int n, b
   }
   __syncthreads();
   if (w < NV) {
-    if (fence && t == 0) __threadfence();
+    if (fence && t == 0) rk_fence();
     double s = l < n ? sh.red[w][l] : 0.0;
     for (int j = l + 32; j < n; j += 32) s += sh.red[w][j];
     for (int o = n > 16 ? 16 : n > 8 ? 8 : n > 4 ? 4 : n > 2 ? 2 : n > 1 ? 1 : 0; o > 0; o >>= 1)
@@ -203,7 +214,7 @@ __device__ inline bool rk_collect(const RkGrid& g, RkShared& sh, double* s, bool
       for (int h = 0; h < PU; ++h)
         if (h == 0 || 32 * h < W) x += __longlong_as_double((long long)u[h]);
     }
-    if (fence && w == 0) __threadfence();
+    if (fence && w == 0) rk_fence();
     x = warp_sum(x);
     late = __any_sync(0xffffffffu, late);
     if (l == 0) {
@@ -221,20 +232,23 @@ __device__ inline bool rk_collect(const RkGrid& g, RkShared& sh, double* s, bool
   return ok;
 }
 
-// coordinator: the answer to the sum just collected (stop: 0 go on, else the
-// code the workers find in sh.stop)
-__device__ inline void rk_tell(RkGrid& g, double a, double b, int stop) {
+// coordinator: the answer to the sum just collected, `fence` as there (stop: 0
+// go on, else the code the workers find in sh.stop)
+__device__ inline void rk_tell(RkGrid& g, double a, double b, int stop, bool fence) {
   const int t = threadIdx.x;
   if (t < RK_COPY) {
     unsigned long long* m = g.msg(g.k, t);
     rk_st(m, rk_pack(a));
-    rk_st(m + 1, stop ? RK_STOP | (unsigned long long)stop : rk_pack(b));
+    unsigned long long w = stop ? RK_STOP | (unsigned long long)stop : rk_pack(b);
+    if (fence)
+      rk_st_release(m + 1, w);
+    else
+      rk_st(m + 1, w);
     if (g.k > 0) {
       unsigned long long* o = g.msg(g.k + RK_NBUF - 1, t);
       rk_st(o, RK_EMPTY);
       rk_st(o + 1, RK_EMPTY);
     }
-    __threadfence();
   }
   __syncwarp();
   ++g.k;
@@ -454,19 +468,19 @@ __global__ void __launch_bounds__(RK_T, 1)
     double rz = s[0], rr = s[1], bb = s[1], thr = tol * tol * bb;
     bool conv = bb == 0.0, bad = !ok;
     int iters = 0;
-    rk_tell(g, 0.0, 0.0, conv || bad);
+    rk_tell(g, 0.0, 0.0, conv || bad, true);
     while (!conv && !bad && iters < maxit) {
       double irz = 1.0 / rz;  // ready before the sum it divides
       ok = rk_collect<1>(g, sh, s, false);
       bad = !ok || !rk_positive(s[0]);
-      rk_tell(g, rz / s[0], 0.0, bad);
+      rk_tell(g, rz / s[0], 0.0, bad, false);
       if (bad) break;
       ok = rk_collect<2>(g, sh, s, true);
       rr = s[1];
       ++iters;
       bad = !ok || !rk_finite(rr);
       conv = rk_at_most(rr, thr);
-      rk_tell(g, s[0] * irz, 0.0, conv || bad || iters >= maxit);
+      rk_tell(g, s[0] * irz, 0.0, conv || bad || iters >= maxit, true);
       rz = s[0];
     }
     if (t == 0) {
@@ -561,41 +575,41 @@ __global__ void __launch_bounds__(RK_T, 1)
     // the coordinator
     if (t >= RK_CT) return;
     double s[2];
-    bool ok = rk_collect<1>(g, sh, s, false);
+    bool ok = rk_collect<1>(g, sh, s, true);
     double bb = s[0], rr = bb, thr = tol * tol * bb, rho1 = bb;
     bool conv = bb == 0.0, bad = !ok;
     int it = 0;
     // beta (times p - omega v = 0 at the start) and omega
-    rk_tell(g, bb, 1.0, conv || bad);
+    rk_tell(g, bb, 1.0, conv || bad, true);
     while (!conv && !bad && it < maxit) {
       ++it;
       ok = rk_collect<1>(g, sh, s, true);  // ph is there
       bad = !ok;
-      rk_tell(g, 0.0, 0.0, bad);
+      rk_tell(g, 0.0, 0.0, bad, true);
       if (bad) break;
       double irho = 1.0 / rho1;
       ok = rk_collect<1>(g, sh, s, false);  // r0.v
       bad = !ok || !rk_finite(s[0]) || s[0] == 0.0;
       double alpha = rho1 / s[0];
-      rk_tell(g, alpha, 0.0, bad);
+      rk_tell(g, alpha, 0.0, bad, false);
       if (bad) break;
       ok = rk_collect<1>(g, sh, s, true);  // s.s
       conv = ok && rk_at_most(s[0], thr);
       bad = !ok;
-      rk_tell(g, alpha, 0.0, bad ? 1 : conv ? 2 : 0);
+      rk_tell(g, alpha, 0.0, bad ? 1 : conv ? 2 : 0, true);
       if (conv) rr = s[0];
       if (bad || conv) break;
       ok = rk_collect<2>(g, sh, s, false);  // t.s, t.t
       double omega = rk_positive(s[1]) ? s[0] / s[1] : 0.0;
       bad = !ok;
-      rk_tell(g, alpha, omega, bad);
+      rk_tell(g, alpha, omega, bad, false);
       if (bad) break;
       double f = irho * (alpha / omega);
       ok = rk_collect<2>(g, sh, s, false);  // r.r, r0.r
       rr = s[0];
       conv = rk_at_most(rr, thr);
       bad = !ok || (!conv && (!(omega != 0.0) || !rk_finite(rr)));
-      rk_tell(g, s[1] * f, omega, conv || bad || it >= maxit);
+      rk_tell(g, s[1] * f, omega, conv || bad || it >= maxit, false);
       rho1 = s[1];
     }
     if (t == 0) {

@@ -1,0 +1,31 @@
+"""The exchange between the blocks of the one-launch Krylov solves.
+
+A solve of one launch hands its vectors from block to block through grid sums;
+a block that met an older value of another block's rows would change the
+iterates.  Many solves of the same system therefore have to agree bit for bit,
+on a mesh of short iterations (the exchange is all of the time) and on one
+whose blocks keep K in global memory.
+"""
+import numpy as np
+import pytest
+
+from test_gpu_resident_solve import system  # noqa: F401  (fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("key", ["few_quads", "punch", "block_13k"])
+@pytest.mark.parametrize("method,precision", [(1, 0), (1, 1), (2, 0), (2, 1)])
+def test_every_solve_meets_the_same_vectors(system, key, method, precision):  # noqa: F811
+    s = system(key)
+    mpm, torch = s["mpm"], s["torch"]
+    cfg = dict(s["cfg"], mu=0.3, contact=1) if method == 2 else s["cfg"]
+    K = s["Kd"].float() if precision else s["Kd"]
+    rhs = torch.from_numpy(s["b"]).cuda()
+    run = lambda: mpm.solve(s["ctx"], s["mesh"], cfg, K, rhs, precision=precision, tol=1e-8, maxit=5000,  # noqa: E731
+                            method=method, inner_tol=1e-4)
+    x, st = run()
+    for _ in range(25):
+        y, st2 = run()
+        assert st2 == st and torch.equal(x, y)
+    assert np.isfinite(x.cpu().numpy()).all()
