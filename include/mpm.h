@@ -424,6 +424,11 @@ int mpm_profile(mpm_ctx* ctx, int enable);
 int mpm_profile_read(mpm_ctx* ctx, long long* launches, double* ms);
 int mpm_launch_count(const mpm_ctx* ctx, long long* launches);
 
+/* Bound of the waits between the blocks of a Krylov solve that runs as one
+ * launch, in polls of a word in device memory (0: the default, about a second).
+ * A solve whose wait runs out returns MPM_ERR_KRYLOV; the context stays usable. */
+int mpm_wait_limit(mpm_ctx* ctx, int polls);
+
 /* Measured FP64 fused multiply-add throughput of the context's GPU (no
  * counterpart in the paper; the roofline of the kernels that the precision
  * pattern keeps in FP64): independent FMA chains on every SM, timed with CUDA

@@ -95,6 +95,16 @@ extern "C" int mpm_profile_read(mpm_ctx* c, long long* launches, double* ms) {
   return MPM_OK;
 }
 
+extern "C" int mpm_wait_limit(mpm_ctx* c, int polls) {
+  if (!c) return MPM_ERR_ARG;
+  if (polls < 0) {
+    set_error(c, "mpm_wait_limit: a limit is not negative (0: the default)");
+    return MPM_ERR_ARG;
+  }
+  c->wait_polls = polls;
+  return MPM_OK;
+}
+
 extern "C" int mpm_launch_count(const mpm_ctx* c, long long* n) {
   if (!c || !n) return MPM_ERR_ARG;
   *n = c->nlaunch;

@@ -84,7 +84,8 @@ struct Scal {
   double rz[3], pq[3], rr[3];
   double bb, thr;    // ||b||^2 and tol^2 ||b||^2
   double a[8];       // BiCGStab scalars
-  int done, iters, breakdown, pad;
+  int done, iters, breakdown;
+  int late;         // a wait between the blocks of a one-launch solve ran out
 };
 
 // storage of a fixed-order grid sum (grid_sum below)
@@ -158,6 +159,7 @@ struct mpm_ctx {
   cudaStream_t cap_stream = nullptr;  // private stream on which CUDA graphs are captured
   int device = 0;
   int coop_sms = 0;            // SMs, where cooperative launches are supported (else 0)
+  int wait_polls = 0;          // bound of a wait between blocks (mpm_wait_limit; 0: the default)
   // device reduction slots (64 doubles).  Those of an assembly follow each other:
   // the grid sums' ticket (14, 15), the norms (16-19), the reaction (20-22) and
   // the error word (23), so that one memset starts them and one copy reads them

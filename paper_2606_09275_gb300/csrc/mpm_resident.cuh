@@ -30,7 +30,7 @@ constexpr int RK_QUADS = RK_T / 4;  // quads of storage rows worked on at a time
 constexpr int RK_NBUF = 6;          // rotating sets of sum slots and messages
 constexpr int RK_NV = 2;            // values per grid sum
 constexpr int RK_COPY = 16;         // copies of a message, a line each
-constexpr int RK_POLLS = 1 << 21;   // bound of a wait (about a second; then the solve fails)
+constexpr int RK_POLLS = 1 << 21;   // bound of a wait unless the context sets another (about a second)
 constexpr int RK_ROW = 64;          // slots' worth of a quad's own vector work
 
 // slots of a launch of G blocks: the sums' partials, then the messages
@@ -80,6 +80,7 @@ struct RkPlan {
   int rows;           // most rows of a worker
   int groups;         // most groups of 4 blocks x 4 rows of a worker, if K is kept in shared memory (else 0)
   int smem;           // dynamic shared memory
+  int polls;          // bound of a wait; one that runs out sets Scal::late, and the call fails
 };
 
 // elements of a group of 16 blocks in shared memory, padded so that the quad
@@ -118,7 +119,8 @@ struct RkShared {
 // at their barrier.
 struct RkGrid {
   unsigned long long* slot;
-  int G, me, k;
+  int* late;
+  int G, me, polls, k;
   __device__ unsigned long long* part(int k_) const {
     return slot + (size_t)(k_ % RK_NBUF) * RK_NV * G;
   }
@@ -166,14 +168,16 @@ __device__ inline void rk_sum(RkGrid& g, RkShared& sh, const double* v, int n, b
         }
         const unsigned long long* m = g.msg(g.k, g.me % RK_COPY);
         unsigned long long a = RK_EMPTY, b = RK_EMPTY;
-        for (int p = 0; p < RK_POLLS; ++p) {
+        for (int p = 0; p < g.polls; ++p) {
           a = rk_ld(m);
           b = fence ? rk_ld_acquire(m + 1) : rk_ld(m + 1);
           if (a != RK_EMPTY && b != RK_EMPTY) break;
         }
         sh.scal[0] = __longlong_as_double((long long)a);
         sh.scal[1] = __longlong_as_double((long long)b);
-        sh.stop = a == RK_EMPTY || b == RK_EMPTY ? 1 : (b >> 4) == (RK_STOP >> 4) ? (int)(b & 15) : 0;
+        bool none = a == RK_EMPTY || b == RK_EMPTY;
+        if (none) *g.late = 1;  // this block leaves with its rows as they are
+        sh.stop = none ? 1 : (b >> 4) == (RK_STOP >> 4) ? (int)(b & 15) : 0;
       }
     }
   }
@@ -205,7 +209,7 @@ __device__ inline bool rk_collect(const RkGrid& g, RkShared& sh, double* s, bool
 #pragma unroll
         for (int h = 0; h < PU; ++h) all = all && u[h] != RK_EMPTY;
         if (all) break;
-        if (n >= RK_POLLS) {
+        if (n >= g.polls) {
           late = true;
           break;
         }
@@ -229,6 +233,7 @@ __device__ inline bool rk_collect(const RkGrid& g, RkShared& sh, double* s, bool
     s[i] = sh.red[i][g.k & 1];
     ok = ok && __double_as_longlong(sh.red[i][2 + (g.k & 1)]) == 0;
   }
+  if (!ok && t == 0) *g.late = 1;
   return ok;
 }
 
@@ -459,7 +464,7 @@ __global__ void __launch_bounds__(RK_T, 1)
   __shared__ RkShared sh;
   __shared__ T sy[3][RK_T];
   const int t = threadIdx.x;
-  RkGrid g{slots, pl.G, (int)blockIdx.x, 0};
+  RkGrid g{slots, &sc->late, pl.G, (int)blockIdx.x, pl.polls, 0};
   if (g.me == g.G - 1) {
     // the coordinator
     if (t >= RK_CT) return;
@@ -570,7 +575,7 @@ __global__ void __launch_bounds__(RK_T, 1)
   __shared__ RkShared sh;
   __shared__ T sy[3][RK_T];
   const int t = threadIdx.x;
-  RkGrid g{slots, pl.G, (int)blockIdx.x, 0};
+  RkGrid g{slots, &sc->late, pl.G, (int)blockIdx.x, pl.polls, 0};
   if (g.me == g.G - 1) {
     // the coordinator
     if (t >= RK_CT) return;

@@ -508,6 +508,7 @@ RkPlan resident_plan(const mpm_ctx* c, const mpm_mesh* m, int nv) {
   if (state > SMEM) return p;
   if (state + kept <= SMEM) p.groups = groups;
   p.smem = (int)(state + (p.groups ? kept : 0));
+  p.polls = c->wait_polls > 0 ? c->wait_polls : RK_POLLS;
   p.G = W + 1;
   return p;
 }
@@ -537,6 +538,11 @@ int run_resident(mpm_ctx* c, bool* ran, void (*kern)(A...), const RkPlan& pl, un
   MPM_COUNT(c);
   MPM_CUDA(cudaMemcpyAsync(sc_h, sc_d, sizeof(Scal), cudaMemcpyDeviceToHost, st));
   MPM_CUDA(cudaStreamSynchronize(st));
+  if (sc_h->late) {
+    // some blocks left before the others: x is not that of any iteration
+    MPM_CUDA(cudaMemsetAsync(c->d_err, 0, sizeof(int), st));
+    throw CudaError(MPM_ERR_KRYLOV, "Krylov solve: a wait between the blocks of its launch ran out");
+  }
   *iters = 0;
   *relres = 0.0;
   if (sc_h->bb == 0.0 && !sc_h->breakdown) return MPM_OK;

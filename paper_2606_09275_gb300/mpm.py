@@ -28,7 +28,8 @@ EXPORT = dict(leaf_level=0, leaf_anchor=1, node_coord=2, node_hang=3, node_dof=4
 SYMBOLS = ["mpm_create", "mpm_destroy", "mpm_last_error", "mpm_octree_build", "mpm_mesh_free",
            "mpm_mesh_counts", "mpm_mesh_export", "mpm_assemble", "mpm_solve", "mpm_step",
            "mpm_profile", "mpm_profile_read", "mpm_launch_count", "mpm_solve_static",
-           "mpm_blocks_export", "mpm_adjoint", "mpm_fp64_peak", "mpm_assemble_body"]
+           "mpm_blocks_export", "mpm_adjoint", "mpm_fp64_peak", "mpm_assemble_body",
+           "mpm_wait_limit"]
 
 
 class Domain(C.Structure):
@@ -137,6 +138,7 @@ def lib():
         L.mpm_profile_read.argtypes = [vp, vp, vp]
         L.mpm_launch_count.argtypes = [vp, vp]
         L.mpm_fp64_peak.argtypes = [vp, d, vp, vp]
+        L.mpm_wait_limit.argtypes = [vp, i]
         L.mpm_assemble_body.argtypes = [vp, vp, C.POINTER(Material), C.POINTER(Rigid), vp, vp, d, d,
                                         i, vp, vp, vp, vp, vp, vp, vp, vp]
         L.mpm_adjoint.argtypes = [vp, C.POINTER(Domain), C.POINTER(Rigid), C.POINTER(Adapt),

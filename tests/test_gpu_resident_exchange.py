@@ -29,3 +29,28 @@ def test_every_solve_meets_the_same_vectors(system, key, method, precision):  # 
         y, st2 = run()
         assert st2 == st and torch.equal(x, y)
     assert np.isfinite(x.cpu().numpy()).all()
+
+
+@pytest.mark.parametrize("method,precision", [(1, 0), (1, 1), (2, 0), (2, 1)])
+def test_a_wait_that_runs_out_is_an_error(system, method, precision):  # noqa: F811
+    # with one poll a wait ends before the other blocks can have answered: every
+    # block leaves and the call says so; the next solve on the context is the usual one
+    s = system("punch")
+    mpm, torch = s["mpm"], s["torch"]
+    cfg = dict(s["cfg"], mu=0.3, contact=1) if method == 2 else s["cfg"]
+    K = s["Kd"].float() if precision else s["Kd"]
+    rhs = torch.from_numpy(s["b"]).cuda()
+    ctx = s["ctx"]
+    run = lambda: mpm.solve(ctx, s["mesh"], cfg, K, rhs, precision=precision, tol=1e-8, maxit=5000,  # noqa: E731
+                            method=method, inner_tol=1e-4)
+    x, st = run()
+    ctx.check(mpm.lib().mpm_wait_limit(ctx.h, 1))
+    try:
+        with pytest.raises(mpm.MPMError) as e:
+            run()
+    finally:
+        ctx.check(mpm.lib().mpm_wait_limit(ctx.h, 0))
+    assert e.value.code == 4 and "wait" in str(e.value)
+    y, st2 = run()
+    assert st2 == st and torch.equal(x, y)
+    assert mpm.lib().mpm_wait_limit(ctx.h, -1) == 1
