@@ -128,7 +128,9 @@ extern "C" int mpm_create(mpm_ctx** out, void* stream) {
   try {
     c->stream = (cudaStream_t)stream;
     MPM_CUDA(cudaGetDevice(&c->device));
-    int coop = 0;
+    int coop = 0, l2 = 0;
+    MPM_CUDA(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, c->device));
+    c->l2_bytes = l2;
     MPM_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device));
     if (coop) MPM_CUDA(cudaDeviceGetAttribute(&c->coop_sms, cudaDevAttrMultiProcessorCount, c->device));
     MPM_CUDA(cudaMallocAsync((void**)&c->d_red, 64 * sizeof(double), c->stream));

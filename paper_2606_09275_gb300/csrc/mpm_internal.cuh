@@ -159,6 +159,7 @@ struct mpm_ctx {
   cudaStream_t cap_stream = nullptr;  // private stream on which CUDA graphs are captured
   int device = 0;
   int coop_sms = 0;            // SMs, where cooperative launches are supported (else 0)
+  long long l2_bytes = 0;      // size of the L2
   int wait_polls = 0;          // bound of a wait between blocks (mpm_wait_limit; 0: the default)
   // device reduction slots (64 doubles).  Those of an assembly follow each other:
   // the grid sums' ticket (14, 15), the norms (16-19), the reaction (20-22) and
@@ -275,6 +276,7 @@ struct Sliced {
   const int* scol;       // column of each slot (padding slots: the row itself)
   const int* row;        // dof row of each storage row
   const int* pos;        // storage row of each dof row
+  int stream;            // FP32 and FP16 products take streaming loads (sliced_view)
 };
 constexpr int RESIDENT_SLICES = 4096;  // most slices of a mesh whose solves may run resident (mpm_solve.cu)
 constexpr int SLICE_WINDOW = 256;  // storage rows over which the dof rows are sorted
@@ -314,8 +316,11 @@ inline T* ptr(const Buf& b) {
 
 // the kernels' view of a mesh's sliced storage
 inline Sliced sliced_view(const mpm_mesh* m) {
+  // streaming loads where FP32 values with their columns take more than 3/4 of
+  // L2: between 90 and 100 MB of the 135.5 MB here (mpm_sliced.cuh, ld_once)
+  long long bytes = (9 * sizeof(float) + sizeof(int)) * m->nslot;
   return Sliced{ptr<int>(m->slice_w), ptr<long long>(m->slice_base), ptr<int>(m->scol), ptr<int>(m->srow),
-                ptr<int>(m->spos)};
+                ptr<int>(m->spos), bytes > m->ctx->l2_bytes / 4 * 3};
 }
 
 inline void free_buf(mpm_ctx* c, Buf& b) {

@@ -987,7 +987,7 @@ __global__ void k_mg_jac0(int n, const T* __restrict__ Dinv, const T* __restrict
 // groups of loads in flight the kernel needs about 96 registers; at 4 blocks
 // (64 registers) it spilled and ran 10 % slower (0.120 against 0.108 ms at
 // 248 k rows)
-template <class T, int MODE, class TK>
+template <class T, int MODE, class TK, bool STREAM>
 __global__ void __launch_bounds__(256, 2) k_mg_fine(int nd, int npad, Sliced SK, const TK* __restrict__ K, const float* kscale,
                           const T* __restrict__ b, const T* __restrict__ x, const T* __restrict__ Dinv,
                           T* out, const int* __restrict__ fmask, double* rz, const Scal* sk, int k,
@@ -1001,11 +1001,11 @@ __global__ void __launch_bounds__(256, 2) k_mg_fine(int nd, int npad, Sliced SK,
     T y[3];
     if constexpr (sizeof(TK) == 2) {
       float yf[3];
-      sliced_row_h(sr, SK, (const __half*)K, (const float*)x, yf);
+      sliced_row_h<STREAM>(sr, SK, (const __half*)K, (const float*)x, yf);
       float ks = *kscale;
       for (int c = 0; c < 3; ++c) y[c] = (T)(yf[c] * ks);
     } else {
-      sliced_row<T, T, T, 4>(sr, SK, (const T*)K, x, y);
+      sliced_row<T, T, T, 4, false>(sr, SK, (const T*)K, x, y);
     }
     T bv[4], res[4];
     ld4(b + 4 * (size_t)r, bv);
@@ -1141,13 +1141,10 @@ __global__ void k_mg_lvl(int nrow, int S, int R, int n1, const int* __restrict__
       if (j[u] < 0) continue;
       T xv[4];
       ld4(x + 4 * (size_t)j[u], xv);
-      // the post-smoothing is the operator's last use in a cycle: streaming
-      // loads leave L2 to what comes (9.1 -> 8.5 us a launch in the mean over the
-      // levels, and 11.4 -> 10.8 for MODE 0; streaming in MODE 0 too, 9.4 and 10.1)
       const T* vp = row + 9 * (o0 + 32 * u + lane);
       T v[9];
 #pragma unroll
-      for (int e = 0; e < 9; ++e) v[e] = MODE == 1 ? __ldcs(vp + e) : vp[e];
+      for (int e = 0; e < 9; ++e) v[e] = vp[e];
       y0 += v[0] * xv[0] + v[1] * xv[1] + v[2] * xv[2];
       y1 += v[3] * xv[0] + v[4] * xv[1] + v[5] * xv[2];
       y2 += v[6] * xv[0] + v[7] * xv[1] + v[8] * xv[2];
@@ -1515,10 +1512,10 @@ void vcycle_launch(mpm_ctx* c, const mpm_mesh* mc, const T* K, const T* r, T* z,
   MPM_LAUNCH_P(MPM_PROF_MG, k_mg_jac0<T><<<grid_for(npad, 256), 256, 0, st>>>(npad, fD, r, fx, sk, k));
   const float* ksc = (const float*)(c->d_red + 11);
   if constexpr (sizeof(T) == 4)
-    MPM_LAUNCH_P(MPM_PROF_MG_FINE, k_mg_fine<T, 0, __half><<<grid_for(npad, FB), FB, 0, st>>>(
+    MPM_LAUNCH_P(MPM_PROF_MG_FINE, (SK.stream ? k_mg_fine<T, 0, __half, true> : k_mg_fine<T, 0, __half, false>)<<<grid_for(npad, FB), FB, 0, st>>>(
         nd, npad, SK, ptr<__half>(G.fKh), ksc, r, fx, fD, fr, fmask, nullptr, sk, k, gr));
   else
-    MPM_LAUNCH_P(MPM_PROF_MG_FINE, k_mg_fine<T, 0, T><<<grid_for(npad, FB), FB, 0, st>>>(
+    MPM_LAUNCH_P(MPM_PROF_MG_FINE, k_mg_fine<T, 0, T, false><<<grid_for(npad, FB), FB, 0, st>>>(
         nd, npad, SK, K, ksc, r, fx, fD, fr, fmask, nullptr, sk, k, gr));
   MPM_LAUNCH_P(MPM_PROF_MG, k_mg_restrict1<T><<<grid_for(L0.npad, MGW), 32 * MGW, 0, st>>>(
       L0.nrow, L0.npad, ptr<int>(G.t_ptr), ptr<int>(G.t_idx), ptr<float>(G.t_w), fr, ptr<T>(L0.Dinv),
@@ -1553,10 +1550,10 @@ void vcycle_launch(mpm_ctx* c, const mpm_mesh* mc, const T* K, const T* r, T* z,
   MPM_LAUNCH_P(MPM_PROF_MG, k_mg_prolong1<T><<<grid_for(nd, 128), 128, 0, st>>>(nd, ptr<int>(G.p_idx), ptr<float>(G.p_w), fmask,
                                                                   xcur[0], fx, sk, k));
   if constexpr (sizeof(T) == 4)
-    MPM_LAUNCH_P(MPM_PROF_MG_FINE, k_mg_fine<T, 1, __half><<<grid_for(npad, FB), FB, 0, st>>>(
+    MPM_LAUNCH_P(MPM_PROF_MG_FINE, (SK.stream ? k_mg_fine<T, 1, __half, true> : k_mg_fine<T, 1, __half, false>)<<<grid_for(npad, FB), FB, 0, st>>>(
         nd, npad, SK, ptr<__half>(G.fKh), ksc, r, fx, fD, z, nullptr, rz, sk, k, gr));
   else
-    MPM_LAUNCH_P(MPM_PROF_MG_FINE, k_mg_fine<T, 1, T><<<grid_for(npad, FB), FB, 0, st>>>(
+    MPM_LAUNCH_P(MPM_PROF_MG_FINE, k_mg_fine<T, 1, T, false><<<grid_for(npad, FB), FB, 0, st>>>(
         nd, npad, SK, K, ksc, r, fx, fD, z, nullptr, rz, sk, k, gr));
 }
 

@@ -17,20 +17,30 @@ __device__ inline void ld4(const double* p, double* v) {
   double2 a = *reinterpret_cast<const double2*>(p), b = *reinterpret_cast<const double2*>(p + 2);
   v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
 }
-// the same for matrix values read once per product: streaming loads, which leave
-// L1 to the gathered vector (FP32 and FP16 values; products at 248 k rows: PCG's
-// 0.173 -> 0.167 ms, the V-cycle's 0.100 and 0.091 -> 0.097 and 0.088, the
-// refinement residual's 0.239 -> 0.225; no difference on meshes of 2 k rows).
-// The FP64 products are bound by the FP64 rate and keep the plain loads.
+// the same for the values and columns of a matrix, read once per product; STREAM
+// (Sliced::stream): streaming loads, which leave the caches to the gathered vector.
+// A matrix that stays in L2 from one product to the next keeps the plain loads,
+// and FP64 products, which the FP64 rate bounds, always do.  Two instances of a
+// kernel: with both loops in one the products of large meshes are 2 % slower.  Plain -> streaming,
+// us an iteration with the set-up (mixed multigrid PCG | mixed GMRES(30)), K and its
+// columns in MB:
+//     2.9 k rows (12 MB)  154 -> 154 | 123 -> 145     16.3 k (70)  229 -> 238 | 154 -> 203
+//    11.8 k rows (50 MB)  182 -> 247 | 145 -> 197     20.6 k (90)  260 -> 259 | 200 -> 220
+//    25.0 k rows (110 MB) 270 -> 259 | 231 -> 226    110.7 k (495) 411 -> 373 |
+template <bool STREAM, class V>
+__device__ inline V ld_once(const V* p) {
+  return STREAM ? __ldcs(p) : *p;
+}
+template <bool STREAM>
 __device__ inline void ld4_once(const float* p, float* v) {
-  float4 t = __ldcs(reinterpret_cast<const float4*>(p));
+  float4 t = ld_once<STREAM>(reinterpret_cast<const float4*>(p));
   v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
 }
+template <bool STREAM>
 __device__ inline void ld4_once(const double* p, double* v) { ld4(p, v); }
-template <class T>
+template <bool STREAM>
 __device__ inline int4 ld_cols(const int* p) {
-  const int4* q = reinterpret_cast<const int4*>(p);
-  return sizeof(T) == 8 ? *q : __ldcs(q);
+  return ld_once<STREAM>(reinterpret_cast<const int4*>(p));
 }
 __device__ inline void st4(float* p, const float* v) {
   *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
@@ -43,7 +53,7 @@ __device__ inline void st4(double* p, const double* v) {
 // y = storage row r of K (dof row S.row[r]) times x, sliced storage (one
 // thread per storage row; a warp is one slice).  XS = 4: x padded to 4
 // components per dof; XS = 3: plain 3-vectors.
-template <class T, class V, class A, int XS>
+template <class T, class V, class A, int XS, bool STREAM>
 __device__ inline void sliced_row(int r, Sliced S, const T* __restrict__ K,
                                   const V* __restrict__ x, A* y) {
   int s = r >> 5, ln = r & 31;
@@ -55,11 +65,11 @@ __device__ inline void sliced_row(int r, Sliced S, const T* __restrict__ K,
   y[0] = y[1] = y[2] = (A)0;
   for (int k4 = 0; k4 < (W >> 2); ++k4) {
     size_t off = ((size_t)k4 * 32 + ln) * 4;
-    int4 c = ld_cols<T>(cb + off);
+    int4 c = ld_cols<STREAM>(cb + off);
     int cc[4] = {c.x, c.y, c.z, c.w};
     T v[9][4];
 #pragma unroll
-    for (int e = 0; e < 9; ++e) ld4_once(Kb + e * plane + off, v[e]);
+    for (int e = 0; e < 9; ++e) ld4_once<STREAM>(Kb + e * plane + off, v[e]);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       A x0, x1, x2;
@@ -117,6 +127,7 @@ __device__ inline void df_acc(float& hi, float& lo, float k, float xh, float xl)
   lo += err + e;
 }
 
+template <bool STREAM>
 __device__ inline void sliced_row_df(int r, Sliced S, const float* __restrict__ K,
                                      const float4* __restrict__ xs, double* y) {
   int s = r >> 5, ln = r & 31;
@@ -128,11 +139,11 @@ __device__ inline void sliced_row_df(int r, Sliced S, const float* __restrict__ 
   float h[3] = {0.f, 0.f, 0.f}, l[3] = {0.f, 0.f, 0.f};
   for (int k4 = 0; k4 < (W >> 2); ++k4) {
     size_t off = ((size_t)k4 * 32 + ln) * 4;
-    int4 c = ld_cols<float>(cb + off);
+    int4 c = ld_cols<STREAM>(cb + off);
     int cc[4] = {c.x, c.y, c.z, c.w};
     float v[9][4];
 #pragma unroll
-    for (int e = 0; e < 9; ++e) ld4_once(Kb + e * plane + off, v[e]);
+    for (int e = 0; e < 9; ++e) ld4_once<STREAM>(Kb + e * plane + off, v[e]);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       // x split into hi and lo floats, two 16-byte loads per column
@@ -209,10 +220,11 @@ __device__ inline void acc_h4(const uint4* u, uint2 u8, int4 c, const float* __r
   }
 }
 
+template <bool STREAM>
 __device__ inline void load_h4(const __half* Kb, size_t plane, size_t off, uint4* u, uint2& u8) {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) u[q] = __ldcs(reinterpret_cast<const uint4*>(Kb + 2 * q * plane + 2 * off));
-  u8 = __ldcs(reinterpret_cast<const uint2*>(Kb + 8 * plane + off));
+  for (int q = 0; q < 4; ++q) u[q] = ld_once<STREAM>(reinterpret_cast<const uint4*>(Kb + 2 * q * plane + 2 * off));
+  u8 = ld_once<STREAM>(reinterpret_cast<const uint2*>(Kb + 8 * plane + off));
 }
 
 // y = storage row r of the FP16 copy of K (values scaled by a power of two) times x;
@@ -220,6 +232,7 @@ __device__ inline void load_h4(const __half* Kb, size_t plane, size_t off, uint4
 // per trip, all of their loads issued before the arithmetic: FP16 blocks are
 // half the bytes of FP32 ones, so a trip over one group would keep half as
 // many bytes in flight as the FP32 row product.
+template <bool STREAM>
 __device__ inline void sliced_row_h(int r, Sliced S, const __half* __restrict__ K,
                                     const float* __restrict__ x, float* y) {
   int s = r >> 5, ln = r & 31;
@@ -232,21 +245,21 @@ __device__ inline void sliced_row_h(int r, Sliced S, const __half* __restrict__ 
   int n4 = W >> 2, k4 = 0;
   for (; k4 + 2 <= n4; k4 += 2) {
     size_t off0 = ((size_t)k4 * 32 + ln) * 4, off1 = off0 + 128;
-    int4 c0 = ld_cols<float>(cb + off0);
-    int4 c1 = ld_cols<float>(cb + off1);
+    int4 c0 = ld_cols<STREAM>(cb + off0);
+    int4 c1 = ld_cols<STREAM>(cb + off1);
     uint4 u0[4], u1[4];
     uint2 v0, v1;
-    load_h4(Kb, plane, off0, u0, v0);
-    load_h4(Kb, plane, off1, u1, v1);
+    load_h4<STREAM>(Kb, plane, off0, u0, v0);
+    load_h4<STREAM>(Kb, plane, off1, u1, v1);
     acc_h4(u0, v0, c0, x, y);
     acc_h4(u1, v1, c1, x, y);
   }
   if (k4 < n4) {
     size_t off = ((size_t)k4 * 32 + ln) * 4;
-    int4 c0 = ld_cols<float>(cb + off);
+    int4 c0 = ld_cols<STREAM>(cb + off);
     uint4 u0[4];
     uint2 v0;
-    load_h4(Kb, plane, off, u0, v0);
+    load_h4<STREAM>(Kb, plane, off, u0, v0);
     acc_h4(u0, v0, c0, x, y);
   }
 }

@@ -102,7 +102,7 @@ __global__ void k_pcg_init(int nd, int npad, const double* __restrict__ b, const
 }
 
 // q = K p, pq_0 (one thread per row)
-template <class T, class V>
+template <class T, class V, bool STREAM>
 __global__ void k_pcg_q0(int nd, int npad, Sliced S, const T* __restrict__ K, const V* __restrict__ p,
                          V* q, Scal* sc, GridRed gr) {
   int sr = blockIdx.x * blockDim.x + threadIdx.x;  // storage row
@@ -110,7 +110,7 @@ __global__ void k_pcg_q0(int nd, int npad, Sliced S, const T* __restrict__ K, co
   if (sr < npad) {
     int r = S.row[sr];
     V y[3];
-    sliced_row<T, V, V, 4>(sr, S, K, p, y);
+    sliced_row<T, V, V, 4, STREAM>(sr, S, K, p, y);
     V yv[4] = {y[0], y[1], y[2], (V)0};
     if (r >= nd) yv[0] = yv[1] = yv[2] = (V)0;
     st4(q + 4 * (size_t)r, yv);
@@ -192,7 +192,7 @@ __global__ void k_copy4(int npad, const V* __restrict__ a, V* b) {
 
 // B_k: converged? else beta = rz_{k+1}/rz_k; w = K z; p = z + beta p;
 // q = w + beta q; pq_{k+1}  (one thread per row)
-template <class T, class V>
+template <class T, class V, bool STREAM>
 __global__ void k_pcg_b(int nd, int npad, int k, Sliced S, const T* __restrict__ K,
                         const V* __restrict__ z, V* p, V* q, Scal* sc, GridRed gr) {
   if (sc->done) return;
@@ -216,7 +216,7 @@ __global__ void k_pcg_b(int nd, int npad, int k, Sliced S, const T* __restrict__
   if (sr < npad) {
     int r = S.row[sr];
     V y[3];
-    sliced_row<T, V, V, 4>(sr, S, K, z, y);
+    sliced_row<T, V, V, 4, STREAM>(sr, S, K, z, y);
     if (r < nd) {
       V zv[4], pv[4], qv[4];
       ld4(z + 4 * (size_t)r, zv);
@@ -245,7 +245,7 @@ __global__ void k_pcg_b(int nd, int npad, int k, Sliced S, const T* __restrict__
 // matrix and the grid sum through shared memory, 4 blocks (64 registers, a
 // spill) take 0.329 ms and 3 (80 registers) 0.307 (FP32, 41.7 M blocks of the
 // cone); in FP64 0.781 (1.112 with 4 blocks, plain sums of products)
-template <class T, class V>
+template <class T, class V, bool STREAM>
 __global__ void __launch_bounds__(256, 3) k_spmv_dot(int nd, int npad, Sliced S, const T* __restrict__ K,
                            const V* __restrict__ x, V* y, const V* __restrict__ a,
                            double* slot, double* slot2, const Scal* sc, int check_s, GridRed gr) {
@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(256, 3) k_spmv_dot(int nd, int npad, Sliced S,
   if (sr < npad) {
     int r = S.row[sr];
     V v[3];
-    sliced_row<T, V, V, 4>(sr, S, K, x, v);
+    sliced_row<T, V, V, 4, STREAM>(sr, S, K, x, v);
     if (r >= nd) v[0] = v[1] = v[2] = (V)0;
     V yv[4] = {v[0], v[1], v[2], (V)0};
     st4(y + 4 * (size_t)r, yv);
@@ -419,7 +419,7 @@ __global__ void k_bicg_rotate(Scal* sc, const double* next_rho1, const double* n
 // r = b - K x (FP64 x in 3 components, FP64 accumulation, any matrix
 // precision), masked, written in 3 (R3) or 4 components; slot += r.r.  Bounded
 // to 4 resident blocks per SM: 0.266 -> 0.239 ms at 28.3 M blocks
-template <class T, int RS>
+template <class T, int RS, bool STREAM>
 __global__ void __launch_bounds__(256, 4) k_residual64(int nd, int npad, Sliced S, const T* __restrict__ K,
                              const double* __restrict__ x, const float4* __restrict__ xs,
                              const double* __restrict__ b, const int* __restrict__ mask, double* r,
@@ -430,9 +430,9 @@ __global__ void __launch_bounds__(256, 4) k_residual64(int nd, int npad, Sliced 
     int rr = S.row[sr];
     double y[3];
     if constexpr (sizeof(T) == 4)
-      sliced_row_df(sr, S, (const float*)K, xs, y);
+      sliced_row_df<STREAM>(sr, S, (const float*)K, xs, y);
     else
-      sliced_row<T, double, double, 3>(sr, S, K, x, y);
+      sliced_row<T, double, double, 3, STREAM>(sr, S, K, x, y);
     double v[4] = {0.0, 0.0, 0.0, 0.0};
     if (rr < nd) {
       int mk = mask[rr];
@@ -475,6 +475,9 @@ const float4* residual_split(mpm_ctx* c, const mpm_mesh* m, const T* K, const do
 }
 
 Sliced sliced_of(const mpm_mesh* m) { return sliced_view(m); }
+
+// the instance of a product kernel for S (FP64 has one: plain loads)
+#define MPM_STREAM(S, T, ...) ((S).stream && sizeof(T) == 4 ? __VA_ARGS__, sizeof(T) == 4> : __VA_ARGS__, false>)
 
 // The plan of a resident solve (mpm_resident.cuh) of this mesh with nv vectors
 // per row, G = 0 for the launches per iteration.  Resident is the faster way
@@ -572,7 +575,7 @@ int run_pcg(mpm_ctx* c, const mpm_mesh* m, const T* K, const V* Dinv, const doub
   int vb = grid_strided(npad);
   GridRed gr = grid_red(c, 2, std::max(vb, grid_for(npad, 32 * SW)));
   MPM_LAUNCH(k_pcg_init<V><<<vb, 256, 0, st>>>(nd, npad, b, ptr<int>(m->dof_mask), Dinv, x, r, z, p, sc_d, gr));
-  MPM_LAUNCH(k_pcg_q0<T, V><<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, K, p, q, sc_d, gr));
+  MPM_LAUNCH(MPM_STREAM(S, T, k_pcg_q0<T, V)<<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, K, p, q, sc_d, gr));
   MPM_CUDA(cudaMemcpyAsync(sc_h, sc_d, sizeof(Scal), cudaMemcpyDeviceToHost, st));
   MPM_CUDA(cudaStreamSynchronize(st));
   double bb = sc_h->bb;
@@ -590,7 +593,7 @@ int run_pcg(mpm_ctx* c, const mpm_mesh* m, const T* K, const V* Dinv, const doub
     int kend = std::min(maxit, k + batch);
     for (; k < kend; ++k) {
       MPM_LAUNCH_P(MPM_PROF_PCG_UPDATE, k_pcg_a<V><<<vb, 256, 0, st>>>(nd, k, Dinv, x, r, z, p, q, sc_d, gr));
-      MPM_LAUNCH_P(MPM_PROF_PCG_SPMV, k_pcg_b<T, V><<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, k, S, K, z, p, q, sc_d, gr));
+      MPM_LAUNCH_P(MPM_PROF_PCG_SPMV, MPM_STREAM(S, T, k_pcg_b<T, V)<<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, k, S, K, z, p, q, sc_d, gr));
     }
     MPM_CUDA(cudaMemcpyAsync(sc_h, sc_d, sizeof(Scal), cudaMemcpyDeviceToHost, st));
     MPM_CUDA(cudaStreamSynchronize(st));
@@ -621,7 +624,7 @@ int run_pcg_mg(mpm_ctx* c, const mpm_mesh* m, const T* K, const double* b, T* x,
   MPM_LAUNCH(k_pcg_init_mg<T><<<vb, 256, 0, st>>>(nd, npad, b, ptr<int>(m->dof_mask), x, r, sc_d, gr));
   mg_apply<T>(c, m, K, r, z, nullptr, 0, &sc_d->rz[0]);
   MPM_LAUNCH(k_copy4<T><<<grid_for(npad, 256), 256, 0, st>>>(npad, z, p));
-  MPM_LAUNCH(k_pcg_q0<T, T><<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, K, p, q, sc_d, gr));
+  MPM_LAUNCH(MPM_STREAM(S, T, k_pcg_q0<T, T)<<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, K, p, q, sc_d, gr));
   MPM_CUDA(cudaMemcpyAsync(sc_h, sc_d, sizeof(Scal), cudaMemcpyDeviceToHost, st));
   MPM_CUDA(cudaStreamSynchronize(st));
   double bb = sc_h->bb;
@@ -639,7 +642,7 @@ int run_pcg_mg(mpm_ctx* c, const mpm_mesh* m, const T* K, const double* b, T* x,
     for (; k < kend; ++k) {
       MPM_LAUNCH_P(MPM_PROF_PCG_UPDATE, k_pcg_a<T, false><<<vb, 256, 0, st>>>(nd, k, nullptr, x, r, z, p, q, sc_d, gr));
       mg_apply<T>(c, m, K, r, z, sc_d, k, &sc_d->rz[(k + 1) % 3]);
-      MPM_LAUNCH_P(MPM_PROF_PCG_SPMV, k_pcg_b<T, T><<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, k, S, K, z, p, q, sc_d, gr));
+      MPM_LAUNCH_P(MPM_PROF_PCG_SPMV, MPM_STREAM(S, T, k_pcg_b<T, T)<<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, k, S, K, z, p, q, sc_d, gr));
     }
     MPM_CUDA(cudaMemcpyAsync(sc_h, sc_d, sizeof(Scal), cudaMemcpyDeviceToHost, st));
     MPM_CUDA(cudaStreamSynchronize(st));
@@ -724,11 +727,11 @@ int run_bicgstab(mpm_ctx* c, const mpm_mesh* m, const T* K, const T* Dinv, const
       MPM_CUDA(cudaMemsetAsync(red, 0, 2 * sizeof(double), st));
       MPM_LAUNCH(k_bicg_p<V><<<vb, 256, 0, st>>>(npad, p, r, v, ph, Dinv, sc_d));
       if (!Dinv) mg_precondition<T>(c, m, K, p, ph, sc_d);
-      MPM_LAUNCH_P(MPM_PROF_BICG_SPMV, k_spmv_dot<T, V><<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, K, ph, v, r0, &sc_d->a[4], nullptr, sc_d, 0, gr));
+      MPM_LAUNCH_P(MPM_PROF_BICG_SPMV, MPM_STREAM(S, T, k_spmv_dot<T, V)<<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, K, ph, v, r0, &sc_d->a[4], nullptr, sc_d, 0, gr));
       MPM_LAUNCH(k_bicg_s<V><<<vb, 256, 0, st>>>(npad, r, v, s, shv, Dinv, sc_d, gr));
       MPM_LAUNCH(k_bicg_check_s<V, X><<<vb, 256, 0, st>>>(nd, x, ph, sc_d));
       if (!Dinv) mg_precondition<T>(c, m, K, s, shv, sc_d);
-      MPM_LAUNCH_P(MPM_PROF_BICG_SPMV, k_spmv_dot<T, V><<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, K, shv, t, s, &sc_d->a[6], &sc_d->a[7], sc_d, 1, gr));
+      MPM_LAUNCH_P(MPM_PROF_BICG_SPMV, MPM_STREAM(S, T, k_spmv_dot<T, V)<<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, K, shv, t, s, &sc_d->a[6], &sc_d->a[7], sc_d, 1, gr));
       MPM_LAUNCH(k_bicg_x<V, X><<<vb, 256, 0, st>>>(nd, npad, x, r, ph, shv, s, t, r0, sc_d, red, red + 1, gr));
       MPM_LAUNCH(k_bicg_rotate<<<1, 1, 0, st>>>(sc_d, red, red + 1, it + 1));
     }
@@ -755,14 +758,14 @@ int run_bicgstab(mpm_ctx* c, const mpm_mesh* m, const T* K, const T* Dinv, const
 
 // r = b - K x on the free components (x over 4-component rows), rows beyond
 // nd and fixed components zero
-template <class T, class V>
+template <class T, class V, bool STREAM>
 __global__ void k_gm_residual(int nd, int npad, Sliced S, const T* __restrict__ K, const V* __restrict__ x,
                               const double* __restrict__ b, const int* __restrict__ mask, V* r) {
   int sr = blockIdx.x * blockDim.x + threadIdx.x;  // storage row
   if (sr >= npad) return;
   int i = S.row[sr];
   V y[3];
-  sliced_row<T, V, V, 4>(sr, S, K, x, y);
+  sliced_row<T, V, V, 4, STREAM>(sr, S, K, x, y);
   V rv[4] = {(V)0, (V)0, (V)0, (V)0};
   if (i < nd) {
     int mi = mask[i];
@@ -786,13 +789,13 @@ __global__ void k_gm_dinv(int nd, int npad, const V* __restrict__ Dinv, const V*
   st4(z + 4 * (size_t)i, zv);
 }
 
-template <class T, class V>
+template <class T, class V, bool STREAM>
 __global__ void k_gm_spmv(int nd, int npad, Sliced S, const T* __restrict__ K, const V* __restrict__ z, V* w) {
   int sr = blockIdx.x * blockDim.x + threadIdx.x;  // storage row
   if (sr >= npad) return;
   int i = S.row[sr];
   V y[3];
-  sliced_row<T, V, V, 4>(sr, S, K, z, y);
+  sliced_row<T, V, V, 4, STREAM>(sr, S, K, z, y);
   V wv[4] = {y[0], y[1], y[2], (V)0};
   if (i >= nd) wv[0] = wv[1] = wv[2] = (V)0;
   st4(w + 4 * (size_t)i, wv);
@@ -893,7 +896,7 @@ int run_gmres(mpm_ctx* c, const mpm_mesh* m, const T* K, const T* Dinv, const do
   };
   MPM_CUDA(cudaMemsetAsync(x, 0, sizeof(V) * n4, st));
   // ||b|| over the free components
-  MPM_LAUNCH(k_gm_residual<T, V><<<gr, 256, 0, st>>>(nd, npad, S, K, x, b, mask, w));
+  MPM_LAUNCH(MPM_STREAM(S, T, k_gm_residual<T, V)<<<gr, 256, 0, st>>>(nd, npad, S, K, x, b, mask, w));
   dots(1, w, w);
   double bn = sqrt(hh[0]);
   *iters = 0;
@@ -915,7 +918,7 @@ int run_gmres(mpm_ctx* c, const mpm_mesh* m, const T* K, const T* Dinv, const do
     for (; j < mr && total < maxit; ++j) {
       V* vj1 = Vb + (size_t)(j + 1) * n4;
       MPM_LAUNCH(k_gm_dinv<V><<<gr, 256, 0, st>>>(nd, npad, Dinv, Vb + (size_t)j * n4, z));
-      MPM_LAUNCH_P(MPM_PROF_BICG_SPMV, k_gm_spmv<T, V><<<gr, 256, 0, st>>>(nd, npad, S, K, z, w));
+      MPM_LAUNCH_P(MPM_PROF_BICG_SPMV, MPM_STREAM(S, T, k_gm_spmv<T, V)<<<gr, 256, 0, st>>>(nd, npad, S, K, z, w));
       double hcol[33];
       for (int i = 0; i <= j; ++i) hcol[i] = 0.0;
       for (int pass = 0; pass < 2; ++pass) {
@@ -958,7 +961,7 @@ int run_gmres(mpm_ctx* c, const mpm_mesh* m, const T* K, const T* Dinv, const do
     MPM_CUDA(cudaMemcpyAsync(yd, y.data(), sizeof(double) * k, cudaMemcpyHostToDevice, st));
     MPM_LAUNCH(k_gm_update_x<V><<<grid_for(nd, 256), 256, 0, st>>>(nd, n4, k, Vb, yd, Dinv, x));
     // the true residual of the restart (and of the end)
-    MPM_LAUNCH(k_gm_residual<T, V><<<gr, 256, 0, st>>>(nd, npad, S, K, x, b, mask, w));
+    MPM_LAUNCH(MPM_STREAM(S, T, k_gm_residual<T, V)<<<gr, 256, 0, st>>>(nd, npad, S, K, x, b, mask, w));
     dots(1, w, w);
     beta = sqrt(hh[0]);
     conv = beta <= tol * bn;
@@ -1053,7 +1056,7 @@ void solve(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const void* 
   float* q = grow<float>(c, c->v[7], n4);
   MPM_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * n3, st));
   MPM_CUDA(cudaMemsetAsync(slot, 0, sizeof(double), st));
-  MPM_LAUNCH_P(MPM_PROF_REFINE, k_residual64<float, 3><<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, Kf, x, residual_split(c, m, Kf, x), b, ptr<int>(m->dof_mask), r64, slot, gred));
+  MPM_LAUNCH_P(MPM_PROF_REFINE, MPM_STREAM(S, float, k_residual64<float, 3)<<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, Kf, x, residual_split(c, m, Kf, x), b, ptr<int>(m->dof_mask), r64, slot, gred));
   MPM_CUDA(cudaMemcpyAsync(c->h_red + 60, slot, sizeof(double), cudaMemcpyDeviceToHost, st));
   MPM_CUDA(cudaStreamSynchronize(st));
   double bb = c->h_red[60], rr = bb;
@@ -1087,7 +1090,7 @@ void solve(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const void* 
     }
     MPM_LAUNCH(k_axpy_f2d<<<grid_for(n3, 256), 256, 0, st>>>(n3, x, d32));
     MPM_CUDA(cudaMemsetAsync(slot, 0, sizeof(double), st));
-    MPM_LAUNCH_P(MPM_PROF_REFINE, k_residual64<float, 3><<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, Kf, x, residual_split(c, m, Kf, x), b, ptr<int>(m->dof_mask), r64, slot, gred));
+    MPM_LAUNCH_P(MPM_PROF_REFINE, MPM_STREAM(S, float, k_residual64<float, 3)<<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, Kf, x, residual_split(c, m, Kf, x), b, ptr<int>(m->dof_mask), r64, slot, gred));
     MPM_CUDA(cudaMemcpyAsync(c->h_red + 60, slot, sizeof(double), cudaMemcpyDeviceToHost, st));
     MPM_CUDA(cudaStreamSynchronize(st));
     rr = c->h_red[60];
@@ -1206,7 +1209,7 @@ extern "C" int mpm_solve_static(mpm_ctx* c, const mpm_mesh* m, const double* K, 
     static_assert((kStaticBytes / (28 * sizeof(double)) / 256 + 1) <= kStaticParts,
                   "partial sums of the row kernels");
     MPM_LAUNCH(k_pcg_init<double><<<vb, 256, 0, st>>>(nd, npad, rhs, ptr<int>(m->dof_mask), Dinv, x, r, z, p, sc, gr));
-    MPM_LAUNCH(k_pcg_q0<double, double><<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, K, p, q, sc, gr));
+    MPM_LAUNCH(k_pcg_q0<double, double, false><<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, K, p, q, sc, gr));
     Scal* h = (Scal*)(c->h_red + 32);
     MPM_CUDA(cudaMemcpyAsync(h, sc, sizeof(Scal), cudaMemcpyDeviceToHost, st));
     MPM_CUDA(cudaStreamSynchronize(st));
@@ -1220,7 +1223,7 @@ extern "C" int mpm_solve_static(mpm_ctx* c, const mpm_mesh* m, const double* K, 
         int kend = std::min(maxit, k + 32);
         for (; k < kend; ++k) {
           MPM_LAUNCH(k_pcg_a<double><<<vb, 256, 0, st>>>(nd, k, Dinv, x, r, z, p, q, sc, gr));
-          MPM_LAUNCH(k_pcg_b<double, double><<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, k, S, K, z, p, q, sc, gr));
+          MPM_LAUNCH(k_pcg_b<double, double, false><<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, k, S, K, z, p, q, sc, gr));
         }
         MPM_CUDA(cudaMemcpyAsync(h, sc, sizeof(Scal), cudaMemcpyDeviceToHost, st));
         MPM_CUDA(cudaStreamSynchronize(st));
