@@ -424,11 +424,13 @@ __global__ void k_residual_rows(int nd, int P, double load, const long long* __r
 // ------------------------------------------------------------------ tangent (row gather)
 
 constexpr int TW = 4;  // warps per block of the tangent gather (at most)
+constexpr int TSMEM = 220 * 1024;  // shared memory of a block of it (at most)
+constexpr int CSMEM = 200 * 1024;  // and of the contact rows
 constexpr int TANGENT_FEW_ROWS = 20000;  // below: a block per row (tangent_passes)
 
 // open-addressing table of a row's columns (dof -> position in the row), in
 // shared memory: a power of two at least twice the longest row
-__host__ __device__ inline int tangent_hash_size(int mr) {
+constexpr int tangent_hash_size(int mr) {
   int h = 64;
   while (h < 2 * mr) h <<= 1;
   return h;
@@ -1516,9 +1518,9 @@ void contact_terms(mpm_ctx* c, mpm_mesh* m, const mpm_material& mat, const mpm_r
   Sliced S = sliced_view(m);
   // 128 threads per row, fewer where four copies of the longest row do not fit
   size_t wb = TANGENT ? sizeof(double) * (9 * (size_t)m->maxrow + 64) : 0;
-  int nw = TANGENT ? (int)std::min<size_t>(4, (size_t)(200 * 1024) / wb) : 4;
+  int nw = TANGENT ? (int)std::min<size_t>(4, CSMEM / wb) : 4;
   auto kern = k_contact_rows<T, RES, TANGENT>;
-  MPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(nw * wb)));
+  dynamic_smem(kern, CSMEM);
   MPM_LAUNCH_P(MPM_PROF_CONTACT, kern<<<m->nct, 32 * nw, nw * wb, st>>>(
       m->maxrow, ptr<int>(m->ct_row), ptr<int>(m->ct_ptr), ptr<int>(m->ct_ent), ptr<int>(m->cb_n),
       ptr<int>(m->cb_idx), ptr<double>(m->cb_phi), cf, ck, con, R, fc, ptr<int>(m->row_ptr),
@@ -1539,11 +1541,11 @@ template <class T, class F>
 void tangent_launch(mpm_ctx* c, mpm_mesh* m, F kern, size_t row_bytes, int rpw, int wpr, int pw, int lo, int hi,
                     int last, const void* gx, const void* Aalg, void* K) {
   size_t wb = rpw * row_bytes;
-  int tw = (int)std::min<size_t>(TW, (size_t)(220 * 1024) / wb) / wpr * wpr;
+  int tw = (int)std::min<size_t>(TW, TSMEM / wb) / wpr * wpr;
   if (tw < 1) throw CudaError(MPM_ERR_SUPPORT, "stiffness row too long for the tangent gather");
   size_t smem = wb * tw;
   Sliced S = sliced_view(m);
-  MPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  dynamic_smem(kern, TSMEM);
   MPM_LAUNCH_P(MPM_PROF_TANGENT, kern<<<grid_for(m->ndof, tw / wpr * rpw), 32 * tw, smem, c->stream>>>(
       m->ndof, m->np, pw, lo, hi, last, ptr<int>(m->row_ptr), ptr<int>(m->col), S, ptr<long long>(m->src_ptr),
       ptr<uint64_t>(m->src_key), ptr<unsigned short>(m->src_pos), (const T*)gx, (const T*)Aalg, ptr<double>(m->kg),
@@ -1566,7 +1568,7 @@ void tangent_passes(mpm_ctx* c, mpm_mesh* m, bool mixed, bool upper, int pw, con
   for (int ps = 0; ps < np_; ++ps) {
     int lo = passes[ps][0], hi = passes[ps][1], last = ps == np_ - 1;
     size_t rb = mixed ? tangent_row_bytes_f32(hi) : tangent_warp_bytes_f64(hi);
-    bool share = (ps > 0 || m->ndof < TANGENT_FEW_ROWS) && 4 * rb <= 220 * 1024;
+    bool share = (ps > 0 || m->ndof < TANGENT_FEW_ROWS) && 4 * rb <= TSMEM;
     if (mixed) {
       if (share)
         tangent_launch<float>(c, m, k_tangent_rows_f32<32, 4>, rb, 1, 4, pw, lo, hi, last, gx, Aalg, K);
@@ -1645,7 +1647,7 @@ void assemble(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const mpm
     bool few = nd < TANGENT_FEW_ROWS;
     size_t smem = (few ? 1 : 4) * 2 * sizeof(int) * (size_t)hs;
     auto kern = few ? k_src_pos<true> : k_src_pos<false>;
-    MPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    dynamic_smem(kern, 4 * 2 * (int)sizeof(int) * tangent_hash_size(MAXROW));
     MPM_LAUNCH_P(MPM_PROF_PATTERN, kern<<<grid_for(nd, few ? 1 : 4), 128, smem, st>>>(
         nd, P, pw, hs, rp, col, ptr<long long>(m->src_ptr), ptr<uint64_t>(m->src_key), nsup, sidx, sp));
     m->src_pos_gen = m->gen;

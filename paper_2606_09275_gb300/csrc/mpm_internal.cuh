@@ -337,6 +337,15 @@ inline GridRed grid_red(mpm_ctx* c, int nv, long long blocks) {
 
 // at least one block: an empty grid is a launch error, and every kernel
 // bounds-checks its index
+// Allows a kernel `most` bytes of dynamic shared memory, the most that any of its
+// launches takes: the attribute is the function's, for all threads of the
+// process, and a launch's own size would take it from under the larger launch
+// of another thread.
+template <class F>
+inline void dynamic_smem(F* kern, int most) {
+  MPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+}
+
 inline int grid_for(long long n, int block) {
   long long g = (n + block - 1) / block;
   return (int)(g < 1 ? 1 : g);

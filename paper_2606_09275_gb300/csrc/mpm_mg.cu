@@ -31,6 +31,7 @@ namespace mpm {
 namespace {
 
 constexpr int MGW = 4;  // warps per block of the warp-per-row level kernels
+constexpr int MG_N3 = 81;  // unknowns of the coarsest level (at most; 27 nodes)
 
 // packed grid coordinates (coarse grids have at most 2^7 + 1 nodes per axis)
 __host__ __device__ inline int pack3(int x, int y, int z) { return x | (y << 10) | (z << 20); }
@@ -1374,7 +1375,7 @@ void mg_structure(mpm_ctx* c, mpm_mesh* m) {
   }
   MGLevel& C = G.lev[G.nlev - 1];
   G.n3c = 3 * C.nrow;
-  if (G.n3c > 81) throw CudaError(MPM_ERR_ARG, "multigrid: coarsest level too large");
+  if (G.n3c > MG_N3) throw CudaError(MPM_ERR_ARG, "multigrid: coarsest level too large");
   int e = check_device_error(c, "multigrid structure");
   if (e) throw CudaError(e, c->err);
   G.gen = m->gen;
@@ -1472,7 +1473,7 @@ void mg_numeric(mpm_ctx* c, mpm_mesh* m, const T* K, bool coarse) {
   int n3 = G.n3c;
   T* Ci = grow<T>(c, G.cinv, (size_t)std::max(n3 * n3, 1));
   size_t dsm = sizeof(double) * (size_t)n3 * (n3 + 1);
-  MPM_CUDA(cudaFuncSetAttribute(k_mg_dense<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm));
+  dynamic_smem(k_mg_dense<T>, (int)sizeof(double) * MG_N3 * (MG_N3 + 1));
   MPM_LAUNCH_P(MPM_PROF_MG_SETUP, k_mg_dense<T><<<1, 1024, dsm, st>>>(C.nrow, C.S, C.R, ptr<int>(C.xyz), C.n1, ptr<int>(C.gid),
                                                 ptr<T>(C.A), Ci));
   G.prec = sizeof(T) == 4 ? MPM_MIXED : MPM_FP64;

@@ -31,6 +31,7 @@ constexpr int RK_NBUF = 6;          // rotating sets of sum slots and messages
 constexpr int RK_NV = 2;            // values per grid sum
 constexpr int RK_COPY = 16;         // copies of a message, a line each
 constexpr int RK_POLLS = 1 << 21;   // bound of a wait unless the context sets another (about a second)
+constexpr int RK_SMEM = 200 * 1024;  // dynamic shared memory of a block (at most)
 constexpr int RK_ROW = 64;          // slots' worth of a quad's own vector work
 
 // slots of a launch of G blocks: the sums' partials, then the messages

@@ -486,7 +486,6 @@ Sliced sliced_of(const mpm_mesh* m) { return sliced_view(m); }
 // RESIDENT_SLICES.
 template <class T>
 RkPlan resident_plan(const mpm_ctx* c, const mpm_mesh* m, int nv) {
-  constexpr int SMEM = 200 * 1024;
   RkPlan p{};
   const std::vector<int>& w = m->slice_w_host;
   int ns = m->nslice;
@@ -508,8 +507,8 @@ RkPlan resident_plan(const mpm_ctx* c, const mpm_mesh* m, int nv) {
   p.rows = std::max(rows, 4);
   long long state = (long long)p.rows * ((3 * nv + 9) * sizeof(T) + 2 * sizeof(int));
   long long kept = (long long)groups * (rk_group<T>() * sizeof(T) + 16 * sizeof(int));
-  if (state > SMEM) return p;
-  if (state + kept <= SMEM) p.groups = groups;
+  if (state > RK_SMEM) return p;
+  if (state + kept <= RK_SMEM) p.groups = groups;
   p.smem = (int)(state + (p.groups ? kept : 0));
   p.polls = c->wait_polls > 0 ? c->wait_polls : RK_POLLS;
   p.G = W + 1;
@@ -530,7 +529,7 @@ int run_resident(mpm_ctx* c, bool* ran, void (*kern)(A...), const RkPlan& pl, un
   void* args[] = {(void*)&a...};
   MPM_CUDA(cudaMemsetAsync(sc_d, 0, sizeof(Scal), st));
   MPM_CUDA(cudaMemsetAsync(slots, 0xff, sizeof(*slots) * rk_slot_words(pl.G), st));
-  MPM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.smem));
+  dynamic_smem(kern, RK_SMEM);
   cudaError_t e = cudaLaunchCooperativeKernel((const void*)kern, dim3(pl.G), dim3(RK_T), args, pl.smem, st);
   *ran = e != cudaErrorCooperativeLaunchTooLarge;
   if (!*ran) {
