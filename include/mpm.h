@@ -255,9 +255,14 @@ enum {
   MPM_EXPORT_BCMASK = 15,      /* int[ndof] fixed components                    */
   MPM_EXPORT_POPULATED = 16,   /* int[nleaf]                                    */
   MPM_EXPORT_GHOST_FACES = 17, /* int[4*nghost]: K, N, axis, sign              */
-  MPM_EXPORT_MG_LEVELS = 18    /* int[32]: per multigrid coarse level (up to 8):
+  MPM_EXPORT_MG_LEVELS = 18,   /* int[32]: per multigrid coarse level (up to 8):
                                   depth, rows, stencil radius, stencil size;
                                   zeros until a method-3 solve on this mesh */
+  MPM_EXPORT_MG_NODES = 19,    /* int[4*rows], level by level: grid coordinates at
+                                  the level's depth, fixed components            */
+  MPM_EXPORT_MG_VALUES = 20    /* double, level by level: the Galerkin operator
+                                  [rows][stencil size][9] (offsets x fastest), then
+                                  the inverse of the last one [3*rows][3*rows]   */
 };
 int mpm_mesh_export(const mpm_mesh* mesh, int what, void* dst, size_t bytes);
 

@@ -454,6 +454,50 @@ extern "C" int mpm_mesh_export(const mpm_mesh* mc, int what, void* dst, size_t b
         memcpy(dst, info, sizeof(info));
         return (int)MPM_OK;
       }
+      case MPM_EXPORT_MG_NODES:
+      case MPM_EXPORT_MG_VALUES: {
+        const MGData* G = (m->mg && m->mg->gen == m->gen && m->mg->num_gen == m->gen) ? m->mg : nullptr;
+        size_t n = 0;
+        for (int l = 0; G && l < G->nlev; ++l)
+          n += what == MPM_EXPORT_MG_NODES ? sizeof(int) * 4 * G->lev[l].nrow
+                                           : sizeof(double) * 9 * (size_t)G->lev[l].S * G->lev[l].nrow;
+        if (G && what == MPM_EXPORT_MG_VALUES) n += sizeof(double) * (size_t)G->n3c * G->n3c;
+        if (bytes < n) {
+          set_error(c, "export buffer too small");
+          return (int)MPM_ERR_ARG;
+        }
+        std::vector<char> h;
+        auto fetch = [&](const Buf& b, size_t size) {
+          h.resize(size);
+          if (size) MPM_CUDA(cudaMemcpyAsync(h.data(), b.p, size, cudaMemcpyDeviceToHost, c->stream));
+          MPM_CUDA(cudaStreamSynchronize(c->stream));
+        };
+        int* oi = (int*)dst;
+        double* od = (double*)dst;
+        auto values = [&](const Buf& b, size_t count) {
+          size_t w = G->prec == MPM_MIXED ? sizeof(float) : sizeof(double);
+          fetch(b, w * count);
+          for (size_t i = 0; i < count; ++i)
+            *od++ = G->prec == MPM_MIXED ? (double)((const float*)h.data())[i] : ((const double*)h.data())[i];
+        };
+        for (int l = 0; G && l < G->nlev; ++l) {
+          const MGLevel& L = G->lev[l];
+          if (what == MPM_EXPORT_MG_VALUES) {
+            values(L.A, 9 * (size_t)L.S * L.nrow);
+            continue;
+          }
+          fetch(L.xyz, sizeof(int) * L.nrow);
+          for (int r = 0; r < L.nrow; ++r) {
+            int v = ((const int*)h.data())[r];  // packed as pack3 (mpm_mg.cu)
+            for (int d = 0; d < 3; ++d) oi[4 * r + d] = (v >> (10 * d)) & 1023;
+          }
+          fetch(L.mask, sizeof(int) * L.nrow);
+          for (int r = 0; r < L.nrow; ++r) oi[4 * r + 3] = ((const int*)h.data())[r];
+          oi += 4 * (size_t)L.nrow;
+        }
+        if (G && what == MPM_EXPORT_MG_VALUES) values(G->cinv, (size_t)G->n3c * G->n3c);
+        return (int)MPM_OK;
+      }
       default:
         set_error(c, "unknown export selector");
         return (int)MPM_ERR_ARG;

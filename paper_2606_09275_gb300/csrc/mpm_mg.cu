@@ -565,26 +565,33 @@ __global__ void k_mg_rapu(int nrow_f, int Rc, int Sc, int n1c, const int* __rest
   }
 }
 
-// One axis of the trilinear interpolation, gathered: five values of the finer
-// nodes i - 2 .. i + 2 to the coarse nodes they interpolate from; i an even node
-// (three of them) or an odd one (four).  Halves to the nearest integer.
+// Twice one axis of the trilinear interpolation, gathered: five values of the
+// finer nodes i - 2 .. i + 2 to the coarse nodes they interpolate from; i an even
+// node (three of them) or an odd one (four)
 __device__ inline void gather_axis(const long long* v, bool odd, long long* o) {
-  auto h = [](long long x) { return (x + 1) >> 1; };
   if (odd) {
-    o[0] = h(v[0]);
-    o[1] = h(v[0]) + v[1] + h(v[2]);
-    o[2] = h(v[2]) + v[3] + h(v[4]);
-    o[3] = h(v[4]);
+    o[0] = v[0];
+    o[1] = v[0] + 2 * v[1] + v[2];
+    o[2] = v[2] + 2 * v[3] + v[4];
+    o[3] = v[4];
   } else {
-    o[0] = v[0] + h(v[1]);
-    o[1] = h(v[1]) + v[2] + h(v[3]);
-    o[2] = h(v[3]) + v[4];
+    o[0] = 2 * v[0] + v[1];
+    o[1] = v[1] + 2 * v[2] + v[3];
+    o[2] = v[3] + 2 * v[4];
     o[3] = 0;
   }
 }
 
 // The same product gathered, for stencils of radius 2 on both levels: one block
-// per coarse row a, in the fixed point of the scattered product.  Over the rows
+// per coarse row a, in fixed point.  An entry of the finer operator is rounded
+// once, in units of 2^3 of the scattered product's, and the weights are whole
+// numbers in units of 2^-6, 2^-3 a side: the product is exactly as symmetric as
+// the finer operator and as accurate as the scattered one, which rounds every
+// term in its unit (rms error against exact sums 55 and 59 ulps of the largest
+// entry for 27 x 125 random entries; halves rounded axis by axis, 578).  No
+// overflow: the sum of an entry's |terms| is at most 8/27 of B, so below
+// 8/27 2^61 in the scattered unit and below 2^63 in the unit 2^-3 of it that the
+// sums are taken in.  Over the rows
 // i of the finer nodes 2 a + {-1, 0, 1}^3, the 5 x 5 x 5 blocks of a row are
 // interpolated an axis at a time, a thread per line, to the 4 x 4 x 4 coarse
 // nodes around i, and added to the row of a in shared memory; the next row's
@@ -610,7 +617,7 @@ __global__ void __launch_bounds__(RG)
   __shared__ unsigned char mask[343];  // their Dirichlet components
   int t = threadIdx.x, a = blockIdx.x;
   double B = __longlong_as_double((long long)*bnd) * 27.0;
-  int ex = !(B > 0.0) || !isfinite(B) ? 0 : 60 - ilogb(B);  // as fixed_scale
+  int ex = !(B > 0.0) || !isfinite(B) ? 0 : 57 - ilogb(B);  // 3 below fixed_scale's
   int ca[3];
   unpack3(xyz_c[a], ca);
   for (int f = t; f < 343; f += RG) {
@@ -649,7 +656,7 @@ __global__ void __launch_bounds__(RG)
       continue;
     }
     int dx = q % 3 - 1, dy = (q / 3) % 3 - 1, dz = q / 9 - 1;
-    int w = abs(dx) + abs(dy) + abs(dz);  // P_ia = 2^-w
+    int w = 3 - (abs(dx) + abs(dy) + abs(dz));  // P_ia = 2^(w - 3)
     long long v[5], o[4];
     if (onx) {
       bool off = (mask[ctr] >> ex3) & 1;
@@ -657,9 +664,9 @@ __global__ void __launch_bounds__(RG)
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
         if constexpr (sizeof(T) == 4)
-          v[k] = __float2ll_rn(scalbnf(next[k], ex - w));
+          v[k] = __float2ll_rn(scalbnf(next[k], ex)) << w;
         else
-          v[k] = __double2ll_rn(scalbn(next[k], ex - w));
+          v[k] = __double2ll_rn(scalbn(next[k], ex)) << w;
         if (off || ((mj[k] >> ec3) & 1)) v[k] = 0;
       }
       gather_axis(v, dx != 0, o);
@@ -694,9 +701,9 @@ __global__ void __launch_bounds__(RG)
   __syncthreads();
   for (int f = t; f < NE; f += RG) {
     if constexpr (sizeof(T) == 4)
-      A[(size_t)a * NE + f] = scalbnf(__ll2float_rn(acc[f]), -ex);
+      A[(size_t)a * NE + f] = scalbnf(__ll2float_rn(acc[f]), -ex - 6);
     else
-      A[(size_t)a * NE + f] = scalbn((double)acc[f], -ex);
+      A[(size_t)a * NE + f] = scalbn((double)acc[f], -ex - 6);
   }
 }
 

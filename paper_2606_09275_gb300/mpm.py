@@ -23,7 +23,7 @@ FP64, MIXED = 0, 1
 
 EXPORT = dict(leaf_level=0, leaf_anchor=1, node_coord=2, node_hang=3, node_dof=4, cptr=5, cidx=6,
               cw=7, nsup=8, sidx=9, S=10, dS=11, row_ptr=12, col=13, ghost=14, bcmask=15,
-              populated=16, ghost_faces=17, mg_levels=18)
+              populated=16, ghost_faces=17, mg_levels=18, mg_nodes=19, mg_values=20)
 
 SYMBOLS = ["mpm_create", "mpm_destroy", "mpm_last_error", "mpm_octree_build", "mpm_mesh_free",
            "mpm_mesh_counts", "mpm_mesh_export", "mpm_assemble", "mpm_solve", "mpm_step",
@@ -363,6 +363,11 @@ class Mesh:
         if what in ("cidx", "cw"):
             ncon = int(self.export("cptr")[-1])
             shape, dt = ncon, (np.int32 if what == "cidx" else np.float64)
+        elif what in ("mg_nodes", "mg_values"):
+            lev = self.export("mg_levels").astype(np.int64)
+            rows, last = lev[:, 1], 3 * lev[lev[:, 1] > 0][-1:, 1].sum()
+            shape, dt = (((int(rows.sum()), 4), np.int32) if what == "mg_nodes" else
+                         (int(9 * (rows * lev[:, 3]).sum() + last * last), np.float64))
         else:
             shape, dt = sizes[what]
         out = np.zeros(shape, dtype=dt)
