@@ -805,19 +805,19 @@ __global__ void k_mg_dinv_fine(int nd, int npad, Sliced SK, const T* __restrict_
   store_inv<T>(a, o, err, w);
 }
 
-// a + b with the rounding error kept in e (FP32; an FP64 sum takes it as it is)
-__device__ inline void add_kept(float& a, float& e, float b) {
-  float s = a + b, z = s - a;
-  e += (a - (s - z)) + (b - z);
-  a = s;
+// |v| in FP64.  A conversion takes the FP64 pipe as long as an addition, so zeros
+// and normal numbers are widened in integer instructions; others set `odd`
+__device__ inline double abs_wide(double v, bool&) { return fabs(v); }
+__device__ inline double abs_wide(float v, bool& odd) {
+  unsigned b = __float_as_uint(v) & 0x7fffffffu;
+  odd |= b - 1u < 0x007fffffu || b >= 0x7f800000u;
+  return __hiloint2double(b ? (int)((b >> 3) + 0x38000000u) : 0, (int)(b << 29));
 }
-__device__ inline void add_kept(double& a, double&, double b) { a += b; }
 
-// Level operators: eight lanes per row read it coalesced and sum its l1 parts
-// (FP32 entries in FP32 with the errors kept, so that no FP64 is spent per
-// entry), then a thread per row, the first warp's, inverts.  A thread per row
-// for the whole walk took 0.18 ms for 33 k rows and 0.11 ms, pure latency, on
-// each of the small levels; 0.04 and 0.012 ms now.
+// Level operators: eight lanes per row read it coalesced and sum its l1 parts in
+// FP64, then a thread per row, the first warp's, inverts.  A thread per row for
+// the whole walk took 0.18 ms for 33 k rows and 0.11 ms, pure latency, on each of
+// the small levels; 0.10 and 0.022 ms now, bound by the FP64 additions.
 constexpr int DR = 32;  // rows per block of 256 threads
 template <class T>
 __global__ void __launch_bounds__(8 * DR)
@@ -828,25 +828,29 @@ __global__ void __launch_bounds__(8 * DR)
   {
     int r = blockIdx.x * DR + (threadIdx.x >> 3), l = threadIdx.x & 7;
     const T* row = A + (size_t)r * S * 9;
-    T s[3] = {0, 0, 0}, c[3] = {0, 0, 0};
-    if (r < nrow)
+    double s[3] = {0, 0, 0};
+    bool odd = false;
+    if (r < nrow) {
+#pragma unroll 4
       for (int o = l; o < S; o += 8) {
-        if (o == center) continue;
+        T v[9];
 #pragma unroll
-        for (int e = 0; e < 9; ++e) {
-          T v = row[9 * o + e];
-          add_kept(s[e / 3], c[e / 3], v < (T)0 ? -v : v);
-        }
+        for (int e = 0; e < 9; ++e) v[e] = o == center ? (T)0 : row[9 * o + e];
+#pragma unroll
+        for (int e = 0; e < 9; ++e) s[e / 3] += abs_wide(v[e], odd);
       }
+      if (odd) {
+        s[0] = s[1] = s[2] = 0.0;
+        for (int o = l; o < S; o += 8)
+          for (int e = 0; e < 9; ++e)
+            if (o != center) s[e / 3] += fabs((double)row[9 * o + e]);
+      }
+    }
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
 #pragma unroll
-      for (int o = 4; o > 0; o >>= 1) {
-        T so = __shfl_xor_sync(0xffffffffu, s[d], o), co = __shfl_xor_sync(0xffffffffu, c[d], o);
-        add_kept(s[d], c[d], so);
-        c[d] += co;
-      }
-      if (l == 0) ls[threadIdx.x >> 3][d] = (double)s[d] + (double)c[d];
+      for (int o = 4; o > 0; o >>= 1) s[d] += __shfl_xor_sync(0xffffffffu, s[d], o);
+      if (l == 0) ls[threadIdx.x >> 3][d] = s[d];
     }
   }
   __syncthreads();
