@@ -407,7 +407,8 @@ int mpm_solve_static(mpm_ctx* ctx, const mpm_mesh* mesh, const double* K_values,
  * of MPM_PROF_NCLASS entries). */
 enum {
   MPM_PROF_PCG_UPDATE = 0,   /* PCG vector update + preconditioner + dots       */
-  MPM_PROF_PCG_SPMV = 1,     /* PCG SpMV fused with the direction update        */
+  MPM_PROF_PCG_SPMV = 1,     /* PCG SpMV fused with the direction update; a whole
+                                block-Jacobi PCG solve where it is one launch   */
   MPM_PROF_TANGENT = 2,      /* row-gather tangent assembly                     */
   MPM_PROF_CONSTITUTIVE = 3, /* per-point return map (+ spatial tangent)        */
   MPM_PROF_KINEMATICS = 4,   /* per-point dF                                     */
@@ -415,7 +416,8 @@ enum {
   MPM_PROF_BASIS = 6,        /* discrete GIMP basis                              */
   MPM_PROF_RESIDUAL = 7,     /* residual rows: internal force gather, ghost term */
   MPM_PROF_CONTACT = 8,      /* penalty contact                                  */
-  MPM_PROF_BICG_SPMV = 9,    /* BiCGStab SpMV                                    */
+  MPM_PROF_BICG_SPMV = 9,    /* BiCGStab and GMRES SpMV; a whole block-Jacobi
+                                BiCGStab solve where it is one launch           */
   MPM_PROF_REFINE = 10,      /* FP64 refinement residual                         */
   MPM_PROF_PATTERN = 11,     /* block pattern rows                               */
   MPM_PROF_MG = 12,          /* V-cycle kernels below level 1 and the transfers  */

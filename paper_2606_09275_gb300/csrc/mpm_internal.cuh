@@ -960,6 +960,14 @@ inline void prof_end(mpm_ctx* c) {
   MPM_CUDA(cudaEventRecord(c->prof.back().b, c->stream));
 }
 
+// takes back the last prof_begin: nothing was launched
+inline void prof_drop(mpm_ctx* c) {
+  if (!c->prof_on || c->prof.empty()) return;
+  c->evpool.push_back(c->prof.back().a);
+  c->evpool.push_back(c->prof.back().b);
+  c->prof.pop_back();
+}
+
 // ------------------------------------------------------------------ host entry helpers
 
 void set_error(mpm_ctx* c, const std::string& m);

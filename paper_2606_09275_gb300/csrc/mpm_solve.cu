@@ -530,14 +530,17 @@ int run_resident(mpm_ctx* c, bool* ran, void (*kern)(A...), const RkPlan& pl, un
   MPM_CUDA(cudaMemsetAsync(sc_d, 0, sizeof(Scal), st));
   MPM_CUDA(cudaMemsetAsync(slots, 0xff, sizeof(*slots) * rk_slot_words(pl.G), st));
   dynamic_smem(kern, RK_SMEM);
+  prof_begin(c, pcg ? MPM_PROF_PCG_SPMV : MPM_PROF_BICG_SPMV);
   cudaError_t e = cudaLaunchCooperativeKernel((const void*)kern, dim3(pl.G), dim3(RK_T), args, pl.smem, st);
   *ran = e != cudaErrorCooperativeLaunchTooLarge;
   if (!*ran) {
     cudaGetLastError();
+    prof_drop(c);
     return MPM_OK;
   }
   MPM_CUDA(e);
   MPM_COUNT(c);
+  prof_end(c);
   MPM_CUDA(cudaMemcpyAsync(sc_h, sc_d, sizeof(Scal), cudaMemcpyDeviceToHost, st));
   MPM_CUDA(cudaStreamSynchronize(st));
   if (sc_h->late) {

@@ -54,3 +54,19 @@ def test_a_wait_that_runs_out_is_an_error(system, method, precision):  # noqa: F
     y, st2 = run()
     assert st2 == st and torch.equal(x, y)
     assert mpm.lib().mpm_wait_limit(ctx.h, -1) == 1
+
+
+@pytest.mark.parametrize("method,precision,cls", [(1, 0, 1), (1, 1, 1), (2, 0, 9), (2, 1, 9)])
+def test_the_profile_has_the_solve(system, method, precision, cls):  # noqa: F811
+    import ctypes as C
+    s = system("punch")
+    mpm, torch, ctx = s["mpm"], s["torch"], s["ctx"]
+    cfg = dict(s["cfg"], mu=0.3, contact=1) if method == 2 else s["cfg"]
+    K = s["Kd"].float() if precision else s["Kd"]
+    n, ms = (C.c_longlong * 17)(), (C.c_double * 17)()
+    ctx.check(mpm.lib().mpm_profile(ctx.h, 1))
+    _, st = mpm.solve(ctx, s["mesh"], cfg, K, torch.from_numpy(s["b"]).cuda(), precision=precision, tol=1e-8,
+                      maxit=5000, method=method, inner_tol=1e-4)
+    ctx.check(mpm.lib().mpm_profile_read(ctx.h, n, ms))
+    ctx.check(mpm.lib().mpm_profile(ctx.h, 0))
+    assert n[cls] == max(st["refinements"], 1) and ms[cls] > 0.0  # one launch a solve
