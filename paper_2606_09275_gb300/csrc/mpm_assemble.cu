@@ -503,7 +503,7 @@ constexpr int TF_AS = 12;  // a block's 9 accumulators, padded for 16-byte acces
 
 // shared memory of one row: the accumulators, then the 32 terms of two sources
 // (the rows of a warp 16 bytes apart in the banks)
-inline size_t tangent_row_bytes_f32(int mr) { return ((size_t)mr * TF_AS + 64) * sizeof(float) + 16; }
+constexpr size_t tangent_row_bytes_f32(int mr) { return ((size_t)mr * TF_AS + 64) * sizeof(float) + 16; }
 
 // the 27 terms (grad_x S_k)^T A'_p of a source, 16-byte aligned, 32 entries
 __device__ inline void tangent_terms(const float* Tt, float* t) {
@@ -1570,12 +1570,12 @@ void tangent_passes(mpm_ctx* c, mpm_mesh* m, bool mixed, bool upper, int pw, con
     size_t rb = mixed ? tangent_row_bytes_f32(hi) : tangent_warp_bytes_f64(hi);
     bool share = (ps > 0 || m->ndof < TANGENT_FEW_ROWS) && 4 * rb <= TSMEM;
     if (mixed) {
+      // (four FP32 copies of the longest row fit: every long row is shared)
+      static_assert(4 * tangent_row_bytes_f32(MAXROW) <= TSMEM, "long rows of the FP32 tangent");
       if (share)
         tangent_launch<float>(c, m, k_tangent_rows_f32<32, 4>, rb, 1, 4, pw, lo, hi, last, gx, Aalg, K);
-      else if (ps == 0)
-        tangent_launch<float>(c, m, k_tangent_rows_f32<16, 1>, rb, 2, 1, pw, lo, hi, last, gx, Aalg, K);
       else
-        tangent_launch<float>(c, m, k_tangent_rows_f32<32, 1>, rb, 1, 1, pw, lo, hi, last, gx, Aalg, K);
+        tangent_launch<float>(c, m, k_tangent_rows_f32<16, 1>, rb, 2, 1, pw, lo, hi, last, gx, Aalg, K);
     } else {
       auto kern = upper ? (share ? k_tangent_rows_f64<true, 4> : k_tangent_rows_f64<true, 1>)
                         : (share ? k_tangent_rows_f64<false, 4> : k_tangent_rows_f64<false, 1>);
