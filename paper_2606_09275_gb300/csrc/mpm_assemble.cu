@@ -1643,7 +1643,7 @@ void assemble(mpm_ctx* c, const mpm_mesh* mc, const mpm_material& mat, const mpm
   void* gx = K ? grow_bytes(c, m->gx, 4 * (size_t)P * pw * asz) : nullptr;
   if (K && m->src_pos_gen != m->gen) {
     int hs = tangent_hash_size(m->maxrow);
-    unsigned short* sp = grow<unsigned short>(c, m->src_pos, (size_t)m->nsrc * pw);
+    unsigned short* sp = grow<unsigned short>(c, m->src_pos, (size_t)m->nsrc_used * pw);
     bool few = nd < TANGENT_FEW_ROWS;
     size_t smem = (few ? 1 : 4) * 2 * sizeof(int) * (size_t)hs;
     auto kern = few ? k_src_pos<true> : k_src_pos<false>;

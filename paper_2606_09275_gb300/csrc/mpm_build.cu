@@ -1926,8 +1926,11 @@ void build_mesh(mpm_ctx* c, mpm_mesh* m, const mpm_domain& dom, const mpm_rigid&
   // FP32 copies of the basis for the mixed-precision path are made on demand
   // by the assembly
   MeshCounts* h = (MeshCounts*)c->h_red;
+  long long* used = (long long*)(c->h_red + 8);
   MPM_CUDA(cudaMemcpyAsync(h, mc, sizeof(MeshCounts), cudaMemcpyDeviceToHost, st));
+  MPM_CUDA(cudaMemcpyAsync(used, ptr<long long>(m->src_ptr) + m->ndof, sizeof(long long), cudaMemcpyDeviceToHost, st));
   MPM_CUDA(cudaStreamSynchronize(st));
+  m->nsrc_used = *used;
   m->npair = (long long)h->npair;
   m->maxs = h->maxs;
   m->maxrow = h->maxrow;

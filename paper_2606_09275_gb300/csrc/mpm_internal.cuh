@@ -223,7 +223,8 @@ struct mpm_mesh {
   mpm::Buf srow, spos;                  // storage row -> dof row, and back (npad each)
   std::vector<int> slice_w_host;        // slice_w of a small mesh (resident solves; else empty)
   // sources of each row: (sorted point or ghost face) << 6 | local index
-  long long nsrc = 0;
+  long long nsrc = 0;       // with the unused slots of the ghost faces, which sort last
+  long long nsrc_used = 0;  // src_ptr[ndof]
   long long npair = 0;  // sum of squared support sizes (host copy, read after the build)
   mpm::Buf src_key, src_ptr;
   // gravity force at load 1
