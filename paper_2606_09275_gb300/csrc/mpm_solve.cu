@@ -241,12 +241,9 @@ __global__ void k_pcg_b(int nd, int npad, int k, Sliced S, const T* __restrict__
 
 // y = K x (+ optional dots a.y into slot and y.y into slot2).  Skipped once
 // the solve is done, or (check_s) once the half-step residual s has converged.
-// Bounded to 3 resident blocks of 256 per SM: with streaming loads of the
-// matrix and the grid sum through shared memory, 4 blocks (64 registers, a
-// spill) take 0.329 ms and 3 (80 registers) 0.307 (FP32, 41.7 M blocks of the
-// cone); in FP64 0.781 (1.112 with 4 blocks, plain sums of products)
-template <class T, class V, bool STREAM>
-__global__ void __launch_bounds__(256, 3) k_spmv_dot(int nd, int npad, Sliced S, const T* __restrict__ K,
+// NB: its launch bound in blocks of 256 per SM (spmv_blocks)
+template <class T, class V, int NB, bool STREAM>
+__global__ void __launch_bounds__(256, NB) k_spmv_dot(int nd, int npad, Sliced S, const T* __restrict__ K,
                            const V* __restrict__ x, V* y, const V* __restrict__ a,
                            double* slot, double* slot2, const Scal* sc, int check_s, GridRed gr) {
   if (sc->done || (check_s && sc->a[5] <= sc->thr)) return;
@@ -267,6 +264,19 @@ __global__ void __launch_bounds__(256, 3) k_spmv_dot(int nd, int npad, Sliced S,
     p2 = (double)v[0] * v[0] + (double)v[1] * v[1] + (double)v[2] * v[2];
   }
   grid_sum2(p1, p2, slot, slot2, gr);
+}
+
+// Launch bound of k_spmv_dot.  With 2 the compiler keeps the most loads in flight
+// (80 registers in FP32, 3 blocks to an SM; 128 in FP64, 2).  4 (64 registers)
+// where that runs all rows of an FP32 matrix at once and 3 blocks to an SM leave a
+// last wave that is nearly empty.  us a launch with 2, 3 and 4, FP32: 22.7 k rows
+// 46, 57, 81; 95 k 81, 86, 95; 123 k 117, 124, 110; 141 k 134, 139, 126; 178 k 141,
+// 146, 181; 248 k 200, 207, 207.  FP64, bound by its rate: 22.7 k 120, 141, 168;
+// 141 k 320, 333, 351
+template <class T>
+int spmv_blocks(int npad) {
+  int n = (npad + 255) / 256;
+  return sizeof(T) == 4 && n > 3 * 152 && n <= 4 * 152 ? 4 : 2;
 }
 
 // start: r = r0 = b (free components), x = 0, ||b||^2
@@ -723,17 +733,20 @@ int run_bicgstab(mpm_ctx* c, const mpm_mesh* m, const T* K, const T* Dinv, const
   init.a[3] = bb;  // r0 . r at the start
   MPM_CUDA(cudaMemcpyAsync(sc_d, &init, sizeof(Scal), cudaMemcpyHostToDevice, st));
   const int batch = Dinv ? 16 : 4;
+  constexpr int NB4 = sizeof(T) == 4 ? 4 : 2;
+  auto spmv = spmv_blocks<T>(npad) == 2 ? MPM_STREAM(S, T, k_spmv_dot<T, V, 2)
+                                        : MPM_STREAM(S, T, k_spmv_dot<T, V, NB4);
   while (it < maxit) {
     int iend = std::min(maxit, it + batch);
     for (; it < iend; ++it) {
       MPM_CUDA(cudaMemsetAsync(red, 0, 2 * sizeof(double), st));
       MPM_LAUNCH(k_bicg_p<V><<<vb, 256, 0, st>>>(npad, p, r, v, ph, Dinv, sc_d));
       if (!Dinv) mg_precondition<T>(c, m, K, p, ph, sc_d);
-      MPM_LAUNCH_P(MPM_PROF_BICG_SPMV, MPM_STREAM(S, T, k_spmv_dot<T, V)<<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, K, ph, v, r0, &sc_d->a[4], nullptr, sc_d, 0, gr));
+      MPM_LAUNCH_P(MPM_PROF_BICG_SPMV, spmv<<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, K, ph, v, r0, &sc_d->a[4], nullptr, sc_d, 0, gr));
       MPM_LAUNCH(k_bicg_s<V><<<vb, 256, 0, st>>>(npad, r, v, s, shv, Dinv, sc_d, gr));
       MPM_LAUNCH(k_bicg_check_s<V, X><<<vb, 256, 0, st>>>(nd, x, ph, sc_d));
       if (!Dinv) mg_precondition<T>(c, m, K, s, shv, sc_d);
-      MPM_LAUNCH_P(MPM_PROF_BICG_SPMV, MPM_STREAM(S, T, k_spmv_dot<T, V)<<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, K, shv, t, s, &sc_d->a[6], &sc_d->a[7], sc_d, 1, gr));
+      MPM_LAUNCH_P(MPM_PROF_BICG_SPMV, spmv<<<grid_for(npad, 32 * SW), 32 * SW, 0, st>>>(nd, npad, S, K, shv, t, s, &sc_d->a[6], &sc_d->a[7], sc_d, 1, gr));
       MPM_LAUNCH(k_bicg_x<V, X><<<vb, 256, 0, st>>>(nd, npad, x, r, ph, shv, s, t, r0, sc_d, red, red + 1, gr));
       MPM_LAUNCH(k_bicg_rotate<<<1, 1, 0, st>>>(sc_d, red, red + 1, it + 1));
     }

@@ -70,3 +70,38 @@ def test_the_profile_has_the_solve(system, method, precision, cls):  # noqa: F81
     ctx.check(mpm.lib().mpm_profile_read(ctx.h, n, ms))
     ctx.check(mpm.lib().mpm_profile(ctx.h, 0))
     assert n[cls] == max(st["refinements"], 1) and ms[cls] > 0.0  # one launch a solve
+
+
+@pytest.mark.parametrize("precision,shear", [(0, 0.02), (0, 1e-4), (1, 1e-4)])
+def test_bicgstab_of_a_nonsymmetric_tangent(precision, shear):
+    # non-associated Drucker-Prager under a shear that yields: the residual of the
+    # solution in FP64 on the host, to the bound of test_gpu_resident_solve
+    import scipy.sparse as sp
+    import torch
+    from paper_2606_09275_gb300 import inputs, mpm
+    from test_gpu_resident_solve import config
+    cfg = config("cone", (4, 6), (12, 11, 9))
+    ctx = mpm.Context()
+    pts = inputs.make_points(cfg)
+    P = mpm.Points(pts, capacity=12 * len(pts["x"]) + 400000)
+    bz = inputs.body_z(cfg, 1)
+    mesh = mpm.octree_build(ctx, cfg, P, body_z=bz)
+    nd = mesh.info()["ndof"]
+    dof, coord, mask = mesh.export("node_dof"), mesh.export("node_coord"), mesh.export("bcmask")
+    x = np.zeros((nd, 3))
+    x[dof[dof >= 0]] = coord[dof >= 0] * (cfg["L"] / (1 << cfg["depth_max"]))
+    free = np.array([[not (m >> c) & 1 for c in range(3)] for m in mask])
+    u = shear * np.stack([x[:, 2], 0.3 * x[:, 2], -0.2 * x[:, 2]], axis=1) * free
+    du = torch.from_numpy(u.ravel().copy()).cuda()
+    Kd = mpm.assemble(ctx, mesh, cfg, du, precision=precision, body_z=bz)["K"]
+    K = sp.bsr_matrix((mpm.blocks(ctx, mesh, Kd, precision), mesh.export("col"), mesh.export("row_ptr")),
+                      shape=(3 * nd, 3 * nd)).tocsr()
+    assert abs(K - K.T).max() > 1e-3 * abs(K).max()
+    b = np.random.default_rng(7).normal(size=3 * nd)
+    bf = b * free.ravel()
+    tol = 1e-8
+    y, st = mpm.solve(ctx, mesh, cfg, Kd, torch.from_numpy(b).cuda(), precision=precision, tol=tol, maxit=5000,
+                      method=0 if precision else 2, inner_tol=1e-4)
+    assert st["status"] == 0 and st["relres"] <= tol
+    r = (bf - K @ y.cpu().numpy()) * free.ravel()
+    assert np.linalg.norm(r) <= 1.2 * tol * np.linalg.norm(bf)
