@@ -279,7 +279,7 @@ struct Sliced {
   const int* pos;        // storage row of each dof row
   int stream;            // FP32 and FP16 products take streaming loads (sliced_view)
 };
-constexpr int RESIDENT_SLICES = 4096;  // most slices of a mesh whose solves may run resident (mpm_solve.cu)
+constexpr int RESIDENT_SLICES = 3072;  // most slices of a mesh whose solves may run resident (mpm_solve.cu)
 constexpr int SLICE_WINDOW = 256;  // storage rows over which the dof rows are sorted
 __host__ __device__ inline long long sliced_slot(long long base, int sr, int idx) {
   return base + ((long long)(idx >> 2) * 32 + (sr & 31)) * 4 + (idx & 3);

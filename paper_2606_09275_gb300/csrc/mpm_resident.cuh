@@ -12,14 +12,19 @@
 // run.  Bound by: the sums (2.4 us, 3.1 us where a vector is published too) on
 // small meshes, the FP64 rate (9 FMAs a block) or the L2 above.
 //
-// us per iteration, launches per iteration -> resident:
-//   rows (blocks)      PCG FP64       PCG FP32       BiCGStab FP64
-//      645 (43 k)      128 -> 12       57 -> 13        285 -> 25
-//    2,026 (178 k)     147 -> 15       57 -> 13        310 -> 31
-//   10,446 (1.04 M)    153 -> 35       56 -> 18        343 -> 72
-//   36,727 (3.98 M)    191 -> 103     107 -> 55        396 -> 208
-//   81,042 (8.90 M)    339 -> 197     123 -> 88        693 (state too large)
-//  133,026 (14.9 M)    495 (too large) 150 -> 139      970 (too large)
+// us per iteration, launches per iteration -> resident (up to 10 k rows the
+// launches as they were before this file, then as they are):
+//   rows (blocks)      PCG FP64       PCG FP32       BiCGStab FP64    FP32
+//      858 (67 k)      128 -> 13       50 -> 9         275 -> 27      104 -> 20
+//    2,026 (178 k)     144 -> 15       51 -> 10        308 -> 32      101 -> 21
+//   10,446 (1.04 M)    146 -> 36       52 -> 16        320 -> 74      102 -> 35
+//   36,935 (3.99 M)    173 -> 103      97 -> 55        271 -> 206     125 -> 114
+//   58,052 (6.29 M)    202 -> 150     103 -> 69        376 -> 299     155 -> 144
+//   78,044 (8.57 M)    212 -> 194     110 -> 84        408 -> 410     188 -> 178
+//   96,364 (10.7 M)    267 -> 230     117 -> 100       530 (state     209 -> 207
+//  110,690 (12.3 M)    278 (281)      123 (129)        550  too       230 (264)
+//  121,837 (13.6 M)    345 (342)      131 (137)        646  large)    277 (423)
+// (in brackets: resident, beyond the limit RESIDENT_SLICES)
 #pragma once
 #include "mpm_sliced.cuh"
 

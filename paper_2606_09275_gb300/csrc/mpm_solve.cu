@@ -491,8 +491,10 @@ Sliced sliced_of(const mpm_mesh* m) { return sliced_view(m); }
 
 // The plan of a resident solve (mpm_resident.cuh) of this mesh with nv vectors
 // per row, G = 0 for the launches per iteration.  Resident is the faster way
-// wherever the rows' state fits in shared memory, by 10x at 2 k rows down to
-// 1.08x at 131 k (FP32 PCG, the table there), where HBM bounds both: the limit
+// where the rows' state fits in shared memory, by 10x at 2 k rows down to nothing
+// at some 100 k (the table there), where HBM bounds both and a block takes its
+// rows in several passes; beyond, up to 1.5x slower (FP32 BiCGStab, 117 k to 122 k
+// rows: 404 to 424 us an iteration, 271 to 275 by launches).  The limit:
 // RESIDENT_SLICES.
 template <class T>
 RkPlan resident_plan(const mpm_ctx* c, const mpm_mesh* m, int nv) {

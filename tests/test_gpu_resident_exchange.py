@@ -105,3 +105,40 @@ def test_bicgstab_of_a_nonsymmetric_tangent(precision, shear):
     assert st["status"] == 0 and st["relres"] <= tol
     r = (bf - K @ y.cpu().numpy()) * free.ravel()
     assert np.linalg.norm(r) <= 1.2 * tol * np.linalg.norm(bf)
+
+
+@pytest.mark.parametrize("method", [1, 2])
+def test_blocks_that_take_their_rows_in_several_passes(method):
+    # more than 512 rows to a block (FP32), just below the largest mesh of these
+    # solves; the bound of test_gpu_resident_solve
+    import scipy.sparse as sp
+    import torch
+    from paper_2606_09275_gb300 import inputs, mpm
+    from test_gpu_resident_solve import config
+    cfg = config("indent", (6, 7), (54, 52, 28))
+    ctx = mpm.Context()
+    P = mpm.Points(inputs.make_points(cfg), capacity=2500000)
+    bz = inputs.body_z(cfg, 1)
+    mesh = mpm.octree_build(ctx, cfg, P, body_z=bz)
+    nd = mesh.info()["ndof"]
+    assert 512 * 151 < nd <= 98304
+    Kd = mpm.assemble(ctx, mesh, cfg, torch.zeros(3 * nd, dtype=torch.float64, device="cuda"), precision=mpm.MIXED,
+                      body_z=bz)["K"]
+    K = sp.bsr_matrix((mpm.blocks(ctx, mesh, Kd, mpm.MIXED), mesh.export("col"), mesh.export("row_ptr")),
+                      shape=(3 * nd, 3 * nd))
+    free = np.array([[not (m >> c) & 1 for c in range(3)] for m in mesh.export("bcmask")]).ravel()
+    b = np.random.default_rng(7).normal(size=3 * nd)
+    cfg = dict(cfg, mu=0.3, contact=1) if method == 2 else cfg
+    n0 = _launches(mpm, ctx)
+    x, st = mpm.solve(ctx, mesh, cfg, Kd, torch.from_numpy(b).cuda(), precision=mpm.MIXED, tol=1e-8, maxit=5000,
+                      method=method, inner_tol=1e-4)
+    assert st["status"] == 0 and _launches(mpm, ctx) - n0 < st["iterations"]  # (in one launch)
+    r = (b * free - K @ x.cpu().numpy()) * free
+    assert np.linalg.norm(r) <= 1.2e-8 * np.linalg.norm(b * free)
+
+
+def _launches(mpm, ctx):
+    import ctypes as C
+    n = C.c_longlong()
+    ctx.check(mpm.lib().mpm_launch_count(ctx.h, C.byref(n)))
+    return n.value
