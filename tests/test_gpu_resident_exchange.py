@@ -137,6 +137,20 @@ def test_blocks_that_take_their_rows_in_several_passes(method):
     assert np.linalg.norm(r) <= 1.2e-8 * np.linalg.norm(b * free)
 
 
+@pytest.mark.parametrize("method", [1, 2])
+def test_a_right_hand_side_near_the_smallest(system, method):  # noqa: F811
+    # r.z and r.r fall below the smallest normal number on the way, where a
+    # reciprocal overflows; the residual keeps 1.2 tol at tol = 1e-6
+    s = system("punch")
+    mpm, torch = s["mpm"], s["torch"]
+    cfg = dict(s["cfg"], mu=0.3, contact=1) if method == 2 else s["cfg"]
+    b = np.ldexp(s["b"] / np.linalg.norm(s["b"]), -490)
+    x, st = mpm.solve(s["ctx"], s["mesh"], cfg, s["Kd"], torch.from_numpy(b).cuda(), tol=1e-6, maxit=2000, method=method)
+    assert st["status"] == 0
+    r = np.ldexp(b * s["free"] - s["K"] @ x.cpu().numpy(), 490) * s["free"]
+    assert np.linalg.norm(r) <= 1.2e-6 * np.linalg.norm(np.ldexp(b, 490) * s["free"])
+
+
 def _launches(mpm, ctx):
     import ctypes as C
     n = C.c_longlong()
