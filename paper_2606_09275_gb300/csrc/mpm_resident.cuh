@@ -65,9 +65,6 @@ __device__ inline unsigned long long rk_ld_acquire(const unsigned long long* p) 
 __device__ inline void rk_st(unsigned long long* p, unsigned long long v) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
-__device__ inline void rk_st_release(unsigned long long* p, unsigned long long v) {
-  asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
 __device__ inline void rk_fence() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
 // loads of a vector that other SMs write during the launch (past the L1)
@@ -120,9 +117,9 @@ struct RkShared {
 // A fenced sum hands the vectors that the blocks stored before it to all of
 // them: every worker fences and posts slot 0 (release); the coordinator's lanes
 // that saw the slots fence (acquire) and meet at its barrier; each lane that
-// answers stores the second word of its message with release, which covers
-// what the other lanes saw; the workers load that word with acquire and meet
-// at their barrier.
+// answers fences again and stores its message (release), which covers what the
+// other lanes saw; the workers load its second word with acquire and meet at
+// their barrier.
 struct RkGrid {
   unsigned long long* slot;
   int* late;
@@ -255,12 +252,9 @@ __device__ inline void rk_tell(RkGrid& g, double a, double b, int stop, bool fen
   const int t = threadIdx.x;
   if (t < RK_COPY) {
     unsigned long long* m = g.msg(g.k, t);
+    if (fence) rk_fence();  // (no store of this warp is under way: some 0.1 us)
     rk_st(m, rk_pack(a));
-    unsigned long long w = stop ? RK_STOP | (unsigned long long)stop : rk_pack(b);
-    if (fence)
-      rk_st_release(m + 1, w);
-    else
-      rk_st(m + 1, w);
+    rk_st(m + 1, stop ? RK_STOP | (unsigned long long)stop : rk_pack(b));
     if (g.k > 0) {
       unsigned long long* o = g.msg(g.k + RK_NBUF - 1, t);
       rk_st(o, RK_EMPTY);
