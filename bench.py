@@ -266,8 +266,9 @@ def kernel_models(s, mixed=True):
                                   what="V-cycle level-1 residual / smoothing, operator stored per "
                                        "stencil offset (FP32)", bytes=r1 * (S1 * 36 + 72), bound="hbm")
     # tangent rows, per Newton iteration (its two launches together): the
-    # 81-entry tangents (with V0), grad_x S and row positions, the source keys,
-    # ghost coefficients and columns in; the sliced K out
+    # 81-entry tangents (V0 in them), grad_x S, the 16-bit row position of each
+    # (source, column) pair, the source keys, ghost coefficients and columns in;
+    # the sliced K out, every array once and without its padding;
     # and its arithmetic: 27 FMA per (source, column) pair, npair = sum of the
     # squared support sizes, plus the 27 terms of each source (81 FMA + 27
     # multiplications); its accumulators take 9 shared-memory read-modify-writes
@@ -275,7 +276,7 @@ def kernel_models(s, mixed=True):
     npair = s.get("npair") or 0
     m["tangent_rows"] = dict(kernel="k_tangent_rows_f32 (both passes)",
                              what="row-gather tangent assembly, per Newton iteration",
-                             bytes=P * (81 * w + 8) + nsrc * (3 * w + 4 + 8) + nnzb * 12 + nslot * 9 * w,
+                             bytes=P * 81 * w + nsrc * (3 * w + 8) + 2 * npair + nnzb * 12 + nslot * 9 * w,
                              fp32_flops=54.0 * npair + 189.0 * nsrc, smem_bytes=2.0 * 9 * w * npair,
                              bound="latency", per="newton_it")
     # internal-force gather + residual rows: FP64, 9 FMA per (point, support)

@@ -441,8 +441,9 @@ __device__ inline unsigned tangent_hash(int c, int hmask) {
 }
 
 // row position of every (source, support node) pair, pw per source (0xffff
-// beyond the source's support, and for ghost faces): made once per mesh build,
-// so that the gather of every Newton iteration needs no lookup.  A hash table
+// beyond the source's support, and for ghost faces): made at a mesh's first
+// tangent, 2.45 ms on the indentation block, so that the gather (6.3 ms, every
+// Newton iteration) needs no lookup.  A hash table
 // of the row's columns in shared memory; a warp per row, or (SHARED, meshes of
 // few rows) a block per row, its warps taking the sources 32 at a time in turn.
 template <bool SHARED>
@@ -576,13 +577,14 @@ __device__ inline void tangent_fetch_f(TangentSrcF<HL>& s, uint32_t sid, long lo
 // mean support), one per half, so that a warp instruction serves two sources.
 // Bound by shared-memory wavefronts: the accumulators' round trip at random
 // 48-byte slots, 37 of them per source, and 15 of the loads (ncu, LSU data
-// pipe 72 % busy).  Indentation, 1.9 M points, 29.7 M sources: 7.6 ms with a
+// pipe 72 % busy).  Indentation, 1.9 M points, 28.8 M sources: 7.6 ms with a
 // hash lookup per pair and 13 loads per source, 6.4 with the precomputed
 // positions and 16-byte loads, 6.0 with two rows per warp (the long rows' pass
-// 1.2 -> 0.36 of it); an entry of the block per lane, as in FP64, 7.0.  HL = 32, WPR > 1: the warps of a block share a
-// row, each taking a contiguous part of its sources with a copy of the
-// accumulators, added up in warp order: for rows whose serial chain of sources
-// would be the time (few rows, and the long rows near hanging nodes).
+// 1.2 -> 0.36 of it); an entry of the block per lane, as in FP64, 7.0.
+// HL = 32, WPR > 1: the warps of a block share a row, each taking a contiguous
+// part of its sources with a copy of the accumulators, added up in warp order:
+// for rows whose serial chain of sources would be the time (few rows, and the
+// long rows near hanging nodes).
 template <int HL, int WPR>
 __global__ void __launch_bounds__(32 * TW)
     k_tangent_rows_f32(int nd, int P, int pw, int minlen, int mr, int last, const int* __restrict__ rp,
@@ -1142,7 +1144,8 @@ __device__ inline int block_compact(F on, G value, int* list, int* wsum) {
 // out[6..41] their derivative in the body's increment q (row-major 6 x 6):
 // [d f / d qt, d f / d qr; [f]x + [d]x d f / d qt, [d]x d f / d qr] with
 // d f / d qt = -d f / d y.  (A tree of shuffles per value and warp, 5 FP64
-// additions at 16 SM cycles each, made this 51 us on the rolling sphere's 2.4 k candidates; 47 so, most of it the scan.)
+// additions at 16 SM cycles each, made this 51 us on the rolling sphere's 2.4 k
+// candidates; 47 so, most of it the scan.)
 constexpr int BSUM_T = 256, BSUM_N = 8;
 __global__ void __launch_bounds__(BSUM_T)
     k_body_sums(int nc8, const double* __restrict__ cf, const double* __restrict__ ck, const double* __restrict__ ct,

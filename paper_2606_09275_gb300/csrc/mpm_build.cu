@@ -955,7 +955,7 @@ __global__ void __launch_bounds__(128)
 // one source write distinct columns and the sources follow one another, so
 // every entry is summed in a fixed order (no atomics).  The faces are the last
 // of a row's sources; the warp looks for the first of them from the end, 32 keys
-// at a time (passing over some 200 points one by one took 0.62 ms for 260 k
+// at a time (passing over some 200 points one by one took 0.62 ms for 248 k
 // rows, most of them without a face; 0.21 now).
 __global__ void k_ghost_rows(int nd, int P, const long long* __restrict__ sptr,
                              const uint64_t* __restrict__ skeys, const int* __restrict__ gdof,
@@ -1004,7 +1004,7 @@ struct MeshCounts {
 // source keys: row dof << 32 | source << 6 | local index (points, then ghost
 // faces).  With these bits the keys of the points, and of the faces after them,
 // are listed in ascending order of their lower 32 bits: a stable sort by the
-// row alone (3 passes of 8 bits at 260 k rows instead of 8) orders them fully.
+// row alone (3 passes of 8 bits at 248 k rows instead of 8) orders them fully.
 __global__ void k_point_sources(int P, const int* __restrict__ nsup, const int* __restrict__ node_dof,
                                 const int* __restrict__ off, int* sidx, uint64_t* keys,
                                 MeshCounts* mc) {
@@ -1062,7 +1062,7 @@ __global__ void k_src_ptr(long long n, const uint64_t* __restrict__ keys, int nd
 // their sorted columns in a staging row, which a copy takes to its place once
 // the row lengths are known; the others are collected again then, by the kernel
 // with the large set.  Two traversals, source by source, of a 2048-slot set took
-// 2 x 5.63 ms for 260 k rows and 51 M sources; now 2.10 ms, bound by
+// 2 x 5.63 ms for 248 k rows and 29 M sources; now 2.10 ms, bound by
 // instruction issue (87 % of the slots), and the copy 0.08 ms.
 constexpr int PSHORT = 256;            // longest row of the small set, and a staging row
 constexpr int PHASH = 2 * PSHORT;      // its slots
