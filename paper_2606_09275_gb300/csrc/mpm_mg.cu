@@ -584,14 +584,14 @@ __device__ inline void gather_axis(const long long* v, bool odd, long long* o) {
 
 // The same product gathered, for stencils of radius 2 on both levels: one block
 // per coarse row a, in fixed point.  An entry of the finer operator is rounded
-// once, in units of 2^3 of the scattered product's, and the weights are whole
-// numbers in units of 2^-6, 2^-3 a side: the product is exactly as symmetric as
-// the finer operator and as accurate as the scattered one, which rounds every
-// term in its unit (rms error against exact sums 55 and 59 ulps of the largest
-// entry for 27 x 125 random entries; halves rounded axis by axis, 578).  No
-// overflow: the sum of an entry's |terms| is at most 8/27 of B, so below
-// 8/27 2^61 in the scattered unit and below 2^63 in the unit 2^-3 of it that the
-// sums are taken in.  Over the rows
+// once, and the weights are whole numbers in units of 2^-6, 2^-3 a side: the
+// product is exactly as symmetric as the finer operator and more accurate than
+// the scattered one, which rounds every term (rms error against exact sums 52
+// and 63 ulps of the largest entry for 27 x 125 random entries; halves rounded
+// axis by axis, 563).  No overflow: with B the largest l1 norm of a finer row, an
+// entry's |terms| add up to at most 8 B (the weights of a column of P to 8), below
+// 2^63 in the unit of the sums; 8.000001 leaves room for the entries' rounding.
+// Over the rows
 // i of the finer nodes 2 a + {-1, 0, 1}^3, the 5 x 5 x 5 blocks of a row are
 // interpolated an axis at a time, a thread per line, to the 4 x 4 x 4 coarse
 // nodes around i, and added to the row of a in shared memory; the next row's
@@ -616,8 +616,8 @@ __global__ void __launch_bounds__(RG)
   __shared__ int node[343];            // rows of the finer nodes 2 a + {-3..3}^3, -1: none
   __shared__ unsigned char mask[343];  // their Dirichlet components
   int t = threadIdx.x, a = blockIdx.x;
-  double B = __longlong_as_double((long long)*bnd) * 27.0;
-  int ex = !(B > 0.0) || !isfinite(B) ? 0 : 57 - ilogb(B);  // 3 below fixed_scale's
+  double B = __longlong_as_double((long long)*bnd) * 8.000001;
+  int ex = !(B > 0.0) || !isfinite(B) ? 0 : 56 - ilogb(B);
   int ca[3];
   unpack3(xyz_c[a], ca);
   for (int f = t; f < 343; f += RG) {

@@ -6,9 +6,9 @@ a coarse cell), hanging nodes, and a thin block.
 Level 1, P^T K P in the matrix precision: each entry is a sum of at most n =
 125 x 27 products taken in some order, so |error| <= n eps (|P|^T |K| |P|)
 entry by entry.  The uniform levels below: the product is defined in whole
-numbers (an entry of the finer operator rounded once, at 2^(57 - floor(log2(27
-B))) with B the largest l1 norm of one of its rows; whole weights of 2^-3 a side),
-so it is recomputed in int64 and has to be the same bit for bit.  The inverse of
+numbers (an entry of the finer operator rounded once, at 2^(56 - floor(log2(
+8.000001 B))) with B the largest l1 norm of one of its rows; whole weights of 2^-3
+a side), so it is recomputed in int64 and has to be the same bit for bit.  The inverse of
 the last level, by elimination without pivoting on a symmetric positive definite
 matrix: |error| <= 10 n cond eps of its largest entry, plus its rounding.
 """
@@ -112,7 +112,7 @@ def test_level_operators(key, depth, block, precision):
         d, c = levels[f], levels[f + 1]
         assert d[2] == c[2] == 2  # the gathered form
         fine = np.array(abs(A[f]).sum(axis=1)).reshape(-1, 3).sum(axis=1).max()
-        ex = 57 - int(np.floor(np.log2(27.0 * fine)))
+        ex = 56 - int(np.floor(np.log2(8.000001 * fine)))
         free = sp.diags((~fixed_rows(nn[f][:, 3])).astype(float))
         ints = (free @ A[f] @ free).tocsr()
         ints.data = np.rint(np.ldexp(ints.data, ex))
