@@ -1099,9 +1099,9 @@ __global__ void k_mg_restrictu(int nrow, int npad, const int* __restrict__ xyz, 
       bool in = fx >= 0 && fy >= 0 && fz >= 0 && fx < n1f && fy < n1f && fz < n1f;
       jq[q] = in ? gid_f[fx + n1f * (fy + n1f * fz)] : -1;
     }
-    // z, then y, then x offsets, in that order
+    // from the last node to the first
 #pragma unroll
-    for (int q = 0; q < 27; ++q) {
+    for (int q = 26; q >= 0; --q) {
       if (jq[q] < 0) continue;
       int dx = q % 3 - 1, dy = (q / 3) % 3 - 1, dz = q / 9 - 1;
       T f = (T)((dx ? 0.5 : 1.0) * (dy ? 0.5 : 1.0) * (dz ? 0.5 : 1.0));

@@ -393,8 +393,14 @@ struct RkRows {
           T xv[4];
           ld4_cg(x + 4 * (size_t)cc[j], xv);
 #pragma unroll
-          for (int d = 0; d < 3; ++d)
-            a[d] = fma(v[3 * d + 2][j], xv[2], fma(v[3 * d + 1][j], xv[1], fma(v[3 * d][j], xv[0], a[d])));
+          for (int d = 0; d < 3; ++d) {
+            // (FP64 nested: its rate is the bound; FP32 with one rounding of the
+            // long sum a block, as sliced_row)
+            if constexpr (sizeof(T) == 8)
+              a[d] = fma(v[3 * d + 2][j], xv[2], fma(v[3 * d + 1][j], xv[1], fma(v[3 * d][j], xv[0], a[d])));
+            else
+              a[d] += fma(v[3 * d + 2][j], xv[2], fma(v[3 * d + 1][j], xv[1], v[3 * d][j] * xv[0]));
+          }
         }
       }
 #pragma unroll
